@@ -192,7 +192,8 @@ typedef struct {
     uint64_t n_adversarial;    /* adversarial points (ties excluded)      */
     uint64_t first_witness;    /* smallest adversarial index, or NO_WITNESS */
     uint64_t n_ties;           /* points with |m| < 1e-9                  */
-    uint64_t n_recheck[4];     /* points re-run: tensor split, FP32,      *
+    uint64_t n_recheck[4];     /* points re-run: tensor split (folded     *
+                                * net: its FP64 form), FP32,              *
                                 * double-float, FP64                      */
     double ms_device;          /* device time of the last verify call     */
     double ms_prologue;        /* of which: FP64 base pass and tables     */
@@ -382,6 +383,13 @@ vbmc_status vbmc_autotune(vbmc_net *net, const char *cache_path, vbmc_tuning *ou
 
 /* Apply given launch shapes (0 in a field: the built-in choice). */
 vbmc_status vbmc_set_tuning(vbmc_net *net, const vbmc_tuning *t);
+
+/* A diagnostic: with on = 0 this net's calls check every query through the
+ * general passes of their precision; with on != 0 (the state of a new net) a
+ * query of a ReLU net whose neurons mostly keep their sign in the box is
+ * checked through its folded net. Results are the same either way; only the
+ * times and n_recheck differ. */
+vbmc_status vbmc_set_folding(vbmc_net *net, int32_t on);
 
 /* Accumulation error per product that the FP8 screen's bound assumes for this
  * net's device, relative to the sum of |products|: 2^-22 when the set-up

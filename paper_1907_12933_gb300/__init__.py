@@ -175,6 +175,7 @@ def lib():
             "vbmc_enum_coverage": [vp, C.POINTER(_Query), C.POINTER(_CoverParams), C.POINTER(_PairMasks), vp,
                                    C.POINTER(C.c_uint64), vp],
             "vbmc_set_tuning": [vp, C.POINTER(_Tuning)],
+            "vbmc_set_folding": [vp, C.c_int32],
             "vbmc_proposal_create": [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32,
                                      C.c_uint64, C.POINTER(vp)],
             "vbmc_proposal_free": [vp],
@@ -467,6 +468,11 @@ def set_tuning(net: Net, **fields) -> None:
     """vbmc_set_tuning: apply launch shapes (missing fields: the built-in choice)."""
     t = _Tuning(**{k: int(v) for k, v in fields.items() if k in dict(_Tuning._fields_)})
     _check(lib().vbmc_set_tuning(net.h, C.byref(t)))
+
+
+def set_folding(net: Net, on: bool) -> None:
+    """vbmc_set_folding: with on=False every query of this net takes the general passes."""
+    _check(lib().vbmc_set_folding(net.h, int(bool(on))))
 
 
 def search_query(net: Net, res: Result, image, pixels, k: int, order, precision="bf16",

@@ -70,6 +70,7 @@ struct vbmc_net {
     int n_sm = 0;
     int device = 0;
     TcNet tc{};  // tensor-core copies (built on first use per precision)
+    bool fold = true;  // calls may check a query through its folded net (vbmc_set_folding)
     WideNet wide{};  // rounded copies for the wide-layer path (built on first use per type)
     std::vector<std::vector<float>> hW, hb;  // host copies for tensor-core set-up
 };
@@ -89,7 +90,8 @@ struct BatchArena {
     uint8_t* d_stage = nullptr;
     size_t stage_stride = 0;
     unsigned long long* d_qcount = nullptr;
-    unsigned long long* d_claim = nullptr;  // tile claims of each wave's first pass
+    unsigned long long* d_claim = nullptr;  // tile claims of each wave's first pass: the general
+                                            // one, the folded nets'; queries not folded
     QEntry* d_queue[4] = {nullptr, nullptr, nullptr, nullptr};
     uint64_t queue_cap = 0;
     cudaEvent_t ev[7] = {};  // start, prologue, screen, end, split, FP32, double-float
@@ -124,7 +126,7 @@ struct vbmc_result {
     unsigned long long* d_tiles = nullptr;  // VBMC_MAX_TILES counters of vbmc_tile_counts
     TcQueryWork tw{};  // compacted operands of the fused tensor screen (single-query calls)
     bool have_tw = false;
-    unsigned long long* d_claim = nullptr;  // tile claim counter of the first pass
+    unsigned long long* d_claim = nullptr;  // tile claim counters: the general first pass, the folded net's
     unsigned long long* h_claim = nullptr;  // pinned copy after the call
     unsigned long long ntiles = 0;          // first-pass tiles of the last call
     int tile_pts = 0;                       // points per first-pass tile (0: no claim counter)
@@ -355,10 +357,23 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
     r->caps.queue_cap = qc;
     for (int i = 0; i < 4; ++i) A(&r->d_queue[i], (size_t)qc);
     A(&r->d_tiles, (size_t)VBMC_MAX_TILES);
-    A(&r->d_claim, 1);
+    A(&r->d_claim, 2);
     // compacted columns of the fused tensor screen (calls with one query)
     const bool tcnet = tc_supported(v, VBMC_PREC_BF16) || tc_supported(v, VBMC_PREC_FP16);
     const bool fused = !arena && tcnet;
+    if (fold_supported(v)) {
+        q.fstride = S + kFoldMax;
+        A(&q.fco, T * (size_t)q.fstride);
+        A(&q.fbd, T);
+        A(&q.fer, T);
+        A(&q.fx, (size_t)kMaxS);
+        A(&q.fcls, T);
+        A(&q.fst, (size_t)kFoldSt);
+        A(&q.fnode, (size_t)kFoldMax);
+        A(&q.fc32, fold_coeff_entries(v, S));
+        A(&q.fk32, (size_t)kFoldMax + kFoldOut);
+        A(&q.fxs, (size_t)S * RM);
+    }
     if (tcnet) A(&q.kcol, 2 * T);
     if (fused) {
         A(&q.kcolc, 2 * T);
@@ -447,7 +462,7 @@ extern "C" vbmc_status vbmc_result_create_batch(const vbmc_net* net, const vbmc_
     A(&ar->d_tp, 2 * (size_t)nq + 2);  // one tile prefix per wave, back to back
     A(&ar->d_stage, ar->stage_stride * (size_t)nq);
     A(&ar->d_qcount, 4);
-    A(&ar->d_claim, 1);
+    A(&ar->d_claim, 3);
     ar->queue_cap = std::max<uint64_t>(1, caps->queue_cap);
     for (int i = 0; i < 4; ++i) A(&ar->d_queue[i], (size_t)ar->queue_cap);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&ar->h_cnt, sizeof(Counters) * (size_t)nq);
@@ -575,9 +590,21 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
             return fail(VBMC_ERR_STATE, "the result has no wide-layer workspace (created with caps.wide_chunk = -1, "
                                         "or as a batch member without one)");
     }
+    // the folded net checks the queries whose set-up builds one (fold.cu); which
+    // they are is known on the device only, so the general passes are launched too
+    // and leave those queries out
+    bool fold = false;
+    for (int i = 0; i < nq; ++i) fold = fold || hq[i].fold;
+    unsigned long long* const d_unfolded = nq > 1 && d_claim ? d_claim + 2 : nullptr;
     VB_CUDA(cudaMemsetAsync(d_qcount, 0, sizeof(unsigned long long) * 4, st));
+    if (d_claim) VB_CUDA(cudaMemsetAsync(d_claim, 0, sizeof(unsigned long long) * (nq > 1 ? 3 : 2), st));
     VB_CUDA(record(ev[0]));
-    if (stages & STAGE_SETUP) launch_prologue(v, d_qs, nq, max_sr, st);
+    if (stages & STAGE_SETUP) {
+        unsigned long long max_hi = 0;
+        for (int i = 0; i < nq; ++i)
+            if (hq[i].bitmap) max_hi = std::max(max_hi, hq[i].hi);
+        launch_prologue(v, d_qs, nq, max_sr, st, max_hi, fold, d_unfolded);
+    }
     VB_CUDA(record(ev[1]));
     if (tensor && any) {
         if (!tc_supported(v, opt.precision))
@@ -599,9 +626,19 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
         }
         return cudaSuccess;
     };
+    if (any && fold) {
+        // tiles as in the general first pass; the wide-layer path has none, and its
+        // work count is one unit, which its own run takes away
+        const int mt = opt.precision == VBMC_PREC_FP32 ? simt_tile_points(v) : tc_tile_points();
+        if (wide) ntiles = (hq[0].hi - (hq[0].lo & ~31ull) + mt - 1) / mt;
+        launch_fold(v, d_qs, nq, wide ? nullptr : d_tp, ntiles, mt, !wide, wide || !d_claim ? nullptr : d_claim + 1,
+                    qsplit, 0, net->n_sm, st);
+        launch_fold64(v, d_qs, d_queue[0], d_qcount + 0, cap, q64, 3, net->n_sm, st);
+        if (wide) launch_fp64(v, d_qs, nq, d_queue[3], d_qcount + 3, cap, 0, 0, net->n_sm, st);
+    }
     if (any && wide) {
         // the chunk loop interleaves the screen and the rechecks: all of it counts as screen
-        vbmc_status fs = wide_run(net->wide, wtype, *ww, v, d_qs, hq[0].lo, hq[0].hi, d_qcount, d_queue, cap,
+        vbmc_status fs = wide_run(net->wide, wtype, *ww, v, d_qs, hq[0], hq[0].lo, hq[0].hi, d_qcount, d_queue, cap,
                                   net->n_sm, st);
         if (fs != VBMC_OK) return fail(fs, "wide-layer tensor screen launch failed");
         VB_CUDA(record(ev[2]));
@@ -616,14 +653,15 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
         if (opt.precision == VBMC_PREC_FP32) {
             if (simt_tile_points(v) == 0) return fail(VBMC_ERR_UNSUPPORTED, "layer width above 1024");
             launch_screen_simt(v, d_qs, nq, d_tp, ntiles, nullptr, nullptr, 0, qdf, 2, net->n_sm, st,
-                               (nq == 1 && small_supported(v)) ? nullptr : d_claim);
+                               (nq == 1 && small_supported(v)) ? nullptr : d_claim, d_unfolded);
             VB_CUDA(record(ev[2]));
             VB_CUDA(record(ev[4]));
             VB_CUDA(record(ev[5]));
         } else {
             // one query: screen -> split tensor pass -> FP32; many: screen -> FP32 directly
             vbmc_status sst = tc_launch_screen(net->tc, v, d_qs, nq, d_tp, ntiles, opt.precision,
-                                   nq == 1 ? qsplit : q32, nq == 1 ? 0 : 1, net->n_sm, st, tw, d_claim);
+                                   nq == 1 ? qsplit : q32, nq == 1 ? 0 : 1, net->n_sm, st, tw, d_claim,
+                                   d_unfolded);
             if (sst != VBMC_OK)
                 return fail(sst, std::string("tensor-core screen launch failed: ") + cudaGetErrorString(cudaGetLastError()));
             VB_CUDA(record(ev[2]));
@@ -676,7 +714,7 @@ vbmc_status query_extra(const vbmc_query& q, QueryExtra* x) {
 
 QueryView make_view(const vbmc_result* r, const uint8_t* d_image, const int* d_pix, int s, int k,
                     uint64_t lo, uint64_t hi, uint64_t n, const vbmc_options& opt, int qid,
-                    const QueryExtra& x = QueryExtra()) {
+                    const QueryExtra& x = QueryExtra(), bool fold = true) {
     QueryView q = r->hq;
     q.filter = x.filter;
     q.l2max = x.l2max;
@@ -693,14 +731,19 @@ QueryView make_view(const vbmc_result* r, const uint8_t* d_image, const int* d_p
     q.pix_in = d_pix;
     if (!opt.coverage) q.flip = q.flip_tie = q.ss = q.ss_tie = nullptr;
     if (!opt.bitmap) q.bitmap = nullptr;
+    // the folded net: ReLU nets at every precision whose first pass is a screen, except
+    // the FP32 pass of small nets (one thread per point: no less direct than folding)
+    // and calls with a time budget, which cuts the general first pass's tile order
+    q.fold = fold && q.fco && r->net->fold && opt.precision != VBMC_PREC_FP64 && !(opt.time_budget_ms > 0.0) &&
+             !(opt.precision == VBMC_PREC_FP32 && small_supported(r->net->v));
     return q;
 }
 
 // Enqueue the full pipeline for one query whose image/pixels are on the device.
 vbmc_status enqueue(vbmc_net* net, vbmc_result* r, const uint8_t* d_image, const int* d_pix, int s,
                     int k, uint64_t lo, uint64_t hi, uint64_t n, const vbmc_options& opt,
-                    cudaStream_t st, const QueryExtra& x = QueryExtra()) {
-    QueryView q = make_view(r, d_image, d_pix, s, k, lo, hi, n, opt, 0, x);
+                    cudaStream_t st, const QueryExtra& x = QueryExtra(), bool fold = true) {
+    QueryView q = make_view(r, d_image, d_pix, s, k, lo, hi, n, opt, 0, x, fold);
     q.budget_ns = opt.time_budget_ms > 0.0 ? (unsigned long long)(opt.time_budget_ms * 1e6) : 0ull;
     std::vector<unsigned long long> tp = tile_prefix(net->v, opt.precision, &q, 1);
     // the first pass takes its tiles from the claim counter on the fused tensor
@@ -819,8 +862,10 @@ extern "C" vbmc_status vbmc_verify_query_device(vbmc_net* net, const uint8_t* d_
     return enqueue(net, res, d_image, d_pixels, s, k, lo, h, n, *opt, (cudaStream_t)stream);
 }
 
-extern "C" vbmc_status vbmc_verify_query(vbmc_net* net, const vbmc_query* q, const vbmc_options* opt,
-                                         vbmc_result* res, void* stream) {
+namespace {
+
+vbmc_status verify_query(vbmc_net* net, const vbmc_query* q, const vbmc_options* opt, vbmc_result* res,
+                         void* stream, bool fold) {
     if (!net || !q || !res || !opt || !q->image || (!q->pixels && q->s > 0))
         return fail(VBMC_ERR_ARG, "null argument");
     if (res->net != net) return fail(VBMC_ERR_ARG, "result belongs to another net");
@@ -845,11 +890,18 @@ extern "C" vbmc_status vbmc_verify_query(vbmc_net* net, const vbmc_query* q, con
     QueryExtra x;
     st = query_extra(*q, &x);
     if (st != VBMC_OK) return st;
-    st = enqueue(net, res, res->d_image, res->d_pix_in, q->s, q->k, q->lo, h, n, *opt, stq, x);
+    st = enqueue(net, res, res->d_image, res->d_pix_in, q->s, q->k, q->lo, h, n, *opt, stq, x, fold);
     if (st != VBMC_OK) return st;
     res->image.assign(q->image, q->image + H0);
     res->pixels.assign(q->pixels, q->pixels + q->s);
     return finish(res);
+}
+
+}  // namespace
+
+extern "C" vbmc_status vbmc_verify_query(vbmc_net* net, const vbmc_query* q, const vbmc_options* opt,
+                                         vbmc_result* res, void* stream) {
+    return verify_query(net, q, opt, res, stream, true);
 }
 
 extern "C" vbmc_status vbmc_result_summary(vbmc_result* res, vbmc_summary* out) {
@@ -1105,7 +1157,7 @@ extern "C" vbmc_status vbmc_verify_batch(vbmc_net* net, const vbmc_query* querie
         // outside); captured and instantiated once per batch shape, then relaunched
         std::string sig = std::to_string(nq) + ":" + std::to_string(opt->precision) + ":" +
                           std::to_string(opt->coverage) + ":" + std::to_string(opt->bitmap) + ":" +
-                          std::to_string(opt->schedule);
+                          std::to_string(opt->schedule) + ":" + std::to_string(hrun[0].fold);
         for (int j = 0; j < nq; ++j) {
             const QueryView& h = hrun[j];
             sig += "|" + std::to_string(h.s) + "," + std::to_string(h.k) + "," + std::to_string(h.lo) + "," +
@@ -1252,7 +1304,7 @@ extern "C" vbmc_status vbmc_wide_trace(vbmc_net* net, const vbmc_query* q, int32
     qq.hi = (uint64_t)n_points;
     vbmc_options o{};
     o.precision = precision;
-    vbmc_status st = vbmc_verify_query(net, &qq, &o, res, stream);
+    vbmc_status st = verify_query(net, &qq, &o, res, stream, false);  // the traced path itself
     if (st == VBMC_OK) st = finish(res);
     wide_set_trace(nullptr);
     if (st == VBMC_OK &&
@@ -1482,6 +1534,12 @@ void apply_tuning(vbmc_net* net, const vbmc_tuning& t) {
 
 }  // namespace
 
+extern "C" vbmc_status vbmc_set_folding(vbmc_net* net, int32_t on) {
+    if (!net) return fail(VBMC_ERR_ARG, "null argument");
+    net->fold = on != 0;
+    return VBMC_OK;
+}
+
 extern "C" vbmc_status vbmc_set_tuning(vbmc_net* net, const vbmc_tuning* t) {
     if (!net || !t) return fail(VBMC_ERR_ARG, "null argument");
     apply_tuning(net, *t);
@@ -1528,7 +1586,7 @@ extern "C" vbmc_status vbmc_autotune(vbmc_net* net, const char* cache_path, vbmc
         cudaStream_t s;
         ~SGuard() { cudaStreamDestroy(s); }
     } sguard{sq};
-    st = vbmc_verify_query(net, &q, &o32, r, sq);  // prologue, tables, warm-up
+    st = verify_query(net, &q, &o32, r, sq, false);  // prologue, tables, warm-up
     if (st != VBMC_OK) return st;
     cudaEvent_t e0, e1;
     VB_CUDA(cudaEventCreate(&e0));

@@ -19,6 +19,8 @@ constexpr int kMaxS = 16;
 constexpr int kMaxR = 255;
 constexpr int kMaxWidth = 1024;
 constexpr double kTau = 1e-9;  // tie band of margins and potentials
+constexpr int kFoldMax = 128;  // neurons whose sign can change that a folded net holds (fold.cu)
+constexpr int kFoldOut = 32;   // classes (output width) it holds
 
 enum { ACT_IDENTITY = 0, ACT_SIGMOID = 1, ACT_RELU = 2 };
 
@@ -70,6 +72,7 @@ struct Counters {
     unsigned long long t_final;     // ... when its result became final (0: not yet)
     unsigned long long work;        // unfinished units: screen tiles not yet done plus
                                     // queued points not yet resolved (see work_done)
+    int folded;                     // 1: the folded net (fold.cu) checked the query's points
 };
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
@@ -127,6 +130,21 @@ struct QueryView {
     // kcolc in compacted order (padding positions "neg").
     float4* kcol;           // [total][2]
     float4* kcolc;          // [total][2]
+    // Folded net (fold.cu): what is left of the net on the box when every neuron
+    // whose sign cannot change in it is carried as the linear map it is.
+    int fold;               // 1: the call may use it (the set-up then builds it)
+    int fstride;            // row stride of fco: column p < s is pixel p, s + m is node m
+    double* fco;            // [total][fstride]: du_n = sum of these times the sources' changes
+    double* fbd;            // [total] bound on |du_n| over the box
+    double* fer;            // [total] bound on the error of du_n from rounded fco entries
+    double* fx;             // [kMaxS] max over the digits of |dv_p| / 255
+    unsigned char* fcls;    // [total] hidden neurons: 0 pos, 1 neg, 2 node (sign can change)
+    int* fst;               // [kFoldSt]: [0] 1: folded, [1] 1: more than kFoldMax nodes,
+                            //   [2 + l] nodes of hidden layer l
+    int* fnode;             // [kFoldMax] node -> neuron (concatenated index)
+    float4* fc32;           // packed FP32 coefficients, see FoldLayout
+    float4* fk32;           // [kFoldMax + kFoldOut] node (ub, c1, c2, thr); output (ub, e, em, thr)
+    float* fxs;             // [s][R] fl(dv / 255)
     Counters* cnt;
     uint32_t* bitmap;       // verdict bits (nullptr: off)
     unsigned long long bitmap_bits;
@@ -134,6 +152,11 @@ struct QueryView {
     unsigned long long* ties;
     unsigned int ties_cap;
 };
+
+constexpr int kFoldSt = 2 + kMaxL + 2;
+
+// The query's points are checked through its folded net (set by its set-up).
+__device__ __forceinline__ bool folded(const QueryView& Q) { return Q.fst && Q.fst[0]; }
 
 struct QEntry {
     unsigned long long t;
@@ -244,6 +267,28 @@ __device__ __forceinline__ unsigned long long claim_tile(unsigned long long* ctr
     if (deadline && globaltimer_ns() > deadline) return kNoTile;
     const unsigned long long g = atomicAdd(ctr, 1ull);
     return g < ntiles ? g : kNoTile;
+}
+
+// The query whose tiles tile_prefix[q] .. tile_prefix[q + 1] - 1 hold tile g.
+__device__ __forceinline__ int query_of_tile(const unsigned long long* tile_prefix, int nq, unsigned long long g) {
+    int a = 0, b = nq - 1;
+    while (a < b) {
+        const int mid = (a + b + 1) >> 1;
+        if (tile_prefix[mid] <= g) a = mid; else b = mid - 1;
+    }
+    return a;
+}
+
+// claim_tile for a general first pass: tiles of queries that the folded net
+// checks are passed over (with one query the whole launch returns instead).
+__device__ __forceinline__ unsigned long long claim_open_tile(unsigned long long* ctr, unsigned long long i,
+                                                              unsigned long long ntiles,
+                                                              unsigned long long deadline, const QueryView* qs,
+                                                              int nq, const unsigned long long* tile_prefix) {
+    for (;;) {
+        const unsigned long long g = claim_tile(ctr, i, ntiles, deadline);
+        if (g == kNoTile || nq == 1 || !ctr || !folded(qs[query_of_tile(tile_prefix, nq, g)])) return g;
+    }
 }
 
 // Mixed-radix decode: first pixel most significant.

@@ -7,8 +7,26 @@
 namespace vbmc {
 
 // FP64 base pass, tables and screen constants for nq queries (d_qs on device).
-// max_sr: max over queries of s * R.
-void launch_prologue(const NetView& net, QueryView* d_qs, int nq, int max_sr, cudaStream_t st);
+// max_sr: max over queries of s * R; max_hi: of the verdict bitmaps' bits (0: off).
+// fold: some view has its fold flag set; *d_unfolded (optional) then gains the
+// queries that did not fold.
+void launch_prologue(const NetView& net, QueryView* d_qs, int nq, int max_sr, cudaStream_t st,
+                     unsigned long long max_hi, bool fold, unsigned long long* d_unfolded);
+
+// Folded nets (fold.cu): a net whose calls may fold; the packed form of the
+// queries' rows after the base pass; the first pass over folded queries; the
+// FP64 evaluation of the folded net for the points it queued.
+bool fold_supported(const NetView& net);
+size_t fold_coeff_entries(const NetView& net, int max_s);  // float4 entries of QueryView::fc32
+void launch_fold_pack(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long* d_unfolded);
+// Tiles of mt points, numbered as in the general first pass (d_tile_prefix; null
+// with one query); work_units: the queries' work counts are in these tiles;
+// claim: tile counter (null: static tiles).
+void launch_fold(const NetView& net, const QueryView* d_qs, int nq, const unsigned long long* d_tile_prefix,
+                 unsigned long long n_tiles, int mt, bool work_units, unsigned long long* claim, Queue out,
+                 int out_level, int n_sm, cudaStream_t st);
+void launch_fold64(const NetView& net, const QueryView* d_qs, const QEntry* in, const unsigned long long* count,
+                   unsigned long long cap, Queue out, int out_level, int n_sm, cudaStream_t st);
 
 // Shape class of the FP32 SIMT screen for a net (0: unsupported).
 int simt_variant(const NetView& net);
@@ -17,12 +35,14 @@ int simt_variant(const NetView& net);
 // numbered tile_prefix[q] .. tile_prefix[q+1]-1, n_tiles in total, taken from
 // the claim counter when one is given (zeroed here; in order, under the time
 // budget: see claim_tile). Gather mode: the points are gather[0 ..
-// *gather_count). Points the FP32 bound cannot decide go to `out`.
+// *gather_count). Points the FP32 bound cannot decide go to `out`. Ranges of
+// folded queries are left out; unfolded: the number of the others (many queries).
 void launch_screen_simt(const NetView& net, const QueryView* d_qs, int nq,
                         const unsigned long long* d_tile_prefix, unsigned long long n_tiles,
                         const QEntry* gather, const unsigned long long* gather_count,
                         unsigned long long gather_cap, Queue out, int out_level, int n_sm,
-                        cudaStream_t st, unsigned long long* claim = nullptr);
+                        cudaStream_t st, unsigned long long* claim = nullptr,
+                        const unsigned long long* unfolded = nullptr);
 
 // Points per tile of the SIMT screen for this net (its range-pass variant).
 int simt_tile_points(const NetView& net);
@@ -57,7 +77,7 @@ void launch_margin64(const NetView& net, const QueryView* d_qs, unsigned long lo
 void launch_stamp_final(QueryView* d_qs, int nq, cudaStream_t st);
 
 // Single prologue steps (the allocation-free entry point runs these directly).
-void launch_pro_init(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st);
+void launch_pro_init(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long max_hi);
 void launch_pro_layer(const NetView& net, QueryView* d_qs, int nq, int l, cudaStream_t st);
 
 // Upper bound of the spectral norm of the row-major m x n matrix A (host data;

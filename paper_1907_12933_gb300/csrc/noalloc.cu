@@ -177,7 +177,7 @@ extern "C" vbmc_status vbmc_verify_range_fp64_noalloc(const vbmc_net* net, const
         e = cudaMemsetAsync(out->bitmap, 0, 4ull * ((hi + 31) / 32), st);
     if (e != cudaSuccess) return set_error(VBMC_ERR_CUDA, cudaGetErrorString(e));
     // k_pro_init resets the counters in the scratch and validates the pixels
-    launch_pro_init(v, d_q, 1, st);
+    launch_pro_init(v, d_q, 1, st, out->bitmap ? hi : 0);
     for (int l = 1; l <= v.L; ++l) launch_pro_layer(v, d_q, 1, l, st);
     k_na_class<<<1, 1, 0, st>>>(v, d_q);
     if (hi > lo) {

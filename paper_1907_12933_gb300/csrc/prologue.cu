@@ -20,7 +20,7 @@ namespace vbmc {
 __global__ void k_pro_init(NetView net, QueryView* qs, int nq) {
     QueryView& Q = qs[blockIdx.x];
     const int H0 = net.dims[0];
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && blockIdx.y == 0) {
         bool ok = Q.s >= 0 && Q.s <= kMaxS;
         for (int p = 0; p < Q.s && ok; ++p) {
             int v = Q.pix_in[p];
@@ -39,22 +39,26 @@ __global__ void k_pro_init(NetView net, QueryView* qs, int nq) {
         c->t0 = globaltimer_ns();
         c->t_final = 0;
         c->work = Q.ntiles;
+        c->folded = 0;
+        if (Q.fst) Q.fst[0] = Q.fst[1] = 0;
         for (int p = 0; p < Q.s; ++p) {
             int v = Q.pix_in[p];
             Q.pix[p] = (ok && v >= 0 && v < H0) ? v : 0;  // never index out of range
         }
     }
     // results start from zero on every call
+    const int nb = gridDim.y, bt = blockIdx.y * blockDim.x + threadIdx.x, nt = nb * blockDim.x;
     if (Q.flip)
-        for (int w = threadIdx.x; w < net.flip_words; w += blockDim.x) Q.flip[w] = Q.flip_tie[w] = 0u;
+        for (int w = bt; w < net.flip_words; w += nt) Q.flip[w] = Q.flip_tie[w] = 0u;
     if (Q.ss)
-        for (int w = threadIdx.x; w < net.ss_words; w += blockDim.x) Q.ss[w] = Q.ss_tie[w] = 0u;
+        for (int w = bt; w < net.ss_words; w += nt) Q.ss[w] = Q.ss_tie[w] = 0u;
     if (Q.bitmap && Q.hi > 0) {
         const unsigned long long nw = (Q.hi + 31) / 32;
         uint4* b4 = reinterpret_cast<uint4*>(Q.bitmap);
-        for (unsigned long long w = threadIdx.x; w < nw / 4; w += blockDim.x) b4[w] = make_uint4(0, 0, 0, 0);
-        for (unsigned long long w = (nw / 4) * 4 + threadIdx.x; w < nw; w += blockDim.x) Q.bitmap[w] = 0u;
+        for (unsigned long long w = bt; w < nw / 4; w += nt) b4[w] = make_uint4(0, 0, 0, 0);
+        for (unsigned long long w = (nw / 4) * 4 + bt; w < nw; w += nt) Q.bitmap[w] = 0u;
     }
+    if (blockIdx.y != 0) return;
     __syncthreads();
     for (int e = threadIdx.x; e < Q.s * Q.R; e += blockDim.x) {
         int p = e / Q.R, d = e % Q.R;
@@ -62,6 +66,11 @@ __global__ void k_pro_init(NetView net, QueryView* qs, int nq) {
         int w = v + d - Q.k;
         w = w < 0 ? 0 : (w > 255 ? 255 : w);
         Q.dv[e] = w - v;
+        if (Q.fold) Q.fxs[e] = __fdiv_rn((float)(w - v), 255.f);
+    }
+    if (Q.fold && threadIdx.x < Q.s) {  // the largest change of each pixel (steps -k and k, clipped)
+        const int v = Q.image[Q.pix[threadIdx.x]];
+        Q.fx[threadIdx.x] = (double)max(min(Q.k, 255 - v), min(Q.k, v)) / 255.0;
     }
 }
 
@@ -75,11 +84,75 @@ __device__ __forceinline__ double act64(int act, double u) {
 // the FP64 error of the result: rounding of the K products and sums,
 // (K + 2) 2^-53 (sum_j |w_j h_j| + |b|), plus the input errors propagated,
 // sum_j |w_j| e_j (the activations are 1-Lipschitz).
-__global__ void k_pro_layer(NetView net, QueryView* qs, int nq, int l) {
+//
+// With Q.fold the warp also writes its neuron's row of the folded net (fold.cu):
+// du_i as a linear form in the s pixel changes and the output changes of the
+// nodes of earlier layers, the row of W_l times the rows of the layer below
+// ("pos" inputs), W_l itself in the columns of that layer's nodes; the bound
+// B_i on |du_i| over the box; and the class that follows from it. Each block
+// lists the layer below's "pos" neurons and nodes once, in order. A row's
+// columns lie across the lanes; fewer than 32 of them split the inputs too.
+__global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, int nq, int l) {
+    __shared__ short plist[kMaxWidth], clist[kFoldMax];
+    __shared__ int wpos[8], wnode[8];
     const QueryView& Q = qs[blockIdx.y];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x * (blockDim.x >> 5) + warp;
     const int K = net.dims[l - 1], N = net.dims[l];
+    const int offp = l >= 2 ? net.noff[l - 1] : 0;
+    const bool fold = Q.fold != 0;
+    int npos = 0, nnode = 0, nb = 0;  // the layer below: "pos" neurons, nodes; nodes of the layers below it
+    bool rows = fold;                 // false: more nodes than a folded net holds
+    if (fold && l >= 2) {
+        const unsigned char* cls = Q.fcls + offp;
+        unsigned mp[kMaxWidth / 256], mn[kMaxWidth / 256];
+        int cp = 0, cn = 0;
+#pragma unroll
+        for (int e = 0; e < kMaxWidth / 256; ++e) {
+            const int j = warp * (kMaxWidth / 8) + 32 * e + lane;
+            const int c = j < K ? cls[j] : 1;
+            mp[e] = __ballot_sync(0xffffffffu, c == 0);
+            mn[e] = __ballot_sync(0xffffffffu, c == 2);
+            cp += __popc(mp[e]);
+            cn += __popc(mn[e]);
+        }
+        if (lane == 0) {
+            wpos[warp] = cp;
+            wnode[warp] = cn;
+        }
+        for (int m = 1; m < l - 1; ++m) nb += Q.fst[2 + m];
+        __syncthreads();
+        int bp = 0, bn = 0;
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) {
+                bp += wpos[w];
+                bn += wnode[w];
+            }
+            npos += wpos[w];
+            nnode += wnode[w];
+        }
+        rows = nb + nnode <= kFoldMax;  // the same for every block (and for the layers above)
+        if (rows) {
+#pragma unroll
+            for (int e = 0; e < kMaxWidth / 256; ++e) {
+                const int j = warp * (kMaxWidth / 8) + 32 * e + lane;
+                const unsigned below = (1u << lane) - 1u;
+                if ((mp[e] >> lane) & 1u) plist[bp + __popc(mp[e] & below)] = (short)j;
+                if ((mn[e] >> lane) & 1u) {
+                    const int c = bn + __popc(mn[e] & below);
+                    clist[c] = (short)j;
+                    if (blockIdx.x == 0) Q.fnode[nb + c] = offp + j;
+                }
+                bp += __popc(mp[e]);
+                bn += __popc(mn[e]);
+            }
+        }
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            Q.fst[2 + l - 1] = nnode;
+            if (!rows) Q.fst[1] = 1;
+        }
+        __syncthreads();
+    }
     if (i >= N) return;
     const float* Wr = net.W[l] + (size_t)i * K;
     double acc = 0.0, mag = 0.0, prop = 0.0;
@@ -105,21 +178,86 @@ __global__ void k_pro_layer(NetView net, QueryView* qs, int nq, int l) {
         mag += __shfl_xor_sync(0xffffffffu, mag, o);
         prop += __shfl_xor_sync(0xffffffffu, prop, o);
     }
+    const int n = net.noff[l] + i;
+    const double bi = (double)net.b[l][i];
+    const double u = acc + bi;
+    // (x/255 carries one more rounding on layer 1; activations add 2^-50 |u|)
+    const double eu = ((K + 4) * 0x1p-53 * (mag + fabs(bi)) + prop + 0x1p-50 * fabs(u)) * (1.0 + 1e-9);
     if (lane == 0) {
-        const double bi = (double)net.b[l][i];
-        double u = acc + bi;
-        Q.ub[net.noff[l] + i] = u;
-        Q.hb[net.noff[l] + i] = (l < net.L) ? act64(net.act, u) : u;
-        // (x/255 carries one more rounding on layer 1; activations add 2^-50 |u|)
-        const double e = ((K + 4) * 0x1p-53 * (mag + fabs(bi)) + prop + 0x1p-50 * fabs(u)) * (1.0 + 1e-9);
-        Q.eub[net.noff[l] + i] = e;
+        Q.ub[n] = u;
+        Q.hb[n] = (l < net.L) ? act64(net.act, u) : u;
+        Q.eub[n] = eu;
+    }
+    if (!rows) return;
+    const int s = Q.s;
+    double* row = Q.fco + (size_t)n * Q.fstride;
+    double B = 0.0, er = 0.0;  // sum of |coefficient| x bound of its source; error of the carried rows
+    if (l == 1) {
+        if (lane < s) {
+            const double w = (double)Wr[Q.pix[lane]];
+            row[lane] = w;
+            B = fabs(w) * Q.fx[lane];
+        }
+    } else {
+        // the rows of the layer below carry errors fer, and each sum over npos inputs
+        // rounds by at most (npos + 4) 2^-53 sum_j |w_j| B_j
+        double e1 = 0.0, m1 = 0.0;
+        for (int jj = lane; jj < npos; jj += 32) {
+            const int j = plist[jj];
+            const double w = fabs((double)Wr[j]);
+            e1 += w * Q.fer[offp + j];
+            m1 += w * Q.fbd[offp + j];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            e1 += __shfl_xor_sync(0xffffffffu, e1, o);
+            m1 += __shfl_xor_sync(0xffffffffu, m1, o);
+        }
+        er = (e1 + (npos + 4) * 0x1p-53 * m1) * (1.0 + 1e-9);
+        const int S = s + nb;
+        const double* prev = Q.fco + (size_t)offp * Q.fstride;
+        for (int k0 = 0; k0 < S; k0 += 32) {
+            int sp = 1;  // lanes per input: a power of two that holds the columns left
+            while (sp < 32 && sp < S - k0) sp <<= 1;
+            const int k = k0 + (lane & (sp - 1)), g = lane / sp, G = 32 / sp;
+            double a = 0.0;
+            if (k < S) {
+#pragma unroll 8
+                for (int jj = g; jj < npos; jj += G) {
+                    const int j = plist[jj];
+                    a = fma((double)Wr[j], prev[(size_t)j * Q.fstride + k], a);
+                }
+            }
+            for (int o = sp; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (g == 0 && k < S) {
+                row[k] = a;
+                B += fabs(a) * (k < s ? Q.fx[k] : Q.fbd[Q.fnode[k - s]]);
+            }
+        }
+        for (int c = lane; c < nnode; c += 32) {
+            const double w = (double)Wr[clist[c]];
+            row[S + c] = w;
+            B += fabs(w) * Q.fbd[offp + clist[c]];
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) B += __shfl_xor_sync(0xffffffffu, B, o);
+    if (lane == 0) {
+        B = B * (1.0 + 1e-9) + er;
+        Q.fbd[n] = B;
+        Q.fer[n] = er;
+        // a neuron keeps its sign, clear of the tie band, over the whole box
+        if (l < net.L) {
+            const bool keeps = fabs(u) > (B + eu) * (1.0 + 1e-6) + 4.0 * kTau;
+            Q.fcls[n] = keeps ? (u >= 0.0 ? 0 : 1) : 2;
+        }
     }
 }
 
 __global__ void k_pro_tables(NetView net, QueryView* qs, int nq) {
     const QueryView& Q = qs[blockIdx.y];
     const int e = blockIdx.x;  // e = p * R + d
-    if (e >= Q.s * Q.R) return;
+    if (e >= Q.s * Q.R || folded(Q)) return;
     const int p = e / Q.R;
     const int H0 = net.dims[0], H1 = net.dims[1];
     const double step = (double)Q.dv[e] / 255.0;
@@ -164,6 +302,7 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 __global__ void k_pro_finish(NetView net, QueryView* qs, int nq) {
     __shared__ double red[33];
     QueryView& Q = qs[blockIdx.x];
+    if (folded(Q)) return;
     const int L = net.L, HL = net.dims[L];
     const double* y = Q.ub + net.noff[L];
     if (threadIdx.x == 0) {
@@ -250,20 +389,28 @@ void launch_stamp_final(QueryView* d_qs, int nq, cudaStream_t st) {
     k_stamp_final<<<(nq + 127) / 128, 128, 0, st>>>(d_qs, nq);
 }
 
-void launch_pro_init(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st) {
-    k_pro_init<<<nq, 256, 0, st>>>(net, d_qs, nq);
+// Blocks per query that clear the result buffers: one for the small masks, more
+// where a verdict bitmap makes them large (a single block of 256 threads clears
+// 1.4 MB in about 40 us), fewer when many queries fill the chip by themselves.
+static unsigned clear_blocks(int nq, unsigned long long max_hi) {
+    const unsigned long long b = 1 + max_hi / (32ull * 4 * 256 * 4);
+    const unsigned long long most = nq >= 64 ? 4 : 256 / (unsigned)nq;
+    return (unsigned)(b < most ? b : most);
+}
+
+void launch_pro_init(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long max_hi) {
+    k_pro_init<<<dim3((unsigned)nq, clear_blocks(nq, max_hi)), 256, 0, st>>>(net, d_qs, nq);
 }
 
 void launch_pro_layer(const NetView& net, QueryView* d_qs, int nq, int l, cudaStream_t st) {
     k_pro_layer<<<dim3((net.dims[l] + 7) / 8, nq), 256, 0, st>>>(net, d_qs, nq, l);
 }
 
-void launch_prologue(const NetView& net, QueryView* d_qs, int nq, int max_sr, cudaStream_t st) {
-    k_pro_init<<<nq, 256, 0, st>>>(net, d_qs, nq);
-    for (int l = 1; l <= net.L; ++l) {
-        dim3 grid((net.dims[l] + 7) / 8, nq);
-        k_pro_layer<<<grid, 256, 0, st>>>(net, d_qs, nq, l);
-    }
+void launch_prologue(const NetView& net, QueryView* d_qs, int nq, int max_sr, cudaStream_t st,
+                     unsigned long long max_hi, bool fold, unsigned long long* d_unfolded) {
+    launch_pro_init(net, d_qs, nq, st, max_hi);
+    for (int l = 1; l <= net.L; ++l) launch_pro_layer(net, d_qs, nq, l, st);
+    if (fold) launch_fold_pack(net, d_qs, nq, st, d_unfolded);
     if (max_sr > 0) k_pro_tables<<<dim3(max_sr, nq), 256, 0, st>>>(net, d_qs, nq);
     k_pro_finish<<<nq, 256, 0, st>>>(net, d_qs, nq);
 }

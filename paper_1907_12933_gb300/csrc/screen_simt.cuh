@@ -811,7 +811,8 @@ __global__ void __launch_bounds__(THREADS, PPW * NQ <= 64 ? 2 : 1)
 k_screen_simt(NetView net, const QueryView* __restrict__ qs, int nq,
               const unsigned long long* __restrict__ tile_prefix, unsigned long long n_tiles,
               const QEntry* __restrict__ gather, const unsigned long long* __restrict__ gather_count,
-              unsigned long long gather_cap, Queue out, int out_level, unsigned long long* claim) {
+              unsigned long long gather_cap, Queue out, int out_level, unsigned long long* claim,
+              const unsigned long long* __restrict__ unfolded) {
     using Sm = SimtSmem<PPW, NQ>;
     constexpr int MT = Sm::MT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -820,6 +821,8 @@ k_screen_simt(NetView net, const QueryView* __restrict__ qs, int nq,
     const int L = net.L;
 
     if (ONEQ) nq = 1;
+    // the folded net checks the query's range, or every query's (fold.cu)
+    if (!gather && (nq == 1 ? folded(qs[0]) : (unfolded && *unfolded == 0))) return;
     // compacted columns: one query whose set-up built them (tensor-screen calls)
     const bool cmp = ONEQ && qs[0].compact;
     unsigned long long tiles = n_tiles;
@@ -835,7 +838,7 @@ k_screen_simt(NetView net, const QueryView* __restrict__ qs, int nq,
     const unsigned long long deadline =
         (!gather && qs[0].budget_ns) ? qs[0].cnt->t0 + qs[0].budget_ns : 0ull;
     for (unsigned long long ti = 0;; ++ti) {
-        if (threadIdx.x == 0) S.g = claim_tile(ctr, ti, tiles, deadline);
+        if (threadIdx.x == 0) S.g = claim_open_tile(ctr, ti, tiles, deadline, qs, nq, tile_prefix);
         __syncthreads();
         const unsigned long long g = S.g;
         __syncthreads();  // every thread has read S.g before the next claim overwrites it
@@ -855,12 +858,7 @@ k_screen_simt(NetView net, const QueryView* __restrict__ qs, int nq,
                     q = (int)e.q;
                 }
             } else {
-                int lo = 0, hi = nq - 1;
-                while (lo < hi) {
-                    int mid = (lo + hi + 1) >> 1;
-                    if (tile_prefix[mid] <= g) lo = mid; else hi = mid - 1;
-                }
-                q = lo;
+                q = query_of_tile(tile_prefix, nq, g);
                 const QueryView& Q = qs[q];
                 t = (Q.lo & ~31ull) + (g - tile_prefix[q]) * MT + m;
                 ok = t >= Q.lo && t < Q.hi;
@@ -1093,7 +1091,7 @@ template <int PPW, int NQ>
 void launch_variant(const NetView& net, const QueryView* d_qs, int nq, const unsigned long long* tp,
                     unsigned long long n_tiles, const QEntry* gather, const unsigned long long* gc,
                     unsigned long long gcap, Queue out, int level, int n_sm, cudaStream_t st,
-                    unsigned long long* claim = nullptr) {
+                    unsigned long long* claim, const unsigned long long* unfolded) {
     const size_t smem = sizeof(SimtSmem<PPW, NQ>);
     auto kern = nq == 1 ? k_screen_simt<PPW, NQ, true> : k_screen_simt<PPW, NQ, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1103,7 +1101,7 @@ void launch_variant(const NetView& net, const QueryView* d_qs, int nq, const uns
     unsigned long long grid = (unsigned long long)n_sm * per_sm;
     if (!gather && n_tiles < grid) grid = n_tiles ? n_tiles : 1;
     kern<<<(unsigned)grid, THREADS, smem, st>>>(net, d_qs, nq, tp, n_tiles, gather, gc, gcap, out,
-                                                level, claim);
+                                                level, claim, unfolded);
 }
 
 }  // namespace simt

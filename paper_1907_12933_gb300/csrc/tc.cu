@@ -170,7 +170,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 k_tc(const __grid_constant__ TcParams P, NetView net, const QueryView* __restrict__ qs, int nq,
      const unsigned long long* __restrict__ tile_prefix, const QEntry* __restrict__ gather_in,
      const unsigned long long* __restrict__ gcount, unsigned long long gcap, Queue out,
-     int out_level, unsigned long long* claim_ctr) {
+     int out_level, unsigned long long* claim_ctr, const unsigned long long* __restrict__ unfolded) {
+    // nothing to do where the folded net checks every query (fold.cu)
+    if (nq == 1 ? folded(qs[0]) : (unfolded && *unfolded == 0)) return;
     // the split pass always reads a queue (gather mode), the screen always ranges
     // (launch_k): the mode is known at compile time, and each instantiation keeps
     // only its own mode's code
@@ -218,7 +220,7 @@ k_tc(const __grid_constant__ TcParams P, NetView net, const QueryView* __restric
         tc::mbar_init(bar(CLAIMB(1)), 1);
         S.abort_flag = 0;
         S.curq = -1;
-        S.claim[0] = claim_tile(ctr, 0, ntiles, deadline);  // this CTA's first tile
+        S.claim[0] = claim_open_tile(ctr, 0, ntiles, deadline, qs, nq, tile_prefix);  // this CTA's first tile
         // loop sizes per layer; compacted: the widths of the (single) query's
         // non-"neg" columns, rounded up to 64, from its set-up
         for (int l = 2; l <= L; ++l) {
@@ -373,19 +375,11 @@ k_tc(const __grid_constant__ TcParams P, NetView net, const QueryView* __restric
             if (g == kNoTile) break;
             unsigned long long nxt = kNoTile;
             if (wtid == kAtomT) {
-                nxt = claim_tile(ctr, ti + 1, ntiles, deadline);
+                nxt = claim_open_tile(ctr, ti + 1, ntiles, deadline, qs, nq, tile_prefix);
                 if (pend_n) work_done(pend_c, pend_n);  // after the barrier that followed its pushes
                 pend_n = 0;
             }
-            int q = 0;
-            if (!SPLIT) {
-                int a = 0, b = nq - 1;
-                while (a < b) {
-                    const int mid = (a + b + 1) >> 1;
-                    if (tile_prefix[mid] <= g) a = mid; else b = mid - 1;
-                }
-                q = a;
-            }
+            const int q = SPLIT ? 0 : query_of_tile(tile_prefix, nq, g);
             const QueryView& Q = qs[q];
             const int s = Q.s, R = Q.R;
             const int ni = s >= 2 ? 2 : s;       // inner digits handled per row
@@ -1130,6 +1124,7 @@ __global__ void k_classes_tc(const __grid_constant__ TcParams P, NetView net, Qu
     __shared__ double Bh[1024];
     __shared__ double red[64];
     QueryView& Q = qs[blockIdx.x];
+    if (folded(Q)) return;
     const int L = P.L, H1 = net.dims[1];
     const double u24 = 0x1p-24;
     const double uq = P.bf16 ? 0x1p-8 : 0x1p-11;
@@ -1231,6 +1226,7 @@ __global__ void k_classes_tc(const __grid_constant__ TcParams P, NetView net, Qu
 __global__ void __launch_bounds__(512) k_compact_perm(const __grid_constant__ TcParams P, NetView net,
                                                       QueryView* qs) {
     QueryView& Q = qs[0];
+    if (folded(Q)) return;
     __shared__ int wsum[16];
     __shared__ int cnt1_s, kc1_s;
     const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
@@ -1291,7 +1287,7 @@ __global__ void k_compact_gather(const __grid_constant__ TcParams P, NetView net
                                  CompactDst dst) {
     const QueryView& Q = qs[0];
     const int l = 2 + (int)blockIdx.y;
-    if (l > P.L) return;
+    if (l > P.L || folded(Q)) return;
     const TcLayer& ly = P.ly[l];
     const int K = ly.K;
     const bool out = l == P.L;
@@ -1868,26 +1864,30 @@ template <bool SPLIT, bool BF>
 static void launch_k(const TcParams& P, const NetView& v, const QueryView* d_q, int nq,
                      const unsigned long long* tp, unsigned long long ntiles, const QEntry* g,
                      const unsigned long long* gc, unsigned long long cap, Queue out, int level,
-                     int n_sm, cudaStream_t st, unsigned long long* claim) {
+                     int n_sm, cudaStream_t st, unsigned long long* claim, const unsigned long long* unfolded) {
     const size_t smem = sizeof(TcSmem) + 1024;
     auto kern = k_tc<SPLIT, BF>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     unsigned grid = (unsigned)n_sm;
     if (!g && ntiles < grid) grid = (unsigned)(ntiles ? ntiles : 1);
-    kern<<<grid, TC_THREADS, smem, st>>>(P, v, d_q, nq, tp, g, gc, cap, out, level, claim);
+    kern<<<grid, TC_THREADS, smem, st>>>(P, v, d_q, nq, tp, g, gc, cap, out, level, claim, unfolded);
 }
 
 vbmc_status tc_launch_screen(TcNet& tc, const NetView& v, const QueryView* d_q, int nq,
                              const unsigned long long* d_tile_prefix, unsigned long long ntiles,
                              int precision, Queue out, int out_level, int n_sm, cudaStream_t st,
-                             TcQueryWork* qw, unsigned long long* d_claim) {
+                             TcQueryWork* qw, unsigned long long* d_claim, const unsigned long long* d_unfolded) {
     const bool bf = precision == VBMC_PREC_BF16;
     TcParams Pc;
     if (qw && nq == 1 && !compact_params(tc.prec[bf ? 0 : 1].p, v, *qw, bf ? 0 : 1, Pc)) return VBMC_ERR_CUDA;
     const TcParams& P = (qw && nq == 1) ? Pc : tc.prec[bf ? 0 : 1].p;
     if (d_claim && cudaMemsetAsync(d_claim, 0, sizeof(unsigned long long), st) != cudaSuccess) return VBMC_ERR_CUDA;
-    if (bf) launch_k<false, true>(P, v, d_q, nq, d_tile_prefix, ntiles, nullptr, nullptr, 0, out, out_level, n_sm, st, d_claim);
-    else launch_k<false, false>(P, v, d_q, nq, d_tile_prefix, ntiles, nullptr, nullptr, 0, out, out_level, n_sm, st, d_claim);
+    if (bf)
+        launch_k<false, true>(P, v, d_q, nq, d_tile_prefix, ntiles, nullptr, nullptr, 0, out, out_level, n_sm, st,
+                              d_claim, d_unfolded);
+    else
+        launch_k<false, false>(P, v, d_q, nq, d_tile_prefix, ntiles, nullptr, nullptr, 0, out, out_level, n_sm, st,
+                               d_claim, d_unfolded);
     return cudaPeekAtLastError() == cudaSuccess ? VBMC_OK : VBMC_ERR_CUDA;  // the caller reports the error
 }
 
@@ -1898,8 +1898,8 @@ vbmc_status tc_launch_gather(TcNet& tc, const NetView& v, const QueryView* d_q, 
     TcParams Pc;
     if (qw && !compact_params(tc.prec[bf ? 0 : 1].p, v, *qw, bf ? 0 : 1, Pc)) return VBMC_ERR_CUDA;
     const TcParams& P = qw ? Pc : tc.prec[bf ? 0 : 1].p;
-    if (bf) launch_k<true, true>(P, v, d_q, 1, nullptr, 0, in, in_count, cap, out, 1, n_sm, st, nullptr);
-    else launch_k<true, false>(P, v, d_q, 1, nullptr, 0, in, in_count, cap, out, 1, n_sm, st, nullptr);
+    if (bf) launch_k<true, true>(P, v, d_q, 1, nullptr, 0, in, in_count, cap, out, 1, n_sm, st, nullptr, nullptr);
+    else launch_k<true, false>(P, v, d_q, 1, nullptr, 0, in, in_count, cap, out, 1, n_sm, st, nullptr, nullptr);
     return cudaPeekAtLastError() == cudaSuccess ? VBMC_OK : VBMC_ERR_CUDA;  // the caller reports the error
 }
 

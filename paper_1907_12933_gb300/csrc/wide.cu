@@ -1031,18 +1031,23 @@ void wide_work_free(WideWork& w) {
 }
 
 vbmc_status wide_run(const WideNet& wn, int type, WideWork& w, const NetView& v, QueryView* d_q,
-                     unsigned long long lo, unsigned long long hi, unsigned long long* d_qcount,
+                     const QueryView& hq, unsigned long long lo, unsigned long long hi, unsigned long long* d_qcount,
                      QEntry* const* d_queue, unsigned long long cap, int n_sm, cudaStream_t st) {
     if (type < 0 || type >= WIDE_NTYPES || !wn.prec[type].ready || !w.chunk) return VBMC_ERR_STATE;
     const WDev dv{w.scale, w.n2, w.r2, w.sN, w.sR, w.sE, w.unc, w.fcnt, w.flist, w.chunk, w.row_bytes};
     Queue q32{d_queue[1], d_qcount + 1, cap};
     Queue qdf{d_queue[2], d_qcount + 2, cap};
     Queue q64{d_queue[3], d_qcount + 3, cap};
+    // the folded net (fold.cu) checks the query where its set-up built one: the
+    // chunks, which clear a workspace each, are then not started
+    if (hq.fold) {
+        int fst = 0;
+        if (cudaMemcpyAsync(&fst, hq.fst, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess)
+            return VBMC_ERR_CUDA;
+        if (fst) hi = lo;
+    }
     // the query's error flags (for waits that gave up) live in its counters
-    QueryView hq;
-    if (cudaMemcpyAsync(&hq, d_q, sizeof(QueryView), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-        return VBMC_ERR_CUDA;
     unsigned int* err = &hq.cnt->err;
     for (unsigned long long c0 = lo; c0 < hi; c0 += w.chunk) {
         const unsigned long long count = std::min<unsigned long long>(w.chunk, hi - c0);

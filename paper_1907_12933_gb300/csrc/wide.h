@@ -88,10 +88,10 @@ struct WideTrace {
 };
 void wide_set_trace(const WideTrace* t);
 
-// Screen [lo, hi) of query d_q[0] chunk by chunk. Each chunk's undecided points
+// Screen [lo, hi) of query d_q[0] (hq: its host copy) chunk by chunk, nothing where it folded. Each chunk's undecided points
 // go through the FP32 (queue level 1), double-float (2) and FP64 (3) passes
 // before the next chunk starts; the queue counters are reset per chunk.
-vbmc_status wide_run(const WideNet& wn, int type, WideWork& w, const NetView& v, QueryView* d_q,
+vbmc_status wide_run(const WideNet& wn, int type, WideWork& w, const NetView& v, QueryView* d_q, const QueryView& hq,
                      unsigned long long lo, unsigned long long hi, unsigned long long* d_qcount,
                      QEntry* const* d_queue, unsigned long long cap, int n_sm, cudaStream_t st);
 
