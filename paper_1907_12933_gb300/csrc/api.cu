@@ -372,6 +372,7 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
         A(&q.fnode, (size_t)kFoldMax);
         A(&q.fc32, fold_coeff_entries(v, S));
         A(&q.fk32, (size_t)kFoldMax + kFoldOut);
+        A(&q.fe64, (size_t)kFoldMax + kFoldOut);
         A(&q.fxs, (size_t)S * RM);
     }
     if (tcnet) A(&q.kcol, 2 * T);

@@ -144,6 +144,7 @@ struct QueryView {
     int* fnode;             // [kFoldMax] node -> neuron (concatenated index)
     float4* fc32;           // packed FP32 coefficients, see FoldLayout
     float4* fk32;           // [kFoldMax + kFoldOut] node (ub, c1, c2, thr); output (ub, e, em, thr)
+    double* fe64;           // [kFoldMax + kFoldOut] error bound of a node's or output's FP64 evaluation
     float* fxs;             // [s][R] fl(dv / 255)
     Counters* cnt;
     uint32_t* bitmap;       // verdict bits (nullptr: off)

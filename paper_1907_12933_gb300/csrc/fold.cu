@@ -17,9 +17,10 @@
 //   k_fold_pack   per query: the rows of nodes and outputs as FP32 in groups of 4,
 //                 their error bounds; D and the margin of the unperturbed image
 //   k_fold        the first pass: 4 points per thread, FP32 on CUDA cores
-//   k_fold64      the points it left undecided, the same rows in FP64
-// and what is still undecided (values in the tie band) goes to the FP64 pass on
-// the whole net. A query with more than kFoldMax nodes is not folded; its general
+//   k_fold64      the points it left undecided, a warp each, the same rows in FP64:
+//                 every result by its definition, sign ties and margin ties included
+// and what lies within its error of the tie band's edge (about 1e-12 around tau)
+// goes to the FP64 pass on the whole net. A query with more than kFoldMax nodes is not folded; its general
 // passes run instead (they return at once for folded queries).
 //
 // Error of k_fold, constant per node (u = 2^-24, K sources, M_n = sum_k |c_nk| bound
@@ -77,7 +78,7 @@ __device__ __forceinline__ int out_of_row(int i, int D) { return i == 0 ? D : (i
 
 __global__ void __launch_bounds__(256) k_fold_pack(NetView net, QueryView* qs, unsigned long long* unfolded) {
     __shared__ FoldShape f;
-    __shared__ double eh[kFoldMax], eo[kFoldOut];
+    __shared__ double eh[kFoldMax], eo[kFoldOut], eh64[kFoldMax];
     __shared__ int D_s;
     QueryView& Q = qs[blockIdx.x];
     if (!Q.fold || Q.fst[1] || (Q.cnt->err & DERR_PIXELS)) {
@@ -117,22 +118,28 @@ __global__ void __launch_bounds__(256) k_fold_pack(NetView net, QueryView* qs, u
         for (int i = threadIdx.x; i < f.n[l]; i += blockDim.x) {
             const int nn = neuron(l, i);
             const double* row = Q.fco + (size_t)nn * Q.fstride;
-            double M = 0.0, pr = 0.0;
+            double M = 0.0, pr = 0.0, pr64 = 0.0;
             for (int p = 0; p < s; ++p) M += fabs(row[p]) * Q.fx[p];
             for (int m = 0; m < cb; ++m) {
                 const double w = fabs(row[s + m]);
                 M += w * (Q.fbd[Q.fnode[m]] + eh[m]);
                 pr += w * eh[m];
+                pr64 += w * eh64[m];
             }
             const double ub = Q.ub[nn], B = Q.fbd[nn];
             const float ub32 = (float)ub;
             const double ed = (s + cb + 4) * 0x1p-24 * 1.00001 * M + pr + Q.fer[nn] + 1e-37;
             const double e = (ed + fabs((double)ub32 - ub) + Q.eub[nn] + 0x1p-24 * 1.001 * (fabs(ub) + B + ed)) *
                              (1.0 + 1e-9);
+            // the same in FP64 (u = 2^-53; x_p = dv_p / 255 rounds once)
+            const double e64 = ((s + cb + 5) * 0x1p-53 * M + pr64 + Q.fer[nn] + Q.eub[nn] +
+                                0x1p-51 * (fabs(ub) + B)) * (1.0 + 1e-9);
+            Q.fe64[l < L ? cb + i : kFoldMax + i] = e64;
             const float e2 = __double2float_ru(e + 2.0 * kTau);
             const float thr = fabs(ub) < kTau ? INFINITY : e2;  // a base tie: every sign is a tie
             if (l < L) {
                 eh[cb + i] = e;
+                eh64[cb + i] = e64;
                 Q.fk32[cb + i] = make_float4(ub32, ub >= 0.0 ? 0.f : ub32, ub >= 0.0 ? -ub32 : 0.f, thr);
             } else {
                 eo[i] = e + 0x1p-23 * 1.001 * (fabs(ub) + B);
@@ -449,115 +456,170 @@ __global__ void __launch_bounds__(FT) k_fold(NetView net, const QueryView* __res
     if (cur >= 0) flush();
 }
 
-// Points k_fold left undecided, one thread each: the folded rows in FP64. The
-// error bound follows the values: fer_n, (K + 4) 2^-53 sum |c_nk x_k| and the
-// sources' errors. What it cannot decide lies in the tie band: the FP64 pass.
-__global__ void __launch_bounds__(128) k_fold64(NetView net, const QueryView* __restrict__ qs,
-                                                const QEntry* __restrict__ in,
-                                                const unsigned long long* __restrict__ count,
-                                                unsigned long long cap, Queue out, int out_level) {
+// ---- FP64 evaluation of one point by a warp
+
+constexpr int F64W = 4;                  // warps per CTA of k_fold64
+constexpr int kSetW = kFoldMax / 32 + 1;  // words of a set of nodes, then of outputs
+
+struct Fold64 {
+    double x[kMaxS + kFoldMax];        // the point's sources
+    uint32_t ch[kSetW], ti[kSetW];     // rows that changed sign, rows whose sign is a tie
+    int nch[kMaxL + 1], nti[kMaxL + 1];  // how many of each, per layer
+};
+
+__device__ __forceinline__ double warp_max(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+// Point t of query Q by the definitions (Eq. 10 / Eq. 11 margin *m; signs and sign
+// ties when coverage is on). A lane holds a row of a layer: its chain of FMAs over
+// the sources is as long as the row, and a layer's rows run side by side (a few
+// layers of at most a few dozen rows: a thread per point took 19 rows of 6..15
+// columns one after the other). Returns false when some value lies within its
+// error of the edge of the tie band, where FP64 rounding would decide.
+__device__ bool fold64_point(const NetView& net, const QueryView& Q, Fold64& F, unsigned long long t, int lane,
+                             double* m) {
+    const int L = net.L, offL = net.noff[L], s = Q.s, D = Q.cnt->D;
+    const bool cov = Q.flip != nullptr;
+    __syncwarp();
+    if (lane < kSetW) F.ch[lane] = F.ti[lane] = 0u;
+    {
+        int d[kMaxS];
+        decode_digits(t, s, Q.R, d);
+        for (int p = 0; p < s; ++p)
+            if (lane == p) F.x[p] = (double)Q.dv[p * Q.R + d[p]] / 255.0;
+    }
+    bool edge = false;
+    int cb = 0;
+    double y = 0.0, ey = 0.0;
+    for (int l = 1; l <= L; ++l) {
+        const int nl = l < L ? Q.fst[2 + l] : net.dims[L], K = s + cb;
+        int nch = 0, nti = 0;
+        __syncwarp();  // the sources of the layers below are written
+        for (int i0 = 0; i0 < nl; i0 += 32) {
+            const int i = i0 + lane;
+            bool ch = false, ti = false;
+            if (i < nl) {
+                const int nn = l < L ? Q.fnode[cb + i] : offL + out_of_row(i, D);
+                const double* row = Q.fco + (size_t)nn * Q.fstride;
+                const double ub = Q.ub[nn], e = Q.fe64[l < L ? cb + i : kFoldMax + i];
+                double a = 0.0;
+#pragma unroll 4
+                for (int k = 0; k < K; ++k) a = fma(row[k], F.x[k], a);
+                const double u = ub + a;
+                const bool base_tie = fabs(ub) < kTau;  // every evaluation of this neuron is a sign tie
+                ti = fabs(u) < kTau || base_tie;
+                ch = !ti && ((u >= 0.0) != (ub >= 0.0));
+                edge = edge || (cov && !base_tie && fabs(fabs(u) - kTau) <= 2.0 * e);
+                if (l < L) {
+                    F.x[K + i] = fmax(u, 0.0) - fmax(ub, 0.0);
+                } else {
+                    y = u;
+                    ey = e;
+                }
+                const int at = l < L ? cb + i : kFoldMax + i;
+                if (ch) atomicOr(&F.ch[at >> 5], 1u << (at & 31));
+                if (ti) atomicOr(&F.ti[at >> 5], 1u << (at & 31));
+            }
+            nch += __popc(__ballot_sync(0xffffffffu, ch));
+            nti += __popc(__ballot_sync(0xffffffffu, ti));
+        }
+        if (lane == 0) {
+            F.nch[l] = nch;
+            F.nti[l] = nti;
+        }
+        if (l < L) cb += nl;
+    }
+    const int HL = net.dims[L];
+    const double yD = __shfl_sync(0xffffffffu, y, 0);
+    const double mx = warp_max(lane > 0 && lane < HL ? y : -DBL_MAX);
+    const double em = warp_max(lane < HL ? ey : 0.0);
+    *m = Q.prop == PROP_THRESHOLD ? fmax(yD - Q.V, Q.V - mx) : yD - mx;
+    if (fabs(fabs(*m) - kTau) <= 4.0 * em + 0x1p-51 * (fabs(yD) + fabs(mx) + fabs(Q.V))) edge = true;
+    __syncwarp();
+    return !__any_sync(0xffffffffu, edge);
+}
+
+// Points k_fold left undecided.
+__global__ void __launch_bounds__(32 * F64W) k_fold64(NetView net, const QueryView* __restrict__ qs,
+                                                      const QEntry* __restrict__ in,
+                                                      const unsigned long long* __restrict__ count,
+                                                      unsigned long long cap, Queue out, int out_level) {
+    __shared__ Fold64 Fs[F64W];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    Fold64& F = Fs[warp];
     unsigned long long n = *count;
     if (n > cap) n = cap;
-    const int L = net.L, offL = net.noff[L];
-    for (unsigned long long e = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-         e += (unsigned long long)gridDim.x * blockDim.x) {
+    const int L = net.L, offL = net.noff[L], HL = net.dims[L];
+    for (unsigned long long e = (unsigned long long)blockIdx.x * F64W + warp; e < n;
+         e += (unsigned long long)gridDim.x * F64W) {
         const QEntry en = in[e];
         const QueryView& Q = qs[en.q];
         if (!folded(Q)) continue;  // queued by another first pass
-        const int s = Q.s;
-        double x[kMaxS + kFoldMax], ex[kMaxS + kFoldMax];
-        unsigned char ch[kFoldMax + kFoldOut];
-        int nch[kMaxL + 1];
-        int d[kMaxS];
-        decode_digits(en.t, s, Q.R, d);
-        for (int p = 0; p < s; ++p) {
-            x[p] = (double)Q.dv[p * Q.R + d[p]] / 255.0;
-            ex[p] = 0x1p-53 * fabs(x[p]);
-        }
-        bool unc = false, unsafe = false, safe = true;
-        bool da = false, db = false, oa = false, ob = true;
-        double yD = 0.0, eD = 0.0;
         const int D = Q.cnt->D;
-        int cb = 0;
-        for (int l = 1; l <= L; ++l) {
-            const int nl = l < L ? Q.fst[2 + l] : net.dims[L], K = s + cb;
-            nch[l] = 0;
-            for (int i = 0; i < nl; ++i) {
-                const int nn = l < L ? Q.fnode[cb + i] : offL + out_of_row(i, D);
-                const double* row = Q.fco + (size_t)nn * Q.fstride;
-                double a = 0.0, M = 0.0, pr = 0.0;
-                for (int k = 0; k < K; ++k) {
-                    const double w = row[k];
-                    a = fma(w, x[k], a);
-                    M += fabs(w * x[k]);
-                    pr += fabs(w) * ex[k];
-                }
-                const double ub = Q.ub[nn], u = ub + a;
-                const double er = (Q.fer[nn] + (K + 4) * 0x1p-53 * M + pr + Q.eub[nn] +
-                                   0x1p-52 * (fabs(ub) + fabs(u))) * (1.0 + 1e-9);
-                const bool cert = fabs(u) > er + 2.0 * kTau && fabs(ub) >= kTau;
-                const bool c = cert && ((u >= 0.0) != (ub >= 0.0));
-                if (!cert && Q.flip) unc = true;  // signs matter only for coverage
-                nch[l] += c;
-                if (l < L) {
-                    ch[cb + i] = c;
-                    x[K + i] = fmax(u, 0.0) - fmax(ub, 0.0);
-                    ex[K + i] = er + 0x1p-52 * (fabs(ub) + fabs(u));
-                } else {
-                    ch[kFoldMax + i] = c;
-                    if (i == 0) {
-                        yD = u;
-                        eD = er;
-                    }
-                    if (Q.prop == PROP_THRESHOLD) {
-                        const double eb = er + 2.0 * kTau + 0x1p-52 * (fabs(u) + fabs(Q.V));
-                        const int sd = u - Q.V > eb ? 1 : (Q.V - u > eb ? -1 : 0);
-                        if (i == 0) { da = sd > 0; db = sd < 0; }
-                        else { oa = oa || sd > 0; ob = ob && sd < 0; }
-                    } else if (i > 0) {
-                        const double diff = yD - u, eb = eD + er + 2.0 * kTau + 0x1p-52 * (fabs(yD) + fabs(u));
-                        if (diff < -eb) unsafe = true;
-                        else if (!(diff > eb)) safe = false;
-                    }
-                }
+        double m;
+        if (!fold64_point(net, Q, F, en.t, lane, &m)) {
+            if (lane == 0) {
+                queue_push(out, en.t, en.q, Q.cnt, out_level);
+                work_done(Q.cnt, 1);
             }
-            if (l < L) cb += nl;
+            continue;
         }
-        if (Q.prop == PROP_THRESHOLD) {
-            const int vv = thr_verdict(da, db, oa, ob);
-            unsafe = vv == 1;
-            safe = vv == 0;
+        if (lane == 0) {
+            if (fabs(m) < kTau) {
+                const unsigned long long k = atomicAdd(&Q.cnt->n_ties, 1ull);
+                if (k < Q.ties_cap) Q.ties[k] = en.t;
+                else atomicOr(&Q.cnt->err, DERR_TIES);
+            } else if (m < 0.0) {
+                record_adversarial(Q, en.t);
+            }
         }
-        if (unc || (!unsafe && !safe)) {
-            queue_push(out, en.t, en.q, Q.cnt, out_level);
-        } else {
-            if (unsafe) record_adversarial(Q, en.t);
-            if (Q.flip) {
-                int c0 = 0;
-                for (int l = 1; l <= L; ++l) {
-                    const int nl = l < L ? Q.fst[2 + l] : net.dims[L];
-                    int only = -1;
-                    for (int i = 0; i < nl; ++i) {
-                        if (!ch[l < L ? c0 + i : kFoldMax + i]) continue;
-                        only = i;
-                        set_bit_once(Q.flip, (unsigned long long)(l < L ? Q.fnode[c0 + i]
-                                                                        : offL + out_of_row(i, D)));
-                    }
-                    if (l < L && nch[l] == 1) {  // SS needs exactly one change in layer l
-                        const int j = Q.fnode[c0 + only] - net.noff[l], Hn = net.dims[l + 1];
-                        const int nx = l + 1 < L ? Q.fst[3 + l] : net.dims[L];
-                        for (int i = 0; i < nx; ++i) {
-                            if (!ch[l + 1 < L ? c0 + nl + i : kFoldMax + i]) continue;
-                            const int o = l + 1 < L ? Q.fnode[c0 + nl + i] - net.noff[l + 1] : out_of_row(i, D);
-                            set_bit_once(Q.ss, (unsigned long long)net.ssoff[l] + (unsigned long long)j * Hn + o);
+        if (Q.flip) {
+            auto in_set = [](const uint32_t* w, int at) { return (w[at >> 5] >> (at & 31)) & 1u; };
+            int c0 = 0;
+            for (int l = 1; l <= L; ++l) {
+                const int nl = l < L ? Q.fst[2 + l] : HL, b0 = l < L ? c0 : kFoldMax;
+                const int b1 = l + 1 < L ? c0 + nl : kFoldMax;  // first row of the layer above
+                const int nx = l + 1 < L ? Q.fst[3 + l] : HL;
+                const int nch = F.nch[l], nti = F.nti[l];
+                auto neuron = [&](int ll, int at, int i) { return ll < L ? Q.fnode[at + i] : offL + out_of_row(i, D); };
+                for (int i = lane; i < nl; i += 32) {
+                    const unsigned long long nn = (unsigned long long)neuron(l, b0, i);
+                    if (in_set(F.ch, b0 + i)) set_bit_once(Q.flip, nn);
+                    if (in_set(F.ti, b0 + i)) set_bit_once(Q.flip_tie, nn);
+                }
+                // SS pairs with layer l + 1: certain with one change and no tie in layer l;
+                // under ties, the one change or (with none) each tie may be the only change
+                if (l < L && (nti == 0 ? nch == 1 : nch <= 1)) {
+                    for (int j = 0; j < nl; ++j) {
+                        if (!in_set(nch == 1 ? F.ch : F.ti, b0 + j)) continue;
+                        const unsigned long long r0 = (unsigned long long)net.ssoff[l] +
+                            (unsigned long long)(Q.fnode[b0 + j] - net.noff[l]) * net.dims[l + 1];
+                        for (int i = lane; i < nx; i += 32) {
+                            const unsigned long long bit = r0 + (neuron(l + 1, b1, i) - net.noff[l + 1]);
+                            if (nti == 0 && in_set(F.ch, b1 + i)) set_bit_once(Q.ss, bit);
+                            else if (in_set(F.ch, b1 + i) || in_set(F.ti, b1 + i)) set_bit_once(Q.ss_tie, bit);
                         }
                     }
-                    if (l < L) c0 += nl;
                 }
+                if (l < L) c0 += nl;
             }
         }
-        work_done(Q.cnt, 1);  // time to verdict: this point is resolved (its push, if any, came first)
+        __syncwarp();
+        if (lane == 0) work_done(Q.cnt, 1);  // time to verdict: this point is resolved
     }
+}
+
+// FP64 margin of one point of query 0, where it folded (k_margin64 otherwise).
+__global__ void __launch_bounds__(32) k_fold_margin(NetView net, const QueryView* __restrict__ qs,
+                                                    unsigned long long t, double* out) {
+    __shared__ Fold64 F;
+    if (!folded(qs[0])) return;
+    double m;
+    fold64_point(net, qs[0], F, t, threadIdx.x, &m);
+    if (threadIdx.x == 0) *out = m;
 }
 
 }  // namespace
@@ -595,7 +657,12 @@ void launch_fold(const NetView& net, const QueryView* d_qs, int nq, const unsign
 
 void launch_fold64(const NetView& net, const QueryView* d_qs, const QEntry* in, const unsigned long long* count,
                    unsigned long long cap, Queue out, int out_level, int n_sm, cudaStream_t st) {
-    k_fold64<<<(unsigned)n_sm, 128, 0, st>>>(net, d_qs, in, count, cap, out, out_level);
+    k_fold64<<<(unsigned)n_sm * 4, 32 * F64W, 0, st>>>(net, d_qs, in, count, cap, out, out_level);
+}
+
+void launch_fold_margin(const NetView& net, const QueryView* d_qs, unsigned long long t, double* d_out,
+                        cudaStream_t st) {
+    k_fold_margin<<<1, 32, 0, st>>>(net, d_qs, t, d_out);
 }
 
 }  // namespace vbmc

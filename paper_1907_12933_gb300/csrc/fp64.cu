@@ -184,6 +184,7 @@ k_margin64(NetView net, const QueryView* __restrict__ qs, unsigned long long t, 
     double* h = u + net.total;
     __shared__ int dstep[kMaxS];
     const QueryView& Q = qs[0];
+    if (folded(Q)) return;  // launch_fold_margin wrote it
     const int L = net.L;
     if (threadIdx.x == 0) {
         int d[kMaxS];
@@ -226,6 +227,9 @@ k_margin64(NetView net, const QueryView* __restrict__ qs, unsigned long long t, 
 
 void launch_margin64(const NetView& net, const QueryView* d_qs, unsigned long long t, double* d_out,
                      cudaStream_t st) {
+    // one CTA walks the whole net (239 us on 784-512-512-10); a folded query's margin
+    // comes from its folded rows, one warp (about 10 us)
+    if (fold_supported(net)) launch_fold_margin(net, d_qs, t, d_out, st);
     const size_t smem = sizeof(double) * (net.total + net.hmax);
     cudaFuncSetAttribute(k_margin64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_margin64<<<1, T64, smem, st>>>(net, d_qs, t, d_out);

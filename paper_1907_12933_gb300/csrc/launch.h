@@ -27,6 +27,9 @@ void launch_fold(const NetView& net, const QueryView* d_qs, int nq, const unsign
                  int out_level, int n_sm, cudaStream_t st);
 void launch_fold64(const NetView& net, const QueryView* d_qs, const QEntry* in, const unsigned long long* count,
                    unsigned long long cap, Queue out, int out_level, int n_sm, cudaStream_t st);
+// FP64 margin of point t of query 0 into *d_out where it folded (nothing otherwise).
+void launch_fold_margin(const NetView& net, const QueryView* d_qs, unsigned long long t, double* d_out,
+                        cudaStream_t st);
 
 // Shape class of the FP32 SIMT screen for a net (0: unsupported).
 int simt_variant(const NetView& net);

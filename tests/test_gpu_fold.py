@@ -152,3 +152,23 @@ def test_fp32_bound_holds_far_from_the_tie_band(vb):
         np.testing.assert_array_equal(a[key], b[key], err_msg=key)
     assert a["summary"]["n_adversarial"] == b["summary"]["n_adversarial"]
     vnet.free()
+
+
+def test_tie_band_points_are_settled_on_the_folded_net(vb):
+    """A hidden neuron whose potential is exactly 0 at some points of the box, and two
+    outputs equal at every point: sign ties, SS pairs under ties and margin ties as the
+    oracle has them, without the FP64 pass on the whole net."""
+    net = synth.make_net(818, [12, 24, 20, 4], "relu", 2.0, "zero")
+    q = synth.make_query(818, 2, 12, 2, 12)
+    p0, p1 = (int(p) for p in q["pixels"])
+    q["image"][p0], q["image"][p1] = 100, 103
+    net["W"][0][5] = 0.0  # u = (x_p0 - x_p1) / 2: 0 where the steps differ by 3
+    net["W"][0][5, p0], net["W"][0][5, p1] = 0.5, -0.5
+    for same_outputs in (False, True):
+        if same_outputs:
+            D = oracle.eval_point(net, q, 0)["D"]
+            net["W"][2][(D + 1) % 4] = net["W"][2][D]
+        o = oracle.verify(net, q)
+        assert o["flip_tie"].any() and o["ss_tie"].any() and (o["n_ties"] > 0) == same_outputs
+        g = run_gpu(vb, net, q, "fp32")
+        compare(g, o, net, q)
