@@ -366,6 +366,7 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
         A(&q.fco, T * (size_t)q.fstride);
         A(&q.fbd, T);
         A(&q.fer, T);
+        A(&q.fhe, T);
         A(&q.fx, (size_t)kMaxS);
         A(&q.fcls, T);
         A(&q.fst, (size_t)kFoldSt);

@@ -134,17 +134,19 @@ struct QueryView {
     // whose sign cannot change in it is carried as the linear map it is.
     int fold;               // 1: the call may use it (the set-up then builds it)
     int fstride;            // row stride of fco: column p < s is pixel p, s + m is node m
-    double* fco;            // [total][fstride]: du_n = sum of these times the sources' changes
-    double* fbd;            // [total] bound on |du_n| over the box
-    double* fer;            // [total] bound on the error of du_n from rounded fco entries
-    double* fx;             // [kMaxS] max over the digits of |dv_p| / 255
+    float2* fco;            // [total][fstride]: du_n = sum of these (FP32 pairs, hi + lo) times the
+                            //   sources' changes
+    float* fbd;             // [total] bound on |du_n| over the box
+    float* fer;             // [total] bound on the error of du_n from rounded fco entries
+    float2* fhe;            // [total] upper bounds of (|hb_n|, eub_n)
+    float* fx;              // [kMaxS] max over the digits of |dv_p| / 255 (rounded up)
     unsigned char* fcls;    // [total] hidden neurons: 0 pos, 1 neg, 2 node (sign can change)
     int* fst;               // [kFoldSt]: [0] 1: folded, [1] 1: more than kFoldMax nodes,
                             //   [2 + l] nodes of hidden layer l
     int* fnode;             // [kFoldMax] node -> neuron (concatenated index)
     float4* fc32;           // packed FP32 coefficients, see FoldLayout
     float4* fk32;           // [kFoldMax + kFoldOut] node (ub, c1, c2, thr); output (ub, e, em, thr)
-    double* fe64;           // [kFoldMax + kFoldOut] error bound of a node's or output's FP64 evaluation
+    float* fe64;            // [kFoldMax + kFoldOut] error bound of a node's or output's FP64 evaluation
     float* fxs;             // [s][R] fl(dv / 255)
     Counters* cnt;
     uint32_t* bitmap;       // verdict bits (nullptr: off)

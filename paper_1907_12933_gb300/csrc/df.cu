@@ -13,6 +13,7 @@
 // clears the bound by 2 tau; if anything is left undecided the whole point
 // goes on to the FP64 pass and contributes nothing here.
 #include "dev.cuh"
+#include "dfloat.cuh"
 #include "launch.h"
 
 #include <cfloat>
@@ -326,24 +327,6 @@ k_df64(NetView net, const QueryView* __restrict__ qs, int nq, const QEntry* __re
 // Potentials within the tie band 2 tau (tau = 1e-9) of 0 are left to the
 // FP64 pass as before; these bounds are about 1e-12 relative, far inside it.
 
-__device__ __forceinline__ float2 two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return make_float2(s, e);
-}
-
-__device__ __forceinline__ float2 df_add(float2 a, float2 b) {
-    const float2 s = two_sum(a.x, b.x);
-    return two_sum(s.x, __fadd_rn(s.y, __fadd_rn(a.y, b.y)));
-}
-
-// an FP64 value as a pair: |v - (hi + lo)| <= 2^-48 |v|
-__device__ __forceinline__ float2 split64(double v) {
-    const float hi = (float)v;
-    return make_float2(hi, (float)(v - (double)hi));
-}
-
 // M block-wide sums of non-negative terms, rounded up (upper bounds); every
 // thread gets the totals. red holds (blockDim.x / 32) x M floats.
 template <int M>
@@ -376,8 +359,6 @@ __device__ __forceinline__ int df_split(int Nn, int K) {
     const int ks = TDF / Nn;
     return ks < 32 ? ks : 32;
 }
-
-__device__ __forceinline__ float abs_up(float2 a) { return __fmul_ru(fabsf(a.x), 1.f + 0x1p-22f); }
 
 template <int PB>
 __global__ void __launch_bounds__(TDF)

@@ -11,8 +11,8 @@
 // evaluating: every other neuron's sign is known to be the unperturbed image's at
 // every point, so it adds neither a sign change nor a sign tie (Sec. III-B).
 //
-//   k_pro_layer (prologue.cu)  rows A, C in FP64, layer by layer, from the rows of
-//                 the layer below; B_n >= |du_n| over the box; the class
+//   k_pro_layer (prologue.cu)  rows A, C as FP32 pairs, layer by layer, from the rows
+//                 of the layer below; B_n >= |du_n| over the box; the class
 //                 ("pos"/"neg" when |ub_n| > B_n, its error and the tie band)
 //   k_fold_pack   per query: the rows of nodes and outputs as FP32 in groups of 4,
 //                 their error bounds; D and the margin of the unperturbed image
@@ -25,7 +25,7 @@
 //
 // Error of k_fold, constant per node (u = 2^-24, K sources, M_n = sum_k |c_nk| bound
 // of source k): the FMA chain and the roundings of c and x give at most
-// (K + 4) u M_n, the sources' own errors sum |C_nm| e_m, the FP64 rows fer_n, the
+// (K + 4) u M_n, the sources' own errors sum |C_nm| e_m, the rows' fer_n, the
 // base potential |fl(ub) - ub| + eub, its addition u (|ub| + B_n). Their sum e_n
 // bounds both |u_n - exact| and, since the ReLU is 1-Lipschitz, |dh_n - exact|.
 // A sign is certain when |u_n| > e_n + 2 tau, a margin when it exceeds e_D + e_o + 2 tau.
@@ -38,6 +38,7 @@
 // points near the boundary) 28.7 -> 1.5 ms; 784-1024x3-10, s = 4, k = 15 with coverage
 // 191 -> 4.3 ms; 784-300-100-10, s = 5, k = 9 in an L2 ball 27.7 -> 0.52 ms.
 #include "dev.cuh"
+#include "dfloat.cuh"
 #include "launch.h"
 
 #include <cfloat>
@@ -76,9 +77,15 @@ __device__ void fold_shape(const NetView& net, const QueryView& Q, FoldShape& f)
 // Output held by row i of the output layer: D first, then the others in order.
 __device__ __forceinline__ int out_of_row(int i, int D) { return i == 0 ? D : (i <= D ? i - 1 : i); }
 
+__device__ __forceinline__ double warp_max(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
 __global__ void __launch_bounds__(256) k_fold_pack(NetView net, QueryView* qs, unsigned long long* unfolded) {
     __shared__ FoldShape f;
-    __shared__ double eh[kFoldMax], eo[kFoldOut], eh64[kFoldMax];
+    __shared__ float eh[kFoldMax], eh64[kFoldMax], eo[kFoldOut];
     __shared__ int D_s;
     QueryView& Q = qs[blockIdx.x];
     if (!Q.fold || Q.fst[1] || (Q.cnt->err & DERR_PIXELS)) {
@@ -86,70 +93,83 @@ __global__ void __launch_bounds__(256) k_fold_pack(NetView net, QueryView* qs, u
         return;
     }
     const int L = net.L, HL = net.dims[L], offL = net.noff[L], s = Q.s;
-    if (threadIdx.x == 0) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp == 0) {  // D: the largest output, the lowest index among equals; HL <= 32
+        const double y = lane < HL ? Q.ub[offL + lane] : -DBL_MAX;
+        const double top = warp_max(y);
+        const int D = __ffs(__ballot_sync(0xffffffffu, lane < HL && y == top)) - 1;
+        const double mx = warp_max(lane == D ? -DBL_MAX : y);
+        if (lane == 0) {
+            D_s = D;
+            Q.cnt->D = D;
+            Q.cnt->base_margin = Q.prop == PROP_THRESHOLD ? fmax(top - Q.V, Q.V - mx) : top - mx;
+        }
+    } else if (threadIdx.x == 32) {
         fold_shape(net, Q, f);
-        const double* y = Q.ub + offL;
-        int D = 0;
-        for (int i = 1; i < HL; ++i)
-            if (y[i] > y[D]) D = i;
-        double mx = -DBL_MAX;
-        for (int i = 0; i < HL; ++i)
-            if (i != D && y[i] > mx) mx = y[i];
-        D_s = D;
-        Q.cnt->D = D;
-        Q.cnt->base_margin = Q.prop == PROP_THRESHOLD ? fmax(y[D] - Q.V, Q.V - mx) : y[D] - mx;
     }
     __syncthreads();
     const int D = D_s;
     auto neuron = [&](int l, int i) { return l < L ? Q.fnode[f.cb[l] + i] : offL + out_of_row(i, D); };
-    for (int l = 1; l <= L; ++l) {
-        const int src = s + f.cb[l], n = f.n[l];
-        for (int e = threadIdx.x; e < ((n + 3) >> 2) * src; e += blockDim.x) {
-            const int g = e / src, k = e - g * src;
-            float c[4];
+    for (int e = threadIdx.x; e < f.entries; e += blockDim.x) {
+        int l = L;
+        while (e < f.off[l]) --l;  // layers without rows have the offset of the next one
+        const int src = s + f.cb[l], n = f.n[l], g = (e - f.off[l]) / src, k = e - f.off[l] - g * src;
+        float c[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
-                c[r] = 4 * g + r < n ? (float)Q.fco[(size_t)neuron(l, 4 * g + r) * Q.fstride + k] : 0.f;
-            Q.fc32[f.off[l] + e] = make_float4(c[0], c[1], c[2], c[3]);
-        }
+        for (int r = 0; r < 4; ++r)
+            c[r] = 4 * g + r < n ? Q.fco[(size_t)neuron(l, 4 * g + r) * Q.fstride + k].x : 0.f;
+        Q.fc32[e] = make_float4(c[0], c[1], c[2], c[3]);
     }
+    // error bounds (FP32, rounded up), layer by layer: a warp per row, its lanes over the sources
+    const float tau2 = __double2float_ru(2.0 * kTau);
     for (int l = 1; l <= L; ++l) {
         const int cb = f.cb[l];
-        for (int i = threadIdx.x; i < f.n[l]; i += blockDim.x) {
+        for (int i = warp; i < f.n[l]; i += blockDim.x / 32) {
             const int nn = neuron(l, i);
-            const double* row = Q.fco + (size_t)nn * Q.fstride;
-            double M = 0.0, pr = 0.0, pr64 = 0.0;
-            for (int p = 0; p < s; ++p) M += fabs(row[p]) * Q.fx[p];
-            for (int m = 0; m < cb; ++m) {
-                const double w = fabs(row[s + m]);
-                M += w * (Q.fbd[Q.fnode[m]] + eh[m]);
-                pr += w * eh[m];
-                pr64 += w * eh64[m];
+            const float2* row = Q.fco + (size_t)nn * Q.fstride;
+            float M = 0.f, pr = 0.f, pr64 = 0.f;
+            for (int k = lane; k < s + cb; k += 32) {
+                const float w = abs_up(row[k]);
+                if (k < s) {
+                    M = __fmaf_ru(w, Q.fx[k], M);
+                } else {
+                    M = __fmaf_ru(w, __fadd_ru(Q.fbd[Q.fnode[k - s]], eh[k - s]), M);
+                    pr = __fmaf_ru(w, eh[k - s], pr);
+                    pr64 = __fmaf_ru(w, eh64[k - s], pr64);
+                }
             }
-            const double ub = Q.ub[nn], B = Q.fbd[nn];
-            const float ub32 = (float)ub;
-            const double ed = (s + cb + 4) * 0x1p-24 * 1.00001 * M + pr + Q.fer[nn] + 1e-37;
-            const double e = (ed + fabs((double)ub32 - ub) + Q.eub[nn] + 0x1p-24 * 1.001 * (fabs(ub) + B + ed)) *
-                             (1.0 + 1e-9);
-            // the same in FP64 (u = 2^-53; x_p = dv_p / 255 rounds once)
-            const double e64 = ((s + cb + 5) * 0x1p-53 * M + pr64 + Q.fer[nn] + Q.eub[nn] +
-                                0x1p-51 * (fabs(ub) + B)) * (1.0 + 1e-9);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                M = __fadd_ru(M, __shfl_xor_sync(0xffffffffu, M, o));
+                pr = __fadd_ru(pr, __shfl_xor_sync(0xffffffffu, pr, o));
+                pr64 = __fadd_ru(pr64, __shfl_xor_sync(0xffffffffu, pr64, o));
+            }
+            if (lane) continue;
+            const double ub = Q.ub[nn];
+            const float ub32 = (float)ub, B = Q.fbd[nn], fer = Q.fer[nn], eub = Q.fhe[nn].y;
+            const float mag = __fadd_ru(__fadd_ru(fabsf(ub32), B), 1e-30f);
+            const float ed = __fadd_ru(__fmaf_ru((float)(s + cb + 5) * 0x1p-24f, M, pr), __fadd_ru(fer, 1e-37f));
+            float e = __fadd_ru(__fadd_ru(ed, __double2float_ru(fabs((double)ub32 - ub))), eub);
+            e = __fmaf_ru(0x1.01p-24f, __fadd_ru(mag, ed), e);
+            // the same in FP64 (u = 2^-53; x_p = dv_p / 255 rounds once, the rows' pairs are exact in it)
+            const float e64 = __fmaf_ru(0x1p-51f, mag, __fadd_ru(__fmaf_ru((float)(s + cb + 6) * 0x1p-53f, M, pr64),
+                                                                 __fadd_ru(fer, eub)));
             Q.fe64[l < L ? cb + i : kFoldMax + i] = e64;
-            const float e2 = __double2float_ru(e + 2.0 * kTau);
+            const float e2 = __fadd_ru(e, tau2);
             const float thr = fabs(ub) < kTau ? INFINITY : e2;  // a base tie: every sign is a tie
             if (l < L) {
                 eh[cb + i] = e;
                 eh64[cb + i] = e64;
                 Q.fk32[cb + i] = make_float4(ub32, ub >= 0.0 ? 0.f : ub32, ub >= 0.0 ? -ub32 : 0.f, thr);
             } else {
-                eo[i] = e + 0x1p-23 * 1.001 * (fabs(ub) + B);
+                eo[i] = __fmaf_ru(0x1.01p-23f, mag, e);
                 Q.fk32[kFoldMax + i] = make_float4(ub32, e2, 0.f, thr);
             }
         }
         __syncthreads();
     }
     for (int i = threadIdx.x; i < HL; i += blockDim.x)
-        Q.fk32[kFoldMax + i].z = __double2float_ru((eo[0] + eo[i] + 2.0 * kTau) * (1.0 + 1e-9));
+        Q.fk32[kFoldMax + i].z = __fadd_ru(__fadd_ru(eo[0], eo[i]), tau2);
     if (threadIdx.x == 0) {
         Q.fst[0] = 1;
         Q.cnt->folded = 1;
@@ -467,12 +487,6 @@ struct Fold64 {
     int nch[kMaxL + 1], nti[kMaxL + 1];  // how many of each, per layer
 };
 
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
 // Point t of query Q by the definitions (Eq. 10 / Eq. 11 margin *m; signs and sign
 // ties when coverage is on). A lane holds a row of a layer: its chain of FMAs over
 // the sources is as long as the row, and a layer's rows run side by side (a few
@@ -503,11 +517,14 @@ __device__ bool fold64_point(const NetView& net, const QueryView& Q, Fold64& F, 
             bool ch = false, ti = false;
             if (i < nl) {
                 const int nn = l < L ? Q.fnode[cb + i] : offL + out_of_row(i, D);
-                const double* row = Q.fco + (size_t)nn * Q.fstride;
-                const double ub = Q.ub[nn], e = Q.fe64[l < L ? cb + i : kFoldMax + i];
+                const float2* row = Q.fco + (size_t)nn * Q.fstride;
+                const double ub = Q.ub[nn], e = (double)Q.fe64[l < L ? cb + i : kFoldMax + i];
                 double a = 0.0;
 #pragma unroll 4
-                for (int k = 0; k < K; ++k) a = fma(row[k], F.x[k], a);
+                for (int k = 0; k < K; ++k) {
+                    const float2 c = row[k];
+                    a = fma((double)c.x + (double)c.y, F.x[k], a);
+                }
                 const double u = ub + a;
                 const bool base_tie = fabs(ub) < kTau;  // every evaluation of this neuron is a sign tie
                 ti = fabs(u) < kTau || base_tie;

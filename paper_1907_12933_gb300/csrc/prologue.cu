@@ -11,6 +11,7 @@
 //  * k_pro_finish: class D and margin of the unperturbed image, and the
 //                  per-neuron constants of the screens' error bounds
 #include "dev.cuh"
+#include "dfloat.cuh"
 #include "launch.h"
 
 #include <cfloat>
@@ -20,30 +21,30 @@ namespace vbmc {
 __global__ void k_pro_init(NetView net, QueryView* qs, int nq) {
     QueryView& Q = qs[blockIdx.x];
     const int H0 = net.dims[0];
-    if (threadIdx.x == 0 && blockIdx.y == 0) {
-        bool ok = Q.s >= 0 && Q.s <= kMaxS;
-        for (int p = 0; p < Q.s && ok; ++p) {
-            int v = Q.pix_in[p];
-            ok = v >= 0 && v < H0;
-            for (int r = 0; r < p && ok; ++r) ok = Q.pix_in[r] != v;
-        }
-        Counters* c = Q.cnt;
-        c->n_adv = 0;
-        c->first = ~0ull;
-        c->n_ties = 0;
-        c->n_q[0] = c->n_q[1] = c->n_q[2] = c->n_q[3] = 0;
-        c->n_points = Q.filter ? 0ull : Q.hi - Q.lo;  // with a filter the passes count
-        c->err = ok ? 0u : DERR_PIXELS;
-        c->D = 0;
-        c->base_margin = 0.0;
-        c->t0 = globaltimer_ns();
-        c->t_final = 0;
-        c->work = Q.ntiles;
-        c->folded = 0;
-        if (Q.fst) Q.fst[0] = Q.fst[1] = 0;
-        for (int p = 0; p < Q.s; ++p) {
-            int v = Q.pix_in[p];
-            Q.pix[p] = (ok && v >= 0 && v < H0) ? v : 0;  // never index out of range
+    if (blockIdx.y == 0 && threadIdx.x < 32) {
+        const int p = threadIdx.x;
+        const bool own = Q.s >= 0 && Q.s <= kMaxS && p < Q.s;
+        const int v = own ? Q.pix_in[p] : -1 - p;
+        const unsigned same = __match_any_sync(0xffffffffu, v);
+        // in range, and in no other lane
+        const bool bad = own && (v < 0 || v >= H0 || __popc(same) > 1);
+        const bool ok = Q.s >= 0 && Q.s <= kMaxS && !__any_sync(0xffffffffu, bad);
+        if (own) Q.pix[p] = (ok && v >= 0 && v < H0) ? v : 0;  // never index out of range
+        if (p == 0) {
+            Counters* c = Q.cnt;
+            c->n_adv = 0;
+            c->first = ~0ull;
+            c->n_ties = 0;
+            c->n_q[0] = c->n_q[1] = c->n_q[2] = c->n_q[3] = 0;
+            c->n_points = Q.filter ? 0ull : Q.hi - Q.lo;  // with a filter the passes count
+            c->err = ok ? 0u : DERR_PIXELS;
+            c->D = 0;
+            c->base_margin = 0.0;
+            c->t0 = globaltimer_ns();
+            c->t_final = 0;
+            c->work = Q.ntiles;
+            c->folded = 0;
+            if (Q.fst) Q.fst[0] = Q.fst[1] = 0;
         }
     }
     // results start from zero on every call
@@ -70,7 +71,7 @@ __global__ void k_pro_init(NetView net, QueryView* qs, int nq) {
     }
     if (Q.fold && threadIdx.x < Q.s) {  // the largest change of each pixel (steps -k and k, clipped)
         const int v = Q.image[Q.pix[threadIdx.x]];
-        Q.fx[threadIdx.x] = (double)max(min(Q.k, 255 - v), min(Q.k, v)) / 255.0;
+        Q.fx[threadIdx.x] = __fdiv_ru((float)max(min(Q.k, 255 - v), min(Q.k, v)), 255.f);
     }
 }
 
@@ -80,24 +81,51 @@ __device__ __forceinline__ double act64(int act, double u) {
     return u;
 }
 
-// One warp per neuron i of layer l; lanes stride over the inputs. Also bounds
-// the FP64 error of the result: rounding of the K products and sums,
-// (K + 2) 2^-53 (sum_j |w_j h_j| + |b|), plus the input errors propagated,
-// sum_j |w_j| e_j (the activations are 1-Lipschitz).
+// v / 255 of every grey level, FP64.
+struct Grey {
+    double v[256];
+    constexpr Grey() : v() {
+        for (int i = 0; i < 256; ++i) v[i] = (double)i / 255.0;
+    }
+};
+__device__ constexpr Grey kGrey;
+
+// Neuron i of layer l, WPN warps each; their lanes stride over the inputs. Also
+// bounds the FP64 error of the result, in FP32 rounded up: a term passes at most
+// c = K / lanes + 16 roundings (its lane's chain, the sums over lanes and warps, the
+// bias; x / 255 on layer 1), so c 2^-53 (sum_j |w_j h_j| + |b|), plus the input errors
+// propagated, sum_j |w_j| e_j (the activations are 1-Lipschitz).
 //
-// With Q.fold the warp also writes its neuron's row of the folded net (fold.cu):
+// With Q.fold the warps also write their neuron's row of the folded net (fold.cu):
 // du_i as a linear form in the s pixel changes and the output changes of the
 // nodes of earlier layers, the row of W_l times the rows of the layer below
 // ("pos" inputs), W_l itself in the columns of that layer's nodes; the bound
 // B_i on |du_i| over the box; and the class that follows from it. Each block
 // lists the layer below's "pos" neurons and nodes once, in order. A row's
-// columns lie across the lanes; fewer than 32 of them split the inputs too.
+// columns lie across a warp's lanes; fewer than 32 of them split the inputs too.
+//
+// Bound by load latency at the start, by FP64 after it: that pipe takes 16 cycles a
+// warp instruction, so only the base product runs on it (2 instructions a term); rows
+// are FP32 pairs (dfloat.cuh: 10 FP32 instructions against 32 cycles), bounds FP32.
+// Few queries leave most of the chip idle with one warp per neuron (an output layer
+// of 10 is 10 warps, each walking 512 inputs one load latency after the other), so
+// wide layers take eight; with many queries the warps come from them. The set-up of
+// one query (init, layers, pack, and the launches that return at once), before (a
+// warp per neuron, FP64 throughout) and after: 784-512-512-10 142 -> 70 us,
+// 784-1024x3-10 310 -> 147 us.
+template <int WPN>
 __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, int nq, int l) {
+    constexpr int NPB = 8 / WPN;  // neurons per block
     __shared__ short plist[kMaxWidth], clist[kFoldMax];
     __shared__ int wpos[8], wnode[8];
+    __shared__ float2 part[8][32];
+    __shared__ double pdot[8];
+    __shared__ float psum[8][4];
     const QueryView& Q = qs[blockIdx.y];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * (blockDim.x >> 5) + warp;
+    const int wn = warp % WPN;  // warp of its neuron
+    const int i = blockIdx.x * NPB + warp / WPN;
+    const int tn = 32 * wn + lane, step = 32 * WPN;
     const int K = net.dims[l - 1], N = net.dims[l];
     const int offp = l >= 2 ? net.noff[l - 1] : 0;
     const bool fold = Q.fold != 0;
@@ -123,6 +151,7 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
         for (int m = 1; m < l - 1; ++m) nb += Q.fst[2 + m];
         __syncthreads();
         int bp = 0, bn = 0;
+#pragma unroll
         for (int w = 0; w < 8; ++w) {
             if (w < warp) {
                 bp += wpos[w];
@@ -153,102 +182,155 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
         }
         __syncthreads();
     }
-    if (i >= N) return;
+    if (WPN == 1 && i >= N) return;  // (WPN == 8: one neuron per block, the grid has N)
     const float* Wr = net.W[l] + (size_t)i * K;
-    double acc = 0.0, mag = 0.0, prop = 0.0;
+    double dot = 0.0;
+    float b[4] = {0.f, 0.f, 0.f, 0.f};  // sum |w h|, sum |w| e; of the carried rows: sum |w| fer, sum |w| B
     if (l == 1) {
-        for (int j = lane; j < K; j += 32) {
-            const double p = (double)Wr[j] * ((double)Q.image[j] / 255.0);
-            acc += p;
-            mag += fabs(p);
+#pragma unroll 4
+        for (int j = tn; j < K; j += step) {
+            const float w = Wr[j];
+            const int v = Q.image[j];
+            dot = fma((double)w, kGrey.v[v], dot);
+            b[0] = __fmaf_ru(fabsf(w), (float)v, b[0]);
         }
+        b[0] = __fdiv_ru(b[0], 255.f);
     } else {
-        const double* h = Q.hb + net.noff[l - 1];
-        const double* eh = Q.eub + net.noff[l - 1];
-        for (int j = lane; j < K; j += 32) {
-            const double p = (double)Wr[j] * h[j];
-            acc += p;
-            mag += fabs(p);
-            prop += fabs((double)Wr[j]) * eh[j];
+        const double* h = Q.hb + offp;
+        const double* eh = Q.eub + offp;
+        if (fold) {
+            const float2* he = Q.fhe + offp;
+#pragma unroll 4
+            for (int j = tn; j < K; j += step) {
+                const float w = Wr[j];
+                const float2 m = he[j];
+                dot = fma((double)w, h[j], dot);
+                b[0] = __fmaf_ru(fabsf(w), m.x, b[0]);
+                b[1] = __fmaf_ru(fabsf(w), m.y, b[1]);
+            }
+            if (rows) {
+#pragma unroll 2
+                for (int jj = tn; jj < npos; jj += step) {
+                    const int j = plist[jj];
+                    const float w = fabsf(Wr[j]);
+                    b[2] = __fmaf_ru(w, Q.fer[offp + j], b[2]);
+                    b[3] = __fmaf_ru(w, Q.fbd[offp + j], b[3]);
+                }
+            }
+        } else {
+#pragma unroll 4
+            for (int j = tn; j < K; j += step) {
+                const float w = Wr[j];
+                dot = fma((double)w, h[j], dot);
+                b[0] = __fmaf_ru(fabsf(w), __double2float_ru(fabs(h[j])), b[0]);
+                b[1] = __fmaf_ru(fabsf(w), __double2float_ru(eh[j]), b[1]);
+            }
         }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        mag += __shfl_xor_sync(0xffffffffu, mag, o);
-        prop += __shfl_xor_sync(0xffffffffu, prop, o);
+        dot += __shfl_xor_sync(0xffffffffu, dot, o);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) b[m] = __fadd_ru(b[m], __shfl_xor_sync(0xffffffffu, b[m], o));
+    }
+    if (WPN > 1) {
+        if (lane == 0) {
+            pdot[warp] = dot;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) psum[warp][m] = b[m];
+        }
+        __syncthreads();
+        dot = 0.0;
+        b[0] = b[1] = b[2] = b[3] = 0.f;
+#pragma unroll
+        for (int w = 0; w < WPN; ++w) {
+            dot += pdot[w];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) b[m] = __fadd_ru(b[m], psum[w][m]);
+        }
     }
     const int n = net.noff[l] + i;
-    const double bi = (double)net.b[l][i];
-    const double u = acc + bi;
-    // (x/255 carries one more rounding on layer 1; activations add 2^-50 |u|)
-    const double eu = ((K + 4) * 0x1p-53 * (mag + fabs(bi)) + prop + 0x1p-50 * fabs(u)) * (1.0 + 1e-9);
-    if (lane == 0) {
+    const float bias = net.b[l][i];
+    const double u = dot + (double)bias;
+    // (activations add 2^-50 |u|)
+    float eu = __fmul_ru((float)((K + step - 1) / step + 17) * 0x1p-53f, __fadd_ru(b[0], fabsf(bias)));
+    eu = __fmaf_ru(0x1p-50f, __double2float_ru(fabs(u)), __fadd_ru(eu, b[1]));
+    eu = __fmul_ru(eu, 1.f + 0x1p-20f);
+    if (tn == 0) {
+        const double h = (l < net.L) ? act64(net.act, u) : u;
         Q.ub[n] = u;
-        Q.hb[n] = (l < net.L) ? act64(net.act, u) : u;
-        Q.eub[n] = eu;
+        Q.hb[n] = h;
+        Q.eub[n] = (double)eu;
+        if (fold) Q.fhe[n] = make_float2(__double2float_ru(fabs(h)), eu);
     }
     if (!rows) return;
     const int s = Q.s;
-    double* row = Q.fco + (size_t)n * Q.fstride;
-    double B = 0.0, er = 0.0;  // sum of |coefficient| x bound of its source; error of the carried rows
+    float2* row = Q.fco + (size_t)n * Q.fstride;
+    float B = 0.f;  // sum of |coefficient| x bound of its source (over lanes of the first warp)
+    // the rows of the layer below carry errors fer; a pair sum over npos inputs, split
+    // over lanes and warps, adds at most (npos + 32) 2^-45 sum_j |w_j| B_j
+    const float er = l == 1 ? 0.f : __fmaf_ru((float)(npos + 32) * 0x1p-45f, b[3], b[2]);
     if (l == 1) {
-        if (lane < s) {
-            const double w = (double)Wr[Q.pix[lane]];
-            row[lane] = w;
-            B = fabs(w) * Q.fx[lane];
+        if (wn == 0 && lane < s) {
+            const float w = Wr[Q.pix[lane]];
+            row[lane] = make_float2(w, 0.f);
+            B = __fmul_ru(fabsf(w), Q.fx[lane]);
         }
     } else {
-        // the rows of the layer below carry errors fer, and each sum over npos inputs
-        // rounds by at most (npos + 4) 2^-53 sum_j |w_j| B_j
-        double e1 = 0.0, m1 = 0.0;
-        for (int jj = lane; jj < npos; jj += 32) {
-            const int j = plist[jj];
-            const double w = fabs((double)Wr[j]);
-            e1 += w * Q.fer[offp + j];
-            m1 += w * Q.fbd[offp + j];
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            e1 += __shfl_xor_sync(0xffffffffu, e1, o);
-            m1 += __shfl_xor_sync(0xffffffffu, m1, o);
-        }
-        er = (e1 + (npos + 4) * 0x1p-53 * m1) * (1.0 + 1e-9);
         const int S = s + nb;
-        const double* prev = Q.fco + (size_t)offp * Q.fstride;
+        const float2* prev = Q.fco + (size_t)offp * Q.fstride;
         for (int k0 = 0; k0 < S; k0 += 32) {
             int sp = 1;  // lanes per input: a power of two that holds the columns left
             while (sp < 32 && sp < S - k0) sp <<= 1;
-            const int k = k0 + (lane & (sp - 1)), g = lane / sp, G = 32 / sp;
-            double a = 0.0;
+            const int per = 32 / sp;
+            const int k = k0 + (lane & (sp - 1)), g = wn * per + lane / sp, G = WPN * per;
+            float2 a = make_float2(0.f, 0.f);
             if (k < S) {
 #pragma unroll 8
                 for (int jj = g; jj < npos; jj += G) {
                     const int j = plist[jj];
-                    a = fma((double)Wr[j], prev[(size_t)j * Q.fstride + k], a);
+                    const float w = Wr[j];
+                    const float2 h = prev[(size_t)j * Q.fstride + k];
+                    const float pr = __fmul_rn(w, h.x);
+                    float ep = __fmaf_rn(w, h.x, -pr);
+                    ep = __fmaf_rn(w, h.y, ep);
+                    const float2 t = two_sum(a.x, pr);
+                    a = make_float2(t.x, __fadd_rn(a.y, __fadd_rn(t.y, ep)));
                 }
+                a = two_sum(a.x, a.y);
             }
-            for (int o = sp; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if (g == 0 && k < S) {
-                row[k] = a;
-                B += fabs(a) * (k < s ? Q.fx[k] : Q.fbd[Q.fnode[k - s]]);
-            }
-        }
-        for (int c = lane; c < nnode; c += 32) {
-            const double w = (double)Wr[clist[c]];
-            row[S + c] = w;
-            B += fabs(w) * Q.fbd[offp + clist[c]];
-        }
-    }
+            for (int o = sp; o < 32; o <<= 1)
+                a = df_add(a, make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o)));
+            if (WPN > 1) {
+                __syncthreads();
+                part[warp][lane] = a;
+                __syncthreads();
+                a = part[0][lane];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) B += __shfl_xor_sync(0xffffffffu, B, o);
+                for (int w = 1; w < WPN; ++w) a = df_add(a, part[w][lane]);
+            }
+            if (wn == 0 && lane < sp && k < S) {
+                row[k] = a;
+                B = __fmaf_ru(abs_up(a), k < s ? Q.fx[k] : Q.fbd[Q.fnode[k - s]], B);
+            }
+        }
+        if (wn == 0)
+            for (int c = lane; c < nnode; c += 32) {
+                const float w = Wr[clist[c]];
+                row[S + c] = make_float2(w, 0.f);
+                B = __fmaf_ru(fabsf(w), Q.fbd[offp + clist[c]], B);
+            }
+    }
+    if (wn != 0) return;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) B = __fadd_ru(B, __shfl_xor_sync(0xffffffffu, B, o));
     if (lane == 0) {
-        B = B * (1.0 + 1e-9) + er;
+        B = __fadd_ru(B, er);
         Q.fbd[n] = B;
         Q.fer[n] = er;
         // a neuron keeps its sign, clear of the tie band, over the whole box
         if (l < net.L) {
-            const bool keeps = fabs(u) > (B + eu) * (1.0 + 1e-6) + 4.0 * kTau;
+            const bool keeps = fabs(u) > ((double)B + (double)eu) * (1.0 + 1e-6) + 4.0 * kTau;
             Q.fcls[n] = keeps ? (u >= 0.0 ? 0 : 1) : 2;
         }
     }
@@ -330,12 +412,10 @@ __global__ void k_pro_finish(NetView net, QueryView* qs, int nq) {
             double e1 = 0.0;
             if (l == 1) {
                 double b1 = 0.0;
-                for (int p = 0; p < s; ++p) {
-                    double mx = 0.0;
-                    for (int d = 0; d < Q.R; ++d)
-                        mx = fmax(mx, fabs((double)Q.tab[((size_t)p * Q.R + d) * H + i]));
-                    b1 += mx;
-                }
+                // dv_p grows with the digit, so |tab| is largest at one of the ends
+                for (int p = 0; p < s; ++p)
+                    b1 += fmax(fabs((double)Q.tab[(size_t)p * Q.R * H + i]),
+                               fabs((double)Q.tab[((size_t)p * Q.R + Q.R - 1) * H + i]));
                 e1 = gam * b1 * (1.0 + 1e-12);
             }
             const bool base_tie = fabs(ub) < kTau;
@@ -403,7 +483,12 @@ void launch_pro_init(const NetView& net, QueryView* d_qs, int nq, cudaStream_t s
 }
 
 void launch_pro_layer(const NetView& net, QueryView* d_qs, int nq, int l, cudaStream_t st) {
-    k_pro_layer<<<dim3((net.dims[l] + 7) / 8, nq), 256, 0, st>>>(net, d_qs, nq, l);
+    // eight warps per neuron for at least 256 inputs (one round of their lanes), until
+    // the queries alone put about 16 warps on every SM
+    if (net.dims[l - 1] >= 256 && (long long)nq * net.dims[l] <= 2432)
+        k_pro_layer<8><<<dim3(net.dims[l], nq), 256, 0, st>>>(net, d_qs, nq, l);
+    else
+        k_pro_layer<1><<<dim3((net.dims[l] + 7) / 8, nq), 256, 0, st>>>(net, d_qs, nq, l);
 }
 
 void launch_prologue(const NetView& net, QueryView* d_qs, int nq, int max_sr, cudaStream_t st,

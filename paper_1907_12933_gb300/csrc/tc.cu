@@ -1137,12 +1137,9 @@ __global__ void k_classes_tc(const __grid_constant__ TcParams P, NetView net, Qu
     __syncthreads();
     for (int j = threadIdx.x; j < H1; j += blockDim.x) {
         double b1 = 0.0;
-        for (int p = 0; p < Q.s; ++p) {
-            double mx = 0.0;
-            for (int d = 0; d < Q.R; ++d)
-                mx = fmax(mx, fabs((double)Q.tab[((size_t)p * Q.R + d) * H1 + j]));
-            b1 += mx;
-        }
+        for (int p = 0; p < Q.s; ++p)  // largest at one of the ends: dv_p grows with the digit
+            b1 += fmax(fabs((double)Q.tab[(size_t)p * Q.R * H1 + j]),
+                       fabs((double)Q.tab[((size_t)p * Q.R + Q.R - 1) * H1 + j]));
         b1 *= 1.0 + 1e-6;
         const double ub = Q.ub[j];
         const bool cross = !(fabs(ub) > (b1 + (double)Q.thr[j]) * (1.0 + 1e-6) + 4.0 * kTau);
