@@ -367,12 +367,14 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
         A(&q.fbd, T);
         A(&q.fer, T);
         A(&q.fhe, T);
+        A(&q.fsb, T);
         A(&q.fx, (size_t)kMaxS);
         A(&q.fcls, T);
         A(&q.fst, (size_t)kFoldSt);
         A(&q.fnode, (size_t)kFoldMax);
         A(&q.fc32, fold_coeff_entries(v, S));
-        A(&q.fk32, (size_t)kFoldMax + kFoldOut);
+        A(&q.fk32, (size_t)1 + kFoldOut);
+        A(&q.forow, (size_t)kFoldOut);
         A(&q.fe64, (size_t)kFoldMax + kFoldOut);
         A(&q.fxs, (size_t)S * RM);
     }

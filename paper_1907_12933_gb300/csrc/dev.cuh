@@ -140,12 +140,14 @@ struct QueryView {
     float* fer;             // [total] bound on the error of du_n from rounded fco entries
     float2* fhe;            // [total] upper bounds of (|hb_n|, eub_n)
     float* fx;              // [kMaxS] max over the digits of |dv_p| / 255 (rounded up)
-    unsigned char* fcls;    // [total] hidden neurons: 0 pos, 1 neg, 2 node (sign can change)
+    float* fsb;             // [total] bound on a node's source (0 at the unperturbed image)
+    unsigned char* fcls;    // [total] hidden neurons: 0 pos, 1 neg, 2 / 3 node (sign can change; ub < 0 / >= 0)
     int* fst;               // [kFoldSt]: [0] 1: folded, [1] 1: more than kFoldMax nodes,
-                            //   [2 + l] nodes of hidden layer l
+                            //   [2 + l] rows of layer l: its nodes, the output layer's rows
     int* fnode;             // [kFoldMax] node -> neuron (concatenated index)
     float4* fc32;           // packed FP32 coefficients, see FoldLayout
-    float4* fk32;           // [kFoldMax + kFoldOut] node (ub, c1, c2, thr); output (ub, e, em, thr)
+    float4* fk32;           // [1 + kFoldOut]: (margin bound, sign bound, -, -); per output (-, e, -, -)
+    int* forow;             // [kFoldOut] rows behind the margins: output, + 256 with a sign test
     float* fe64;            // [kFoldMax + kFoldOut] error bound of a node's or output's FP64 evaluation
     float* fxs;             // [s][R] fl(dv / 255)
     Counters* cnt;

@@ -21,7 +21,7 @@ size_t fold_coeff_entries(const NetView& net, int max_s);  // float4 entries of 
 void launch_fold_pack(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long* d_unfolded);
 // Tiles of mt points, numbered as in the general first pass (d_tile_prefix; null
 // with one query); work_units: the queries' work counts are in these tiles;
-// claim: tile counter (null: static tiles).
+// claim: tile counter (many queries).
 void launch_fold(const NetView& net, const QueryView* d_qs, int nq, const unsigned long long* d_tile_prefix,
                  unsigned long long n_tiles, int mt, bool work_units, unsigned long long* claim, Queue out,
                  int out_level, int n_sm, cudaStream_t st);

@@ -97,10 +97,11 @@ __device__ constexpr Grey kGrey;
 // propagated, sum_j |w_j| e_j (the activations are 1-Lipschitz).
 //
 // With Q.fold the warps also write their neuron's row of the folded net (fold.cu):
-// du_i as a linear form in the s pixel changes and the output changes of the
-// nodes of earlier layers, the row of W_l times the rows of the layer below
-// ("pos" inputs), W_l itself in the columns of that layer's nodes; the bound
-// B_i on |du_i| over the box; and the class that follows from it. Each block
+// du_i as a linear form in the s pixel changes and the sources of the nodes of
+// earlier layers, the row of W_l times the rows of the layer below ("pos" inputs and
+// nodes with ub >= 0, whose linear part is carried too), W_l itself in the columns of
+// that layer's nodes; the bound B_i on |du_i| over the box; and the class that
+// follows from it. Each block
 // lists the layer below's "pos" neurons and nodes once, in order. A row's
 // columns lie across a warp's lanes; fewer than 32 of them split the inputs too.
 //
@@ -139,8 +140,8 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
         for (int e = 0; e < kMaxWidth / 256; ++e) {
             const int j = warp * (kMaxWidth / 8) + 32 * e + lane;
             const int c = j < K ? cls[j] : 1;
-            mp[e] = __ballot_sync(0xffffffffu, c == 0);
-            mn[e] = __ballot_sync(0xffffffffu, c == 2);
+            mp[e] = __ballot_sync(0xffffffffu, c == 0 || c == 3);
+            mn[e] = __ballot_sync(0xffffffffu, c >= 2);
             cp += __popc(mp[e]);
             cn += __popc(mn[e]);
         }
@@ -311,14 +312,14 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
             }
             if (wn == 0 && lane < sp && k < S) {
                 row[k] = a;
-                B = __fmaf_ru(abs_up(a), k < s ? Q.fx[k] : Q.fbd[Q.fnode[k - s]], B);
+                B = __fmaf_ru(abs_up(a), k < s ? Q.fx[k] : Q.fsb[Q.fnode[k - s]], B);
             }
         }
         if (wn == 0)
             for (int c = lane; c < nnode; c += 32) {
                 const float w = Wr[clist[c]];
                 row[S + c] = make_float2(w, 0.f);
-                B = __fmaf_ru(fabsf(w), Q.fbd[offp + clist[c]], B);
+                B = __fmaf_ru(fabsf(w), Q.fsb[offp + clist[c]], B);
             }
     }
     if (wn != 0) return;
@@ -331,7 +332,9 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
         // a neuron keeps its sign, clear of the tie band, over the whole box
         if (l < net.L) {
             const bool keeps = fabs(u) > ((double)B + (double)eu) * (1.0 + 1e-6) + 4.0 * kTau;
-            Q.fcls[n] = keeps ? (u >= 0.0 ? 0 : 1) : 2;
+            Q.fcls[n] = keeps ? (u >= 0.0 ? 0 : 1) : (u >= 0.0 ? 3 : 2);
+            // a node's source is at most as far as its potential can cross 0
+            Q.fsb[n] = fmaxf(0.f, __fadd_ru(__fsub_ru(B, __double2float_rd(fabs(u))), eu));
         }
     }
 }

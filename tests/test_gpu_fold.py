@@ -172,3 +172,15 @@ def test_tie_band_points_are_settled_on_the_folded_net(vb):
         assert o["flip_tie"].any() and o["ss_tie"].any() and (o["n_ties"] > 0) == same_outputs
         g = run_gpu(vb, net, q, "fp32")
         compare(g, o, net, q)
+
+
+@pytest.mark.parametrize("s,k,lo,hi", [(0, 5, 0, 0), (1, 0, 0, 0), (1, 1, 0, 0), (2, 63, 1, 16000),
+                                       (5, 3, 33, 34), (5, 3, 31, 16801), (3, 2, 0, 125), (11, 1, 5, 177001)])
+def test_units_of_the_last_digit(vb, s, k, lo, hi):
+    """Ranges whose ends fall anywhere in the 4-digit pieces of the last pixel's digit, a
+    single point, one digit value, and more pixels than a box usually has."""
+    net = synth.make_net(819, [30, 64, 64, 6], "relu", 2.0, "normal")
+    q = synth.make_query(819, 5, 30, s, k)
+    n = oracle.space_size(s, k)
+    hi = min(hi, n)
+    compare(run_gpu(vb, net, q, "bf16", lo=lo, hi=hi), oracle.verify(net, q, lo=lo, hi=hi), net, q)
