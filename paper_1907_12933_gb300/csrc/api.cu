@@ -64,6 +64,38 @@ cudaError_t dalloc(T** p, size_t n, std::vector<void*>& owned) {
 
 }  // namespace
 
+// Neurons in at least one SS-covered pair (Eq. 3) of a mask in the layout of
+// QueryView::ss, one flag per neuron. Pair (j, i) of layers l, l + 1 is bit
+// ssoff[l] + j H_{l+1} + i: row by row, 32 bits at a time (bit by bit this took
+// 0.2 ms on 784-512-512-10 and 1.4 ms on 784-1024x3-10; now 8 and 50 us).
+namespace vbmc {
+void ss_covered(const NetView& v, const uint32_t* ss, std::vector<char>& cov) {
+    cov.assign((size_t)v.total, 0);
+    std::vector<uint32_t> col;
+    for (int l = 1; l < v.L; ++l) {
+        const int Hl = v.dims[l], Hn = v.dims[l + 1], nw = (Hn + 31) / 32;
+        col.assign((size_t)nw, 0u);
+        for (int j = 0; j < Hl; ++j) {
+            const unsigned long long b0 = (unsigned long long)v.ssoff[l] + (unsigned long long)j * Hn;
+            uint32_t any = 0u;
+            for (int c = 0; c < nw; ++c) {
+                const unsigned long long b = b0 + 32ull * c;
+                const int left = Hn - 32 * c, sh = (int)(b & 31);  // bits of this piece
+                const size_t w = (size_t)(b >> 5);
+                uint32_t x = ss[w] >> sh;
+                if (sh && sh + (left < 32 ? left : 32) > 32) x |= ss[w + 1] << (32 - sh);
+                if (left < 32) x &= (1u << left) - 1u;
+                col[c] |= x;
+                any |= x;
+            }
+            if (any) cov[v.noff[l] + j] = 1;
+        }
+        for (int i = 0; i < Hn; ++i)
+            if ((col[i >> 5] >> (i & 31)) & 1u) cov[v.noff[l + 1] + i] = 1;
+    }
+}
+}  // namespace vbmc
+
 struct vbmc_net {
     NetView v{};
     std::vector<void*> owned;
@@ -128,6 +160,12 @@ struct vbmc_result {
     bool have_tw = false;
     unsigned long long* d_claim = nullptr;  // tile claim counters: the general first pass, the folded net's
     unsigned long long* h_claim = nullptr;  // pinned copy after the call
+    // one block on each side and one copy per call: the view, the tile prefix, pixels and
+    // image on their way in; the counters and the claims on their way out (not for members
+    // of a batch, whose views and counters lie in the arena)
+    uint8_t* h_in = nullptr;
+    uint8_t* d_in = nullptr;
+    uint32_t* h_masks = nullptr;  // pinned: the coverage masks on their way out
     unsigned long long ntiles = 0;          // first-pass tiles of the last call
     int tile_pts = 0;                       // points per first-pass tile (0: no claim counter)
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_pro = nullptr, ev_scr = nullptr;
@@ -297,6 +335,13 @@ extern "C" vbmc_status vbmc_mask_words(const vbmc_net* net, size_t* fw, size_t* 
 
 namespace {
 
+// Byte offsets in a result's input block.
+constexpr size_t kInTp = (sizeof(QueryView) + 15) & ~size_t(15);
+constexpr size_t kInPix = kInTp + 2 * sizeof(unsigned long long);
+constexpr size_t kInImage = kInPix + sizeof(int) * kMaxS;
+
+size_t mask_bytes(const NetView& v) { return 8 * ((size_t)v.flip_words + (size_t)v.ss_words); }
+
 vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena* arena, int slot,
                           vbmc_result** out) {
     if (!net || !caps || !out) return fail(VBMC_ERR_ARG, "null argument");
@@ -322,12 +367,23 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
     if (arena) {
         r->d_q = arena->d_qs + slot;
         r->d_cnt = arena->d_cnt + slot;
+        A(&r->d_image, (size_t)v.dims[0]);
+        A(&r->d_pix_in, (size_t)S);
+        A(&r->d_tp, 2);
+        A(&r->d_claim, 2);
     } else {
-        A(&r->d_q, 1);
-        A(&r->d_cnt, 1);
+        A(&r->d_in, kInImage + (size_t)v.dims[0]);
+        uint8_t* out = nullptr;
+        A(&out, sizeof(Counters) + 2 * sizeof(unsigned long long));
+        if (e == cudaSuccess) {
+            r->d_q = reinterpret_cast<QueryView*>(r->d_in);
+            r->d_tp = reinterpret_cast<unsigned long long*>(r->d_in + kInTp);
+            r->d_pix_in = reinterpret_cast<int*>(r->d_in + kInPix);
+            r->d_image = r->d_in + kInImage;
+            r->d_cnt = reinterpret_cast<Counters*>(out);
+            r->d_claim = reinterpret_cast<unsigned long long*>(out + sizeof(Counters));
+        }
     }
-    A(&r->d_image, (size_t)v.dims[0]);
-    A(&r->d_pix_in, (size_t)S);
     A(&q.pix, (size_t)S);
     A(&q.dv, (size_t)S * RM);
     A(&q.ub, T);
@@ -342,12 +398,11 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
     A(&q.kvec, (size_t)kMaxL + 1);
     A(&q.cpos, (size_t)(kMaxL + 1) * 32);
     A(&q.cneg, (size_t)(kMaxL + 1) * 32);
-    A(&q.flip, (size_t)v.flip_words);
-    A(&q.flip_tie, (size_t)v.flip_words);
-    A(&q.ss, (size_t)v.ss_words);
-    A(&q.ss_tie, (size_t)v.ss_words);
+    A(&q.flip, 2 * ((size_t)v.flip_words + v.ss_words));  // the four masks in one block: one copy out
+    q.flip_tie = q.flip + v.flip_words;
+    q.ss = q.flip_tie + v.flip_words;
+    q.ss_tie = q.ss + v.ss_words;
     A(&q.ties, (size_t)std::max<uint32_t>(1, caps->ties_cap));
-    A(&r->d_tp, 2);
     A(&r->d_qcount, 4);
     A(&r->d_margin, 1);
     if (caps->max_points) A(&q.bitmap, (size_t)((caps->max_points + 31) / 32));
@@ -357,7 +412,6 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
     r->caps.queue_cap = qc;
     for (int i = 0; i < 4; ++i) A(&r->d_queue[i], (size_t)qc);
     A(&r->d_tiles, (size_t)VBMC_MAX_TILES);
-    A(&r->d_claim, 2);
     // compacted columns of the fused tensor screen (calls with one query)
     const bool tcnet = tc_supported(v, VBMC_PREC_BF16) || tc_supported(v, VBMC_PREC_FP16);
     const bool fused = !arena && tcnet;
@@ -387,8 +441,12 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
         A(&q.w1c, (size_t)kMaxS * v.dims[1]);
         for (int l = 2; l <= v.L; ++l) A(&q.wtc[l], (size_t)v.dims[l - 1] * v.dims[l]);
     }
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&r->h_cnt, sizeof(Counters));
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&r->h_claim, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&r->h_cnt, sizeof(Counters) + 2 * sizeof(unsigned long long));
+    r->h_claim = reinterpret_cast<unsigned long long*>(r->h_cnt + 1);
+    if (!arena) {
+        if (e == cudaSuccess) e = cudaMallocHost((void**)&r->h_in, kInImage + (size_t)v.dims[0]);
+        if (e == cudaSuccess) e = cudaMallocHost((void**)&r->h_masks, mask_bytes(v));
+    }
     if (e == cudaSuccess) e = cudaEventCreate(&r->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&r->ev1);
     if (e == cudaSuccess) e = cudaEventCreate(&r->ev_pro);
@@ -498,7 +556,10 @@ extern "C" vbmc_status vbmc_result_free(vbmc_result* r) {
     tc_query_work_free(r->tw);
     arena_release(r->arena);
     if (r->h_cnt) cudaFreeHost(r->h_cnt);
-    if (r->h_claim) cudaFreeHost(r->h_claim);
+    if (r->h_in) {  // not a member of a batch
+        cudaFreeHost(r->h_in);
+        if (r->h_masks) cudaFreeHost(r->h_masks);
+    }
     if (r->ev0) cudaEventDestroy(r->ev0);
     if (r->ev1) cudaEventDestroy(r->ev1);
     if (r->ev_pro) cudaEventDestroy(r->ev_pro);
@@ -757,16 +818,33 @@ vbmc_status enqueue(vbmc_net* net, vbmc_result* r, const uint8_t* d_image, const
                         (opt.precision == VBMC_PREC_FP32 && !small_supported(net->v));
     r->ntiles = tp[1];
     r->tile_pts = claims ? (tensor16 ? tc_tile_points() : simt_tile_points(net->v)) : 0;
-    VB_CUDA(cudaMemcpyAsync(r->d_q, &q, sizeof(QueryView), cudaMemcpyHostToDevice, st));
-    VB_CUDA(cudaMemcpyAsync(r->d_tp, tp.data(), sizeof(unsigned long long) * 2, cudaMemcpyHostToDevice, st));
+    if (r->h_in) {
+        // the result's last call has finished, so the pinned block is free to rewrite;
+        // an image already staged behind the view goes with it
+        std::memcpy(r->h_in, &q, sizeof(QueryView));
+        std::memcpy(r->h_in + kInTp, tp.data(), sizeof(unsigned long long) * 2);
+        const size_t bytes = d_image == r->d_image ? kInImage + (size_t)net->v.dims[0] : kInPix;
+        VB_CUDA(cudaMemcpyAsync(r->d_in, r->h_in, bytes, cudaMemcpyHostToDevice, st));
+    } else {
+        VB_CUDA(cudaMemcpyAsync(r->d_q, &q, sizeof(QueryView), cudaMemcpyHostToDevice, st));
+        VB_CUDA(cudaMemcpyAsync(r->d_tp, tp.data(), sizeof(unsigned long long) * 2, cudaMemcpyHostToDevice, st));
+    }
     const cudaEvent_t ev[7] = {r->ev0, r->ev_pro, r->ev_scr, r->ev1, r->ev_split, r->ev_f32, r->ev_df};
     vbmc_status sst = enqueue_passes(net, r->d_q, &q, 1, r->d_tp, tp[1], r->d_qcount, r->d_queue,
                                      std::max<uint64_t>(1, r->caps.queue_cap), ev, opt, st, false, STAGE_ALL,
                                      &r->ww, r->have_tw ? &r->tw : nullptr, claims ? r->d_claim : nullptr);
-    if (sst != VBMC_OK) return sst;
-    VB_CUDA(cudaMemcpyAsync(r->h_cnt, r->d_cnt, sizeof(Counters), cudaMemcpyDeviceToHost, st));
-    if (claims)
-        VB_CUDA(cudaMemcpyAsync(r->h_claim, r->d_claim, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+    if (sst != VBMC_OK) {
+        if (r->h_in) cudaStreamSynchronize(st);  // the pinned block has been read
+        return sst;
+    }
+    if (r->h_in) {
+        VB_CUDA(cudaMemcpyAsync(r->h_cnt, r->d_cnt, sizeof(Counters) + sizeof(unsigned long long),
+                                cudaMemcpyDeviceToHost, st));
+    } else {
+        VB_CUDA(cudaMemcpyAsync(r->h_cnt, r->d_cnt, sizeof(Counters), cudaMemcpyDeviceToHost, st));
+        if (claims)
+            VB_CUDA(cudaMemcpyAsync(r->h_claim, r->d_claim, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+    }
     r->last_stream = st;
     r->pending = true;
     r->have_result = true;
@@ -887,13 +965,18 @@ vbmc_status verify_query(vbmc_net* net, const vbmc_query* q, const vbmc_options*
             if (q->pixels[r] == q->pixels[p]) return fail(VBMC_ERR_ARG, "duplicate pixel index");
     }
     cudaStream_t stq = (cudaStream_t)stream;
-    VB_CUDA(cudaMemcpyAsync(res->d_image, q->image, H0, cudaMemcpyHostToDevice, stq));
-    if (q->s > 0)
-        VB_CUDA(cudaMemcpyAsync(res->d_pix_in, q->pixels, sizeof(int32_t) * q->s,
-                                cudaMemcpyHostToDevice, stq));
     QueryExtra x;
     st = query_extra(*q, &x);
     if (st != VBMC_OK) return st;
+    if (res->h_in) {  // goes in with the view (enqueue)
+        std::memcpy(res->h_in + kInImage, q->image, (size_t)H0);
+        if (q->s > 0) std::memcpy(res->h_in + kInPix, q->pixels, sizeof(int32_t) * (size_t)q->s);
+    } else {
+        VB_CUDA(cudaMemcpyAsync(res->d_image, q->image, H0, cudaMemcpyHostToDevice, stq));
+        if (q->s > 0)
+            VB_CUDA(cudaMemcpyAsync(res->d_pix_in, q->pixels, sizeof(int32_t) * q->s,
+                                    cudaMemcpyHostToDevice, stq));
+    }
     st = enqueue(net, res, res->d_image, res->d_pix_in, q->s, q->k, q->lo, h, n, *opt, stq, x, fold);
     if (st != VBMC_OK) return st;
     res->image.assign(q->image, q->image + H0);
@@ -972,31 +1055,21 @@ extern "C" vbmc_status vbmc_get_coverage(vbmc_result* res, uint32_t* flip, size_
         return fail(VBMC_ERR_ARG, "flip buffer too small");
     if ((ss || ss_tie || covered_fraction) && ss && ss_words < (size_t)v.ss_words)
         return fail(VBMC_ERR_ARG, "ss buffer too small");
-    if (flip) VB_CUDA(cudaMemcpy(flip, res->hq.flip, 4ull * v.flip_words, cudaMemcpyDeviceToHost));
-    if (flip_tie)
-        VB_CUDA(cudaMemcpy(flip_tie, res->hq.flip_tie, 4ull * v.flip_words, cudaMemcpyDeviceToHost));
-    std::vector<uint32_t> tmp;
-    uint32_t* ssh = ss;
-    if (!ssh && covered_fraction) {
-        tmp.resize(v.ss_words);
-        ssh = tmp.data();
-    }
-    if (ssh) VB_CUDA(cudaMemcpy(ssh, res->hq.ss, 4ull * v.ss_words, cudaMemcpyDeviceToHost));
-    if (ss_tie) VB_CUDA(cudaMemcpy(ss_tie, res->hq.ss_tie, 4ull * v.ss_words, cudaMemcpyDeviceToHost));
+    // the four masks lie in one block (flip, flip_tie, ss, ss_tie): one copy as far as asked for
+    const size_t fw = (size_t)v.flip_words, sw = (size_t)v.ss_words;
+    const bool want_ss = ss || covered_fraction;
+    const size_t words = ss_tie ? 2 * (fw + sw) : want_ss ? 2 * fw + sw : flip_tie ? 2 * fw : flip ? fw : 0;
+    std::vector<uint32_t> own(res->h_masks ? 0 : words);  // a batch member's: no pinned block each
+    uint32_t* const h = res->h_masks ? res->h_masks : own.data();
+    if (words) VB_CUDA(cudaMemcpy(h, res->hq.flip, 4 * words, cudaMemcpyDeviceToHost));
+    if (flip) std::memcpy(flip, h, 4 * fw);
+    if (flip_tie) std::memcpy(flip_tie, h + fw, 4 * fw);
+    if (ss) std::memcpy(ss, h + 2 * fw, 4 * sw);
+    if (ss_tie) std::memcpy(ss_tie, h + 2 * fw + sw, 4 * sw);
     if (covered_fraction) {
         // Eq. 3: neurons in at least one SS-covered pair over all non-input neurons.
-        std::vector<char> cov(v.total, 0);
-        for (int l = 1; l < v.L; ++l) {
-            const int Hl = v.dims[l], Hn = v.dims[l + 1];
-            for (int j = 0; j < Hl; ++j)
-                for (int i = 0; i < Hn; ++i) {
-                    const unsigned long long b = v.ssoff[l] + (unsigned long long)j * Hn + i;
-                    if ((ssh[b >> 5] >> (b & 31)) & 1u) {
-                        cov[v.noff[l] + j] = 1;
-                        cov[v.noff[l + 1] + i] = 1;
-                    }
-                }
-        }
+        std::vector<char> cov;
+        ss_covered(v, h + 2 * fw, cov);
         int c = 0;
         for (char x : cov) c += x;
         *covered_fraction = (double)c / (double)v.total;

@@ -22,6 +22,7 @@
 namespace vbmc {
 const NetView* net_view(const vbmc_net* net);
 vbmc_status set_error(vbmc_status st, const char* msg);
+void ss_covered(const NetView& v, const uint32_t* ss, std::vector<char>& cov);
 }  // namespace vbmc
 
 using namespace vbmc;
@@ -295,22 +296,19 @@ extern "C" vbmc_status vbmc_covered_fraction(const vbmc_net* net, int32_t layout
         return set_error(VBMC_ERR_ARG, "layout must be VBMC_LAYOUT_PAIRS or VBMC_LAYOUT_LAYER");
     const NetView& v = *net_view(net);
     std::vector<char> cov((size_t)v.total, 0);
-    auto bit = [&](unsigned long long b) { return (mask[b >> 5] >> (b & 31)) & 1u; };
-    for (int l = 1; l < v.L; ++l) {
-        const int Hl = v.dims[l], Hn = v.dims[l + 1], off = v.noff[l], on = v.noff[l + 1];
-        if (layout == VBMC_LAYOUT_PAIRS) {
-            for (int j = 0; j < Hl; ++j)
-                for (int i = 0; i < Hn; ++i)
-                    if (bit((unsigned long long)v.ssoff[l] + (unsigned long long)j * Hn + i)) {
-                        cov[off + j] = 1;
-                        cov[on + i] = 1;
-                    }
-        } else {
+    if (layout == VBMC_LAYOUT_PAIRS) {
+        ss_covered(v, mask, cov);
+    } else {
+        auto bit = [&](unsigned long long b) { return (mask[b >> 5] >> (b & 31)) & 1u; };
+        for (int l = 1; l < v.L; ++l) {
+            const int Hl = v.dims[l], Hn = v.dims[l + 1], off = v.noff[l], on = v.noff[l + 1];
+            bool any = false;  // a covered neuron of layer l + 1 covers all of layer l
             for (int i = 0; i < Hn; ++i)
                 if (bit((unsigned long long)(on + i))) {
                     cov[on + i] = 1;
-                    for (int j = 0; j < Hl; ++j) cov[off + j] = 1;
+                    any = true;
                 }
+            for (int j = 0; any && j < Hl; ++j) cov[off + j] = 1;
         }
     }
     long c = 0;

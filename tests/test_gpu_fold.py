@@ -184,3 +184,23 @@ def test_units_of_the_last_digit(vb, s, k, lo, hi):
     n = oracle.space_size(s, k)
     hi = min(hi, n)
     compare(run_gpu(vb, net, q, "bf16", lo=lo, hi=hi), oracle.verify(net, q, lo=lo, hi=hi), net, q)
+
+
+@pytest.mark.parametrize("dims", [[20, 7, 5, 3], [20, 33, 64, 10], [20, 31, 32, 32], [20, 65, 1, 2]])
+def test_covered_fraction_of_dense_and_sparse_masks(vb, dims):
+    """Eq. 3's fraction from masks whose rows start anywhere in a word, against the
+    oracle's loop over pairs."""
+    net = synth.make_net(820, dims, "relu", 2.0, "normal")
+    vnet = vb.Net(net)
+    _, sw = vnet.mask_words()
+    bits = sum(a * b for a, b in zip(dims[1:], dims[2:]))
+    rng = np.random.default_rng(820)
+    import ctypes as C
+    for share in (0.0, 0.002, 0.5, 1.0):
+        m = np.packbits(rng.random(32 * sw) < share, bitorder="little").view(np.uint32)
+        if bits % 32:
+            m[bits // 32] &= (1 << (bits % 32)) - 1
+        f = C.c_double()
+        assert vb.lib().vbmc_covered_fraction(vnet.h, 0, m.ctypes.data_as(C.POINTER(C.c_uint32)), C.byref(f)) == 0
+        assert f.value == oracle.ss_covered_fraction(dims, m)
+    vnet.free()
