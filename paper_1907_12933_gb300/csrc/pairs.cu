@@ -14,8 +14,10 @@
 // resolution of the undecided tests goes to the tie mask.
 #include "../../include/vbmc.h"
 #include "dev.cuh"
+#include "dfloat.cuh"
 #include "launch.h"
 
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -172,6 +174,340 @@ __global__ void __launch_bounds__(TP) k_pairs(NetView net, const uint8_t* x1s, c
     }
 }
 
+// The same covers with the potentials as FP32 pairs (ReLU and identity nets). FP64
+// runs at a sixty-fourth of the FP32 rate on this part and bound k_pairs; here a
+// multiply-add costs five or six FP32 instructions. Every test a bit rests on (sign,
+// value ratio, distance) has to clear its threshold by the potentials' error bound,
+// else the CTA evaluates that pair in FP64 (k_pairs's own steps).
+//
+// A dot product against an anchor sigma = 1.5 2^M, 2^(M-1) >= ||W_i|| ||h|| (so that no
+// partial sum leaves the binade): t = fma(w, h, sigma); q = t - sigma, the product on
+// the grid 2^(M-23), summed exactly; r = fma(w, h, -q) its rest, summed plainly over 16
+// terms and then by two_sum. Per 16 terms the rests lose at most 136 2^(M-48), each
+// rest 2^(M-48); with 2^M < 4 ||W_i|| ||h||: |error| <= 5 (K + 16) 2^-45 ||W_i|| ||h||.
+// Layer 1 runs on the grey levels (exact in FP32) and divides by 255 as a pair.
+//
+// CTA = IB images (IB / 2 pairs), a thread per neuron: one weight load serves IB
+// images, whose activations are shared-memory broadcasts. Bound by FP32 issue. 8,192
+// pairs on 784-512-512-10: 55.3 -> 3.7 ms (0.40 -> 6.0 TFLOP/s of dot products).
+constexpr int TPD = 256;
+
+template <int IB>
+struct PairDf {
+    double dist2[IB / 2][kMaxL + 2];
+    float E[IB], N[IB], X[IB];       // error norm and norm of a layer's input (layer 1: in grey levels);
+    float M[IB];                     // 5 (K + 16) 2^-45 M + E with M the norm on the [0, 1] scale
+    float sq[TPD / 32][IB / 2][4];   // per warp: ||h||^2 and ||u||^2 of a pair's two images
+    double ds[TPD / 32][IB / 2];
+    int nflip[IB / 2][kMaxL + 2], only[IB / 2][kMaxL + 2];
+    int undec[IB / 2];
+};
+
+// K terms of neuron column w0 (stride N) against IB images' inputs.
+template <int IB, bool L1>
+__device__ __forceinline__ void anchored_dot(const float* __restrict__ w0, int N, int K, const void* in, float sig,
+                                             float2 (&u)[IB]) {
+    float S[IB], H[IB], Lo[IB];
+#pragma unroll
+    for (int m = 0; m < IB; ++m) S[m] = H[m] = Lo[m] = 0.f;
+    for (int k0 = 0; k0 < K; k0 += 16) {
+        float r[IB];
+#pragma unroll
+        for (int m = 0; m < IB; ++m) r[m] = 0.f;
+        const int k1 = min(K, k0 + 16);
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) {
+            const float w = __ldg(w0 + (size_t)k * N);
+            float hx[IB], hy[IB];
+            if (L1) {
+                const float* h = static_cast<const float*>(in) + (size_t)k * IB;
+#pragma unroll
+                for (int m = 0; m < IB; m += 2) {
+                    const float2 v = *reinterpret_cast<const float2*>(h + m);
+                    hx[m] = v.x;
+                    hx[m + 1] = v.y;
+                }
+            } else {
+                const float2* h = static_cast<const float2*>(in) + (size_t)k * IB;
+#pragma unroll
+                for (int m = 0; m < IB; m += 2) {
+                    const float4 v = *reinterpret_cast<const float4*>(h + m);
+                    hx[m] = v.x;
+                    hy[m] = v.y;
+                    hx[m + 1] = v.z;
+                    hy[m + 1] = v.w;
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < IB; ++m) {
+                const float q = __fsub_rn(__fmaf_rn(w, hx[m], sig), sig);
+                S[m] = __fadd_rn(S[m], q);
+                float e = __fmaf_rn(w, hx[m], -q);
+                if (!L1) e = __fmaf_rn(w, hy[m], e);
+                r[m] = __fadd_rn(r[m], e);
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < IB; ++m) {
+            const float2 t = two_sum(H[m], r[m]);
+            H[m] = t.x;
+            Lo[m] = __fadd_rn(Lo[m], t.y);
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < IB; ++m) u[m] = df_add(make_float2(S[m], 0.f), two_sum(H[m], Lo[m]));
+}
+
+template <int IB>
+__global__ void __launch_bounds__(TPD) k_pairs_df(NetView net, const uint8_t* __restrict__ x1s,
+                                                  const uint8_t* __restrict__ x2s, int n_pairs, double g, double d,
+                                                  PairOut o, int bufw) {
+    constexpr int PB = IB / 2;
+    extern __shared__ double sh[];
+    __shared__ PairDf<IB> T;
+    float2* const buf0 = reinterpret_cast<float2*>(sh);      // [bufw][IB]
+    float2* const buf1 = buf0 + (size_t)bufw * IB;           // the same; layer 1's grey levels first
+    unsigned char* const fl = reinterpret_cast<unsigned char*>(buf1 + (size_t)bufw * IB);  // [total][PB]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int H0 = net.dims[0], L = net.L;
+    const bool relu = net.act == ACT_RELU;
+    const float tau = __double2float_ru(kTau), gf = __double2float_ru(g);
+    const float inv_hi = 1.f / 255.f;
+    const float2 inv = make_float2(inv_hi, (float)(1.0 / 255.0 - (double)inv_hi));
+    for (int p0 = blockIdx.x * PB; p0 < n_pairs; p0 += gridDim.x * PB) {
+        const int np = min(PB, n_pairs - p0);
+        float* const in0 = reinterpret_cast<float*>(buf1);
+        for (int im = 0; im < IB; ++im) {
+            const uint8_t* x = (im & 1 ? x2s : x1s) + (size_t)(p0 + (im >> 1)) * H0;
+            for (int k = tid; k < H0; k += TPD) in0[k * IB + im] = (im >> 1) < np ? (float)x[k] : 0.f;
+        }
+        if (tid < PB) T.undec[tid] = 0;
+        for (int e = tid; e < PB * (kMaxL + 2); e += TPD) {
+            T.nflip[e / (kMaxL + 2)][e % (kMaxL + 2)] = 0;
+            T.only[e / (kMaxL + 2)][e % (kMaxL + 2)] = -1;
+            T.dist2[e / (kMaxL + 2)][e % (kMaxL + 2)] = 0.0;
+        }
+        if (tid < IB) {  // grey levels: at most 255 sqrt(H_0)
+            T.N[tid] = __fmul_ru(255.f, __fsqrt_ru((float)H0));
+            T.E[tid] = 0.f;
+        }
+        __syncthreads();
+        for (int l = 1; l <= L; ++l) {
+            const int K = net.dims[l - 1], N = net.dims[l], off = net.noff[l];
+            const void* in = l == 1 ? static_cast<const void*>(buf1) : (l & 1 ? buf1 : buf0);
+            float2* const outb = l & 1 ? buf0 : buf1;
+            const float* __restrict__ WT = net.WT[l];
+            const float cK = 5.f * (float)(K + 16) * 0x1p-45f;
+            float Nm = 0.f;
+            for (int m = 0; m < IB; ++m) Nm = fmaxf(Nm, T.N[m]);
+            // sigma of a neuron: 1.5 2^M with 2^(M-1) >= ||W_i|| max ||h|| (and above 0)
+            auto anchor = [&](int n) {
+                const int ex = ilogbf(fmaxf(__fmul_ru(net.rownorm[l][n], Nm), 1e-30f));
+                return 1.5f * ldexpf(1.f, ex + 2);
+            };
+            // potentials: (sum) / 255 on layer 1, plus the bias
+            auto finish = [&](float2 v, int n) {
+                if (l == 1) {
+                    const float p = __fmul_rn(v.x, inv.x);
+                    float e = __fmaf_rn(v.x, inv.x, -p);
+                    e = __fmaf_rn(v.x, inv.y, e);
+                    e = __fmaf_rn(v.y, inv.x, e);
+                    v = two_sum(p, e);
+                }
+                return df_add(v, make_float2(net.b[l][n], 0.f));
+            };
+            if (N * 4 >= TPD) {
+                for (int n = tid; n < N; n += TPD) {
+                    float2 u[IB];
+                    if (l == 1) anchored_dot<IB, true>(WT + n, N, K, in, anchor(n), u);
+                    else anchored_dot<IB, false>(WT + n, N, K, in, anchor(n), u);
+#pragma unroll
+                    for (int m = 0; m < IB; ++m) outb[(size_t)n * IB + m] = finish(u[m], n);
+                }
+            } else {  // a narrow layer: a thread per neuron and pair
+                for (int it = tid; it < N * PB; it += TPD) {
+                    const int n = it / PB, pp = it % PB;
+                    float S[2] = {0.f, 0.f}, Hh[2] = {0.f, 0.f}, Lo[2] = {0.f, 0.f};
+                    const float sig = anchor(n);
+                    for (int k0 = 0; k0 < K; k0 += 16) {
+                        float r[2] = {0.f, 0.f};
+                        const int k1 = min(K, k0 + 16);
+#pragma unroll 4
+                        for (int k = k0; k < k1; ++k) {
+                            const float w = __ldg(WT + (size_t)k * N + n);
+                            float4 h;
+                            if (l == 1) {
+                                const float2 v = *reinterpret_cast<const float2*>(in0 + (size_t)k * IB + 2 * pp);
+                                h = make_float4(v.x, 0.f, v.y, 0.f);
+                            } else {
+                                h = *reinterpret_cast<const float4*>(static_cast<const float2*>(in) + (size_t)k * IB + 2 * pp);
+                            }
+                            float q = __fsub_rn(__fmaf_rn(w, h.x, sig), sig);
+                            S[0] = __fadd_rn(S[0], q);
+                            r[0] = __fadd_rn(r[0], __fmaf_rn(w, h.y, __fmaf_rn(w, h.x, -q)));
+                            q = __fsub_rn(__fmaf_rn(w, h.z, sig), sig);
+                            S[1] = __fadd_rn(S[1], q);
+                            r[1] = __fadd_rn(r[1], __fmaf_rn(w, h.w, __fmaf_rn(w, h.z, -q)));
+                        }
+#pragma unroll
+                        for (int m = 0; m < 2; ++m) {
+                            const float2 t = two_sum(Hh[m], r[m]);
+                            Hh[m] = t.x;
+                            Lo[m] = __fadd_rn(Lo[m], t.y);
+                        }
+                    }
+#pragma unroll
+                    for (int m = 0; m < 2; ++m)
+                        outb[(size_t)n * IB + 2 * pp + m] =
+                            finish(df_add(make_float2(S[m], 0.f), two_sum(Hh[m], Lo[m])), n);
+                }
+            }
+            if (tid < IB) {  // layer 1: the input's norm and error on the [0, 1] scale
+                const float nn = l == 1 ? __fmul_ru(T.N[tid], __fmul_ru(inv_hi, 1.f + 0x1p-22f)) : T.N[tid];
+                T.M[tid] = nn;
+                T.X[tid] = __fmaf_ru(cK, nn, T.E[tid]);
+            }
+            __syncthreads();
+            // ---- the layer's tests, a thread per (neuron, pair); a thread keeps its pair
+            const int pp = tid % PB;
+            const float X1 = T.X[2 * pp], X2 = T.X[2 * pp + 1];
+            const bool live = pp < np;
+            // the value change counts where layer l - 1 has at most one sign change
+            const bool ratio = l >= 2 && T.nflip[pp][l - 1] <= 1;
+            float h1 = 0.f, h2 = 0.f, s1 = 0.f, s2 = 0.f;
+            double dd = 0.0;
+            for (int n = tid / PB; n < N; n += TPD / PB) {
+                float2* up = outb + (size_t)n * IB + 2 * pp;
+                const float2 a = up[0], b = up[1];
+                if (live) {
+                    const float rn = net.rownorm[l][n];
+                    const float e1 = __fmaf_ru(rn, X1, __fmul_ru(0x1p-42f, fabsf(a.x)));
+                    const float e2 = __fmaf_ru(rn, X2, __fmul_ru(0x1p-42f, fabsf(b.x)));
+                    bool und = !(__fmul_rd(fabsf(a.x), 1.f - 0x1p-22f) > __fadd_ru(e1, tau)) ||
+                               !(__fmul_rd(fabsf(b.x), 1.f - 0x1p-22f) > __fadd_ru(e2, tau));
+                    const bool f = !und && ((a.x >= 0.f) != (b.x >= 0.f));
+                    bool v = false;
+                    if (ratio && !f && !und) {  // max - g min against tau
+                        const float A = fabsf(a.x), B = fabsf(b.x), mx = fmaxf(A, B), mi = fminf(A, B);
+                        const float t = fmaf(-(float)g, mi, mx);
+                        const float et = __fadd_ru(__fmaf_ru(gf, fmaxf(e1, e2), fmaxf(e1, e2)), tau);
+                        if (fabsf(t) > __fmaf_ru(0x1p-21f, __fmaf_ru(gf, mi, mx), et)) {
+                            v = t > 0.f;
+                        } else {  // near the threshold: the pairs' values in FP64
+                            const double da = fabs((double)a.x + (double)a.y), db = fabs((double)b.x + (double)b.y);
+                            const double td = fmax(da, db) - g * fmin(da, db);
+                            if (fabs(td - kTau) <= (double)et || fabs(td + kTau) <= (double)et) und = true;
+                            else v = td > kTau;
+                        }
+                    }
+                    if (und) T.undec[pp] = 1;
+                    if (f) {
+                        atomicAdd(&T.nflip[pp][l], 1);
+                        atomicMax(&T.only[pp][l], n);
+                    }
+                    fl[(size_t)(off + n) * PB + pp] = (unsigned char)((f ? 1 : 0) | (v ? 2 : 0));
+                    const double df = ((double)a.x - (double)b.x) + ((double)a.y - (double)b.y);
+                    dd += df * df;
+                }
+                s1 = __fmaf_ru(a.x, a.x, s1);
+                s2 = __fmaf_ru(b.x, b.x, s2);
+                if (l < L) {
+                    if (relu) {
+                        up[0] = a.x > 0.f ? a : make_float2(0.f, 0.f);
+                        up[1] = b.x > 0.f ? b : make_float2(0.f, 0.f);
+                    }
+                    const float p = relu ? fmaxf(a.x, 0.f) : a.x, q = relu ? fmaxf(b.x, 0.f) : b.x;
+                    h1 = __fmaf_ru(p, p, h1);
+                    h2 = __fmaf_ru(q, q, h2);
+                }
+            }
+#pragma unroll
+            for (int x = PB; x < 32; x <<= 1) {
+                h1 = __fadd_ru(h1, __shfl_xor_sync(0xffffffffu, h1, x));
+                h2 = __fadd_ru(h2, __shfl_xor_sync(0xffffffffu, h2, x));
+                s1 = __fadd_ru(s1, __shfl_xor_sync(0xffffffffu, s1, x));
+                s2 = __fadd_ru(s2, __shfl_xor_sync(0xffffffffu, s2, x));
+                dd += __shfl_xor_sync(0xffffffffu, dd, x);
+            }
+            if (lane < PB) {
+                T.sq[warp][pp][0] = h1;
+                T.sq[warp][pp][1] = h2;
+                T.sq[warp][pp][2] = s1;
+                T.sq[warp][pp][3] = s2;
+                T.ds[warp][pp] = dd;
+            }
+            __syncthreads();
+            if (tid < IB) {
+                const int pq = tid >> 1, im = tid & 1;
+                float hs = 0.f, us = 0.f;
+                double ds = 0.0;
+                for (int w = 0; w < TPD / 32; ++w) {
+                    hs = __fadd_ru(hs, T.sq[w][pq][im]);
+                    us = __fadd_ru(us, T.sq[w][pq][2 + im]);
+                    ds += T.ds[w][pq];
+                }
+                // ||err(u_l)|| <= sigma_l E + 5 (K + 16) 2^-45 ||W_l||_F N + 2^-42 ||u||; the
+                // activation is 1-Lipschitz (layer 1: its input carries no error)
+                float En = __fmul_ru(__fmul_ru(cK, net.frob[l]), T.M[tid]);
+                if (l > 1) En = __fmaf_ru(net.sig[l], T.E[tid], En);
+                En = __fmul_ru(__fmaf_ru(0x1p-42f, __fsqrt_ru(us), En), 1.f + 0x1p-20f);
+                const float other = __shfl_xor_sync((1u << IB) - 1u, En, 1);
+                if (im == 0) {
+                    T.dist2[pq][l] = ds;
+                    // a layer without a sign change whose distance lies near d: undecided
+                    if (l < L && T.nflip[pq][l] == 0) {
+                        const double dist = sqrt(ds), ed = (double)__fadd_ru(En, other) * 1.001 + 1e-12 * dist;
+                        if (fabs(dist - d) <= kTau + ed) T.undec[pq] = 1;
+                    }
+                }
+                T.N[tid] = __fmul_ru(__fsqrt_ru(hs), 1.f + 0x1p-20f);
+                T.E[tid] = En;
+            }
+            __syncthreads();
+        }
+        // ---- covers: no sign is a tie in a decided pair, so every bit is certain
+        for (int n = tid; n < net.total; n += TPD) {
+            bool any = false;
+            for (int q = 0; q < np; ++q) any = any || (!T.undec[q] && (fl[(size_t)n * PB + q] & 1));
+            if (any && o.flip) set_bit_once(o.flip, (unsigned long long)n);
+        }
+        for (int q = 0; q < np; ++q) {
+            if (T.undec[q]) continue;
+            for (int l = 1; l < L; ++l) {
+                const int nf = T.nflip[q][l];
+                const bool dc = nf == 0 && sqrt(T.dist2[q][l]) - d > kTau;
+                if (nf != 1 && !dc) continue;
+                const int Hn = net.dims[l + 1], on = net.noff[l + 1];
+                const unsigned long long r0 = (unsigned long long)net.ssoff[l] + (unsigned long long)max(T.only[q][l], 0) * Hn;
+                for (int i = tid; i < Hn; i += TPD) {
+                    const unsigned char x = fl[(size_t)(on + i) * PB + q];
+                    if (nf == 1) {
+                        if ((x & 1) && o.ss) set_bit_once(o.ss, r0 + i);
+                        if ((x & 2) && o.sv) set_bit_once(o.sv, r0 + i);
+                    } else {
+                        if ((x & 1) && o.ds) set_bit_once(o.ds, (unsigned long long)(on + i));
+                        if ((x & 2) && o.dv) set_bit_once(o.dv, (unsigned long long)(on + i));
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        // ---- the pairs left, in FP64
+        unsigned left = 0;
+        for (int q = 0; q < np; ++q) left |= (unsigned)(T.undec[q] != 0) << q;
+        const PairScratch S = pair_scratch(net, sh);
+        while (left) {
+            const int q = __ffs(left) - 1;
+            left &= left - 1u;
+            __syncthreads();
+            forward64(net, x1s + (size_t)(p0 + q) * H0, S.u1, S.h);
+            forward64(net, x2s + (size_t)(p0 + q) * H0, S.u2, S.h);
+            pair_covers(net, S, g, d, o);
+        }
+        __syncthreads();
+    }
+}
+
 // The covers over the enumeration: the pairs (x, x_t) of the unperturbed image
 // and each point t of [lo, hi) that passes the query's filter. x's potentials
 // once per CTA; x_t's layer 1 incrementally from them (its s changed pixels),
@@ -280,11 +616,31 @@ extern "C" vbmc_status vbmc_pair_coverage(const vbmc_net* net, const uint8_t* d_
     size_t smem = 0;
     vbmc_status s = pair_setup(v, params, out, st, &smem);
     if (s != VBMC_OK || n_pairs == 0) return s;
-    cudaFuncSetAttribute(k_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const PairOut o{out->flip, out->flip_tie, out->ss, out->ss_tie, out->sv, out->sv_tie,
                     out->ds, out->ds_tie, out->dv, out->dv_tie};
-    k_pairs<<<pair_grid((unsigned long long)n_pairs), TP, smem, st>>>(v, d_images1, d_images2, n_pairs, params->g,
-                                                                    params->d, o);
+    // FP32 pairs where the activation has a pair form, 8 images per CTA once that still
+    // gives every SM a CTA, else 2 (more CTAs, shorter chains per CTA)
+    const int bufw = std::max(v.hmax, (v.dims[0] + 1) / 2);
+    auto df_smem = [&](int ib) {
+        const size_t need = 2 * sizeof(float2) * (size_t)bufw * ib + (size_t)v.total * (ib / 2);
+        return std::max(need, smem);
+    };
+    int n_sm = 0, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    const int ib = n_pairs >= 4 * n_sm && df_smem(8) <= 200 * 1024 ? 8 : 2;
+    if (v.act != ACT_SIGMOID && df_smem(ib) <= 200 * 1024) {
+        const size_t sm = df_smem(ib);
+        const unsigned long long groups = ((unsigned long long)n_pairs + ib / 2 - 1) / (ib / 2);
+        const unsigned grid = (unsigned)std::min<unsigned long long>(groups, (unsigned long long)n_sm * 8);
+        auto kern = ib == 8 ? k_pairs_df<8> : k_pairs_df<2>;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        kern<<<grid, TPD, sm, st>>>(v, d_images1, d_images2, n_pairs, params->g, params->d, o, bufw);
+    } else {
+        cudaFuncSetAttribute(k_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_pairs<<<pair_grid((unsigned long long)n_pairs), TP, smem, st>>>(v, d_images1, d_images2, n_pairs, params->g,
+                                                                        params->d, o);
+    }
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? VBMC_OK : set_error(VBMC_ERR_CUDA, cudaGetErrorString(e));
 }

@@ -63,3 +63,21 @@ def test_pair_coverage_edge_cases(vb):
     for k, v in exp.items():
         np.testing.assert_array_equal(got[k][:len(v)], v, err_msg=k)
     assert not any(got[k].any() for k in ("flip", "ss", "sv", "ds", "dv"))
+
+
+@pytest.mark.parametrize("act,dims,n,g,d", [
+    ("relu", [17, 33, 70, 5], 700, 1.3, 0.2), ("relu", [784, 65, 3], 613, 1.5, 0.5),
+    ("identity", [20, 40, 24, 6], 640, 2.0, 0.0), ("relu", [9, 260, 12, 2], 3, 1.1, 0.05),
+    ("relu", [30, 16, 16, 16, 4], 1300, 1.2, 0.1)])
+def test_pairs_as_fp32_pairs(vb, act, dims, n, g, d):
+    """The FP32-pair kernel at both of its group sizes, ragged widths and counts; identical
+    images (distance exactly d = 0, ratio exactly 1) leave their pairs to the FP64 steps."""
+    net = synth.make_net(33, dims, act, 2.0, "normal")
+    a, b = _pairs(11, n, dims[0], min(4, dims[0]), 60)
+    b[: n // 9] = a[: n // 9]
+    vnet = vb.Net(net)
+    for gg in (g, 1.0):
+        got = vb.pair_coverage(vnet, a, b, g=gg, d=d)
+        exp = oracle.pairs_coverage(net, a, b, g=gg, d=d)
+        for k, v in exp.items():
+            np.testing.assert_array_equal(got[k][:len(v)], v, err_msg=k)
