@@ -57,6 +57,8 @@ struct vbmc_proposal {
     float* act[4] = {};       // activations of the last forward (act[0]: input copy)
     float* dact[4] = {};
     float* loss = nullptr;    // [2]: loss sum, number of weighted rows
+    float* ws = nullptr;      // partial tiles of a split product, and its arrival counts
+    unsigned int* cnt = nullptr;
     int bmax = 0;
     long step = 0;
     std::vector<void*> owned;
@@ -74,80 +76,184 @@ __device__ __forceinline__ float rnd_bf16(float x) { return __bfloat162float(__f
 //   A(m, k) = TA ? A[k * lda + m] : A[m * lda + k]
 //   B(k, n) = TB ? B[n * ldb + k] : B[k * ldb + n]
 // 64 x 64 tile per CTA of 256 threads, 4 x 4 outputs per thread; bf != 0
-// rounds both operands to BF16 as they are staged.
+// rounds both operands to BF16 as they are staged. rowsum (TA): also sum_k A(m, k).
+// A mini-batch's products have few tiles (128 x 256 x 2352: 8) and were bound by the
+// latency of one CTA's chain of loads. So the next step's operands are loaded (16 bytes
+// a thread where rows and pointers allow it) while this step's are multiplied, and K is
+// split over gridDim.z CTAs: each leaves its partial tile in ws, the last one to arrive
+// (cnt) adds them up in order. 128 x 256 x 2352: 332 -> 16 us; the ten launches of a
+// gradient on 2352-256-256-64, 128 rows (bias gradients ride on the weight products):
+// 541 -> 111 us.
+struct GemmArgs {
+    int M, N, K, lda, ldb, ldc, kc;  // kc: K of a split, a multiple of GK
+    const float *A, *B, *bias, *mask;
+    float *C, *rowsum, *ws;
+    unsigned int* cnt;
+    int relu, bf, va, vb;  // va, vb: A, B may be read 16 bytes at a time
+};
+
+// Four operand elements for this thread: `along` runs over 4 consecutive memory
+// positions (of `lim_a`), `row` over rows of stride ld.
+__device__ __forceinline__ float4 load4(const float* p, int ld, int row, int nrow, int along, int lim_a, int vec) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row >= nrow || along >= lim_a) return v;
+    const float* q = p + (size_t)row * ld + along;
+    if (vec && along + 3 < lim_a) return *reinterpret_cast<const float4*>(q);
+    v.x = q[0];
+    if (along + 1 < lim_a) v.y = q[1];
+    if (along + 2 < lim_a) v.z = q[2];
+    if (along + 3 < lim_a) v.w = q[3];
+    return v;
+}
+
 template <bool TA, bool TB>
-__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const float* __restrict__ A, int lda,
-                                              const float* __restrict__ B, int ldb, float* __restrict__ C,
-                                              int ldc, const float* __restrict__ bias,
-                                              const float* __restrict__ mask, int relu, int bf) {
-    __shared__ float As[GK][GT + 4];
-    __shared__ float Bs[GK][GT + 4];
+__global__ void __launch_bounds__(256) k_gemm(const GemmArgs g) {
+    __shared__ __align__(16) float As[2][GK][GT + 4];
+    __shared__ __align__(16) float Bs[2][GK][GT + 4];
+    __shared__ int last;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += GK) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int e = tid + r * 256;
-            int m, k;
-            if (TA) { k = e / GT; m = e % GT; } else { m = e / GK; k = e % GK; }
-            const int gm = m0 + m, gk = k0 + k;
-            float a = 0.f;
-            if (gm < M && gk < K) a = TA ? A[(size_t)gk * lda + gm] : A[(size_t)gm * lda + gk];
-            As[k][m] = bf ? rnd_bf16(a) : a;
-            int n, kb;
-            if (TB) { n = e / GK; kb = e % GK; } else { kb = e / GT; n = e % GT; }
-            const int gn = n0 + n, gkb = k0 + kb;
-            float bv = 0.f;
-            if (gn < N && gkb < K) bv = TB ? B[(size_t)gn * ldb + gkb] : B[(size_t)gkb * ldb + gn];
-            Bs[kb][n] = bf ? rnd_bf16(bv) : bv;
+    const int kb = blockIdx.z * g.kc, ke = min(g.K, kb + g.kc);
+    // operands whose k is the contiguous index: 4 k of one of 64 rows; else 4 rows of one k
+    const int rk = tid >> 2, ck = (tid & 3) * 4, rr = tid >> 4, cr = (tid & 15) * 4;
+    auto load_a = [&](int k0) {
+        return TA ? load4(g.A, g.lda, k0 + rr, ke, m0 + cr, g.M, g.va) : load4(g.A, g.lda, m0 + rk, g.M, k0 + ck, ke, g.va);
+    };
+    auto load_b = [&](int k0) {
+        return TB ? load4(g.B, g.ldb, n0 + rk, g.N, k0 + ck, ke, g.vb) : load4(g.B, g.ldb, k0 + rr, ke, n0 + cr, g.N, g.vb);
+    };
+    auto store = [&](float (&S)[GK][GT + 4], bool kin, float4 v) {
+        if (g.bf) v = make_float4(rnd_bf16(v.x), rnd_bf16(v.y), rnd_bf16(v.z), rnd_bf16(v.w));
+        if (kin) {
+            S[ck][rk] = v.x;
+            S[ck + 1][rk] = v.y;
+            S[ck + 2][rk] = v.z;
+            S[ck + 3][rk] = v.w;
+        } else {
+            *reinterpret_cast<float4*>(&S[rr][cr]) = v;
         }
-        __syncthreads();
+    };
+    float acc[4][4] = {};
+    float rs = 0.f;
+    const bool sums = g.rowsum && blockIdx.x == 0;
+    if (kb < ke) {
+        float4 a = load_a(kb), b = load_b(kb);
+        store(As[0], !TA, a);
+        store(Bs[0], TB, b);
+    }
+    __syncthreads();
+    int buf = 0;
+    for (int k0 = kb; k0 < ke; k0 += GK, buf ^= 1) {
+        const bool more = k0 + GK < ke;
+        float4 na, nb;
+        if (more) {
+            na = load_a(k0 + GK);
+            nb = load_b(k0 + GK);
+        }
 #pragma unroll
         for (int kk = 0; kk < GK; ++kk) {
-            float a[4], bb[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx * 4 + j];
+            const float4 a = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
+            const float4 b = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
+            const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+        }
+        if (sums && tid < GT) {
+#pragma unroll
+            for (int kk = 0; kk < GK; ++kk) rs += As[buf][kk][tid];
+        }
+        if (more) {
+            store(As[buf ^ 1], !TA, na);
+            store(Bs[buf ^ 1], TB, nb);
         }
         __syncthreads();
+    }
+    if (sums && tid < GT && m0 + tid < g.M) g.rowsum[m0 + tid] = rs;  // (never split)
+    if (gridDim.z > 1) {
+        const unsigned tile = blockIdx.y * gridDim.x + blockIdx.x, S = gridDim.z;
+        float* mine = g.ws + ((size_t)tile * S + blockIdx.z) * GT * GT;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            *reinterpret_cast<float4*>(&mine[(ty * 4 + i) * GT + tx * 4]) =
+                make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            last = atomicAdd(&g.cnt[tile], 1u) == S - 1;
+            if (last) g.cnt[tile] = 0u;  // for the next product on this stream
+        }
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        const float* all = g.ws + (size_t)tile * S * GT * GT;
+#pragma unroll 2
+        for (unsigned z = 0; z < S; ++z) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 v = __ldcg(reinterpret_cast<const float4*>(&all[(size_t)z * GT * GT + (ty * 4 + i) * GT + tx * 4]));
+                acc[i][0] += v.x;
+                acc[i][1] += v.y;
+                acc[i][2] += v.z;
+                acc[i][3] += v.w;
+            }
+        }
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int m = m0 + ty * 4 + i;
-        if (m >= M) continue;
+        if (m >= g.M) continue;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int n = n0 + tx * 4 + j;
-            if (n >= N) continue;
+            if (n >= g.N) continue;
             float v = acc[i][j];
-            if (bias) v += bias[n];
-            if (relu) v = fmaxf(v, 0.f);
-            if (mask && !(mask[(size_t)m * ldc + n] > 0.f)) v = 0.f;
-            C[(size_t)m * ldc + n] = v;
+            if (g.bias) v += g.bias[n];
+            if (g.relu) v = fmaxf(v, 0.f);
+            if (g.mask && !(g.mask[(size_t)m * g.ldc + n] > 0.f)) v = 0.f;
+            g.C[(size_t)m * g.ldc + n] = v;
         }
     }
 }
 
-template <bool TA, bool TB>
-void gemm(int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
-          const float* bias, const float* mask, int relu, int bf, cudaStream_t st) {
-    dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT);
-    k_gemm<TA, TB><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, mask, relu, bf);
-}
+constexpr int kSplitTiles = 304;  // partial tiles a product may leave: two CTAs on each of 152 SMs
 
-// Column sums: out[n] = sum_m X[m][n] (bias gradients).
-__global__ void k_colsum(const float* X, int M, int N, float* out) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float acc = 0.f;
-    for (int m = 0; m < M; ++m) acc += X[(size_t)m * N + n];
-    out[n] = acc;
+template <bool TA, bool TB>
+void gemm(const vbmc_proposal* p, int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C,
+          int ldc, const float* bias, const float* mask, int relu, int bf, float* rowsum, cudaStream_t st) {
+    GemmArgs g{};
+    g.M = M;
+    g.N = N;
+    g.K = K;
+    g.lda = lda;
+    g.ldb = ldb;
+    g.ldc = ldc;
+    g.A = A;
+    g.B = B;
+    g.C = C;
+    g.bias = bias;
+    g.mask = mask;
+    g.rowsum = rowsum;
+    g.relu = relu;
+    g.bf = bf;
+    g.va = lda % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+    g.vb = ldb % 4 == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
+    g.ws = p->ws;
+    g.cnt = p->cnt;
+    dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT, 1);
+    // a split per CTA that would otherwise be missing, of at least two steps of K
+    const long tiles = (long)grid.x * grid.y;
+    long S = rowsum || tiles > kSplitTiles / 2 ? 1 : kSplitTiles / 2 / tiles;
+    if (S > K / (2 * GK)) S = K / (2 * GK);
+    if (S < 1) S = 1;
+    g.kc = (int)(((K + S - 1) / S + GK - 1) / GK * GK);
+    grid.z = (unsigned)((K + g.kc - 1) / g.kc);
+    k_gemm<TA, TB><<<grid, 256, 0, st>>>(g);
 }
 
 // Listwise softmax cross-entropy, one warp per row: dZ = p - t / sum t
@@ -192,6 +298,62 @@ __global__ void k_scale_by_count(float* dZ, long n, const float* loss) {
     if (i >= n) return;
     const float c = loss[1];
     dZ[i] = c > 0.f ? dZ[i] / c : 0.f;
+}
+
+// Both in one block, for a mini-batch: the rows' count is known before they are scaled,
+// and the loss is a sum in a fixed order.
+__global__ void __launch_bounds__(1024) k_softmax_ce_all(const float* Z, const float* Tg, float* dZ, float* loss,
+                                                         int B, int T) {
+    __shared__ float ls[32], cs[32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float lsum = 0.f, cnt = 0.f;
+    for (int r = warp; r < B; r += 32) {
+        float ts = 0.f;
+        for (int i = lane; i < T; i += 32) ts += Tg[(size_t)r * T + i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ts += __shfl_xor_sync(0xffffffffu, ts, o);
+        cnt += ts > 0.f ? 1.f : 0.f;
+    }
+    if (lane == 0) cs[warp] = cnt;
+    __syncthreads();
+    cnt = 0.f;
+    for (int w = 0; w < 32; ++w) cnt += cs[w];
+    for (int r = warp; r < B; r += 32) {
+        const float* z = Z + (size_t)r * T;
+        const float* t = Tg + (size_t)r * T;
+        float mx = -INFINITY, ts = 0.f;
+        for (int i = lane; i < T; i += 32) {
+            mx = fmaxf(mx, z[i]);
+            ts += t[i];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            ts += __shfl_xor_sync(0xffffffffu, ts, o);
+        }
+        float se = 0.f;
+        for (int i = lane; i < T; i += 32) se += expf(z[i] - mx);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+        const float lse = mx + logf(se);
+        float l = 0.f;
+        for (int i = lane; i < T; i += 32) {
+            const float q = ts > 0.f ? t[i] / ts : 0.f;
+            dZ[(size_t)r * T + i] = ts > 0.f ? (expf(z[i] - lse) - q) / cnt : 0.f;
+            l -= q * (z[i] - lse);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (ts > 0.f) lsum += l;
+    }
+    if (lane == 0) ls[warp] = lsum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        lsum = 0.f;
+        for (int w = 0; w < 32; ++w) lsum += ls[w];
+        loss[0] = lsum;
+        loss[1] = cnt;
+    }
 }
 
 // Adam with decoupled weight decay (bias-corrected moments).
@@ -395,6 +557,10 @@ extern "C" vbmc_status vbmc_proposal_create(int32_t n_features, int32_t h1, int3
         A(&p->dact[l], (size_t)max_batch * p->dims[l]);
     }
     A(&p->loss, 2);
+    A(&p->ws, (size_t)kSplitTiles * GT * GT);
+    float* cnt = nullptr;
+    A(&cnt, kSplitTiles);  // zeros
+    p->cnt = reinterpret_cast<unsigned int*>(cnt);
     if (e != cudaSuccess) {
         vbmc_proposal_free(p);
         return set_error(VBMC_ERR_OOM, "proposal_create: device allocation failed");
@@ -418,8 +584,8 @@ void forward(vbmc_proposal* p, const float* d_X, int B, int bf, cudaStream_t st)
     cudaMemcpyAsync(p->act[0], d_X, sizeof(float) * (size_t)B * p->dims[0], cudaMemcpyDeviceToDevice, st);
     for (int l = 1; l <= 3; ++l) {
         const int K = p->dims[l - 1], N = p->dims[l];
-        gemm<false, true>(B, N, K, p->act[l - 1], K, p->W[l], K, p->act[l], N, p->b[l], nullptr, l < 3, bf,
-                          st);
+        gemm<false, true>(p, B, N, K, p->act[l - 1], K, p->W[l], K, p->act[l], N, p->b[l], nullptr, l < 3, bf,
+                          nullptr, st);
     }
 }
 
@@ -449,19 +615,23 @@ extern "C" vbmc_status vbmc_proposal_grads(vbmc_proposal* p, const float* d_X, c
     if (s != VBMC_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     forward(p, d_X, B, bf16 ? 1 : 0, st);
-    cudaMemsetAsync(p->loss, 0, sizeof(float) * 2, st);
     const int T = p->dims[3];
-    k_softmax_ce<<<nblk((long)B * 32, 256), 256, 0, st>>>(p->act[3], d_T, p->dact[3], p->loss, B, T);
-    k_scale_by_count<<<nblk((long)B * T, 256), 256, 0, st>>>(p->dact[3], (long)B * T, p->loss);
+    if ((long)B * T <= 65536) {  // 64 values a thread at most: one launch beats two and a memset
+        k_softmax_ce_all<<<1, 1024, 0, st>>>(p->act[3], d_T, p->dact[3], p->loss, B, T);
+    } else {
+        cudaMemsetAsync(p->loss, 0, sizeof(float) * 2, st);
+        k_softmax_ce<<<nblk((long)B * 32, 256), 256, 0, st>>>(p->act[3], d_T, p->dact[3], p->loss, B, T);
+        k_scale_by_count<<<nblk((long)B * T, 256), 256, 0, st>>>(p->dact[3], (long)B * T, p->loss);
+    }
     for (int l = 3; l >= 1; --l) {
         const int K = p->dims[l - 1], N = p->dims[l];
         // dW_l = dact_l^T act_{l-1}   (N x K),  db_l = column sums of dact_l
-        gemm<true, false>(N, K, B, p->dact[l], N, p->act[l - 1], K, p->gW[l], K, nullptr, nullptr, 0, 0, st);
-        k_colsum<<<nblk(N, 256), 256, 0, st>>>(p->dact[l], B, N, p->gb[l]);
+        gemm<true, false>(p, N, K, B, p->dact[l], N, p->act[l - 1], K, p->gW[l], K, nullptr, nullptr, 0, 0, p->gb[l],
+                          st);
         // dact_{l-1} = (dact_l W_l) * ReLU'(act_{l-1})
         if (l > 1)
-            gemm<false, false>(B, K, N, p->dact[l], N, p->W[l], K, p->dact[l - 1], K, nullptr, p->act[l - 1], 0,
-                               0, st);
+            gemm<false, false>(p, B, K, N, p->dact[l], N, p->W[l], K, p->dact[l - 1], K, nullptr, p->act[l - 1], 0,
+                               0, nullptr, st);
     }
     if (h_loss) {
         float hl[2];

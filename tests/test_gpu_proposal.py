@@ -247,3 +247,25 @@ def test_learned_order_finds_witnesses_sooner(vb):
         assert g["tiles_checked"] == P.first_witness_rank(cte[i:i + 1], learned[i:i + 1])[0]
         assert cte[i, g["witness_tile"]] == g["n_adversarial"] > 0
     prop.free()
+
+
+@pytest.mark.parametrize("dims,B", [((300, 64, 65, 2), 3), ((2352, 256, 256, 64), 256), ((75, 33, 31, 1000), 70),
+                                    ((1001, 130, 64, 16), 64), ((33, 5, 3, 4), 2)])
+def test_gradients_at_split_and_ragged_sizes(vb, dims, B):
+    """Products split over K (few tiles) and not, rows that 16-byte loads cannot take,
+    more values than one block's softmax serves; the same tolerance as the gradient
+    check (FP32 sums, K * 2^-24 of sum |terms|), and the same bits on a second call."""
+    prop = vb.Proposal(dims, max_batch=max(B, 8), seed=4)
+    X, lab = _batch(2, B, dims[0], dims[3])
+    loss = prop.grads(_dev(X), _dev(lab), bf16=False)
+    P = [prop.params(l) for l in (1, 2, 3)]
+    ref_loss, ref = pr.mlp_grads([(p["W"], p["b"]) for p in P], X, lab)
+    assert loss == pytest.approx(ref_loss, rel=1e-5)
+    for l in range(3):
+        for g, r in ((P[l]["gW"], ref[l][0]), (P[l]["gb"], ref[l][1])):
+            assert np.linalg.norm(g - r) <= 1e-4 * np.linalg.norm(r) + 1e-12
+    if B * dims[3] <= 65536:
+        assert prop.grads(_dev(X), _dev(lab), bf16=False) == loss
+        for l in range(3):
+            np.testing.assert_array_equal(prop.params(l + 1)["gW"], P[l]["gW"])
+    prop.free()
