@@ -374,7 +374,7 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
     } else {
         A(&r->d_in, kInImage + (size_t)v.dims[0]);
         uint8_t* out = nullptr;
-        A(&out, sizeof(Counters) + 2 * sizeof(unsigned long long));
+        A(&out, sizeof(Counters) + 6 * sizeof(unsigned long long));
         if (e == cudaSuccess) {
             r->d_q = reinterpret_cast<QueryView*>(r->d_in);
             r->d_tp = reinterpret_cast<unsigned long long*>(r->d_in + kInTp);
@@ -382,6 +382,7 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
             r->d_image = r->d_in + kInImage;
             r->d_cnt = reinterpret_cast<Counters*>(out);
             r->d_claim = reinterpret_cast<unsigned long long*>(out + sizeof(Counters));
+            r->d_qcount = r->d_claim + 2;
         }
     }
     A(&q.pix, (size_t)S);
@@ -403,7 +404,7 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
     q.ss = q.flip_tie + v.flip_words;
     q.ss_tie = q.ss + v.ss_words;
     A(&q.ties, (size_t)std::max<uint32_t>(1, caps->ties_cap));
-    A(&r->d_qcount, 4);
+    if (arena) A(&r->d_qcount, 4);
     A(&r->d_margin, 1);
     if (caps->max_points) A(&q.bitmap, (size_t)((caps->max_points + 31) / 32));
     // members of a batch keep small queues of their own (the batch shares the arena's)
@@ -619,13 +620,17 @@ enum { STAGE_SETUP = 1, STAGE_PASSES = 2, STAGE_ALL = 3 };
 // stage resets the counters and clears the masks and the verdict bitmap over
 // [0, hi); everything else it computes depends on the box, not on [lo, hi),
 // so one set-up over the whole space serves passes over any sub-ranges.
+// h_folded (pinned; one query): the call may wait for the set-up, so it learns here
+// whether the query folded and launches the passes of that form only. Without it both
+// forms are launched and each leaves the other's queries out (about 20 us of launches
+// that return at once).
 vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, int nq,
                            const unsigned long long* d_tp, unsigned long long ntiles,
                            unsigned long long* d_qcount, QEntry* const* d_queue,
                            unsigned long long cap, const cudaEvent_t* ev, const vbmc_options& opt,
                            cudaStream_t st, bool capturing = false, int stages = STAGE_ALL,
                            WideWork* ww = nullptr, TcQueryWork* tw = nullptr,
-                           unsigned long long* d_claim = nullptr) {
+                           unsigned long long* d_claim = nullptr, int* h_folded = nullptr) {
     if (nq != 1) tw = nullptr;  // compacted columns are per query: single-query calls only
     const NetView& v = net->v;
     // inside a stream capture an event record must be an explicit graph node
@@ -655,20 +660,38 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
             return fail(VBMC_ERR_STATE, "the result has no wide-layer workspace (created with caps.wide_chunk = -1, "
                                         "or as a batch member without one)");
     }
-    // the folded net checks the queries whose set-up builds one (fold.cu); which
-    // they are is known on the device only, so the general passes are launched too
-    // and leave those queries out
-    bool fold = false;
+    // the folded net checks the queries whose set-up builds one (fold.cu)
+    bool fold = false, general = true;  // forms to launch
     for (int i = 0; i < nq; ++i) fold = fold || hq[i].fold;
     unsigned long long* const d_unfolded = nq > 1 && d_claim ? d_claim + 2 : nullptr;
-    VB_CUDA(cudaMemsetAsync(d_qcount, 0, sizeof(unsigned long long) * 4, st));
-    if (d_claim) VB_CUDA(cudaMemsetAsync(d_claim, 0, sizeof(unsigned long long) * (nq > 1 ? 3 : 2), st));
+    if (d_claim && d_qcount == d_claim + 2) {  // a result's own counters lie in a row
+        VB_CUDA(cudaMemsetAsync(d_claim, 0, sizeof(unsigned long long) * 6, st));
+    } else {
+        VB_CUDA(cudaMemsetAsync(d_qcount, 0, sizeof(unsigned long long) * 4, st));
+        if (d_claim) VB_CUDA(cudaMemsetAsync(d_claim, 0, sizeof(unsigned long long) * (nq > 1 ? 3 : 2), st));
+    }
     VB_CUDA(record(ev[0]));
     if (stages & STAGE_SETUP) {
         unsigned long long max_hi = 0;
         for (int i = 0; i < nq; ++i)
             if (hq[i].bitmap) max_hi = std::max(max_hi, hq[i].hi);
-        launch_prologue(v, d_qs, nq, max_sr, st, max_hi, fold, d_unfolded);
+        launch_prologue(v, d_qs, nq, st, max_hi, fold, d_unfolded);
+        // the chunks of the wide-layer path clear a workspace each, so it always asks
+        int here = 0;
+        int* const h = h_folded ? h_folded : (wide ? &here : nullptr);
+        if (fold && any && nq == 1 && h) {
+            VB_CUDA(cudaMemcpyAsync(h, hq[0].fst, sizeof(int), cudaMemcpyDeviceToHost, st));
+            VB_CUDA(cudaStreamSynchronize(st));
+            fold = *h != 0;
+            general = !fold;
+        }
+        if (general) launch_prologue_screens(v, d_qs, nq, max_sr, st);
+    } else if (wide && fold && any) {
+        int here = 0;
+        VB_CUDA(cudaMemcpyAsync(&here, hq[0].fst, sizeof(int), cudaMemcpyDeviceToHost, st));
+        VB_CUDA(cudaStreamSynchronize(st));
+        fold = here != 0;
+        general = !fold;
     }
     VB_CUDA(record(ev[1]));
     if (tensor && any) {
@@ -676,7 +699,7 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
             return fail(VBMC_ERR_UNSUPPORTED, "tensor-core screen does not support this net/precision");
         vbmc_status sst = tc_build(net->tc, v, net->hW, net->hb, opt.precision);
         if (sst != VBMC_OK) return fail(sst, "tensor-core set-up failed");
-        if (stages & STAGE_SETUP) tc_launch_query_setup(net->tc, v, d_qs, nq, opt.precision, st, tw);
+        if ((stages & STAGE_SETUP) && general) tc_launch_query_setup(net->tc, v, d_qs, nq, opt.precision, st, tw);
     }
     if (!(stages & STAGE_PASSES)) return VBMC_OK;
     // queue levels: 0 tensor split pass, 1 FP32 pass, 2 double-float pass, 3 FP64 pass
@@ -699,9 +722,15 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
         launch_fold(v, d_qs, nq, wide ? nullptr : d_tp, ntiles, mt, !wide, wide || !d_claim ? nullptr : d_claim + 1,
                     qsplit, 0, net->n_sm, st);
         launch_fold64(v, d_qs, d_queue[0], d_qcount + 0, cap, q64, 3, net->n_sm, st);
-        if (wide) launch_fp64(v, d_qs, nq, d_queue[3], d_qcount + 3, cap, 0, 0, net->n_sm, st);
+        if (!general) {
+            VB_CUDA(record(ev[2]));
+            VB_CUDA(record_rest());
+            launch_fp64(v, d_qs, nq, d_queue[3], d_qcount + 3, cap, 0, 0, net->n_sm, st);
+            if (wide) wide_done(d_qs, st);
+        }
     }
-    if (any && wide) {
+    if (!general) {
+    } else if (any && wide) {
         // the chunk loop interleaves the screen and the rechecks: all of it counts as screen
         vbmc_status fs = wide_run(net->wide, wtype, *ww, v, d_qs, hq[0], hq[0].lo, hq[0].hi, d_qcount, d_queue, cap,
                                   net->n_sm, st);
@@ -804,10 +833,11 @@ QueryView make_view(const vbmc_result* r, const uint8_t* d_image, const int* d_p
     return q;
 }
 
-// Enqueue the full pipeline for one query whose image/pixels are on the device.
+// Enqueue the full pipeline for one query whose image/pixels are on the device. wait:
+// the caller waits for the result anyway (see h_folded of enqueue_passes).
 vbmc_status enqueue(vbmc_net* net, vbmc_result* r, const uint8_t* d_image, const int* d_pix, int s,
                     int k, uint64_t lo, uint64_t hi, uint64_t n, const vbmc_options& opt,
-                    cudaStream_t st, const QueryExtra& x = QueryExtra(), bool fold = true) {
+                    cudaStream_t st, const QueryExtra& x = QueryExtra(), bool fold = true, bool wait = false) {
     QueryView q = make_view(r, d_image, d_pix, s, k, lo, hi, n, opt, 0, x, fold);
     q.budget_ns = opt.time_budget_ms > 0.0 ? (unsigned long long)(opt.time_budget_ms * 1e6) : 0ull;
     std::vector<unsigned long long> tp = tile_prefix(net->v, opt.precision, &q, 1);
@@ -832,7 +862,8 @@ vbmc_status enqueue(vbmc_net* net, vbmc_result* r, const uint8_t* d_image, const
     const cudaEvent_t ev[7] = {r->ev0, r->ev_pro, r->ev_scr, r->ev1, r->ev_split, r->ev_f32, r->ev_df};
     vbmc_status sst = enqueue_passes(net, r->d_q, &q, 1, r->d_tp, tp[1], r->d_qcount, r->d_queue,
                                      std::max<uint64_t>(1, r->caps.queue_cap), ev, opt, st, false, STAGE_ALL,
-                                     &r->ww, r->have_tw ? &r->tw : nullptr, claims ? r->d_claim : nullptr);
+                                     &r->ww, r->have_tw ? &r->tw : nullptr, claims ? r->d_claim : nullptr,
+                                     wait ? reinterpret_cast<int*>(r->h_claim + 1) : nullptr);
     if (sst != VBMC_OK) {
         if (r->h_in) cudaStreamSynchronize(st);  // the pinned block has been read
         return sst;
@@ -977,7 +1008,7 @@ vbmc_status verify_query(vbmc_net* net, const vbmc_query* q, const vbmc_options*
             VB_CUDA(cudaMemcpyAsync(res->d_pix_in, q->pixels, sizeof(int32_t) * q->s,
                                     cudaMemcpyHostToDevice, stq));
     }
-    st = enqueue(net, res, res->d_image, res->d_pix_in, q->s, q->k, q->lo, h, n, *opt, stq, x, fold);
+    st = enqueue(net, res, res->d_image, res->d_pix_in, q->s, q->k, q->lo, h, n, *opt, stq, x, fold, true);
     if (st != VBMC_OK) return st;
     res->image.assign(q->image, q->image + H0);
     res->pixels.assign(q->pixels, q->pixels + q->s);

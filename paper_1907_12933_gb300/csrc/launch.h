@@ -6,12 +6,14 @@
 
 namespace vbmc {
 
-// FP64 base pass, tables and screen constants for nq queries (d_qs on device).
-// max_sr: max over queries of s * R; max_hi: of the verdict bitmaps' bits (0: off).
-// fold: some view has its fold flag set; *d_unfolded (optional) then gains the
-// queries that did not fold.
-void launch_prologue(const NetView& net, QueryView* d_qs, int nq, int max_sr, cudaStream_t st,
-                     unsigned long long max_hi, bool fold, unsigned long long* d_unfolded);
+// FP64 base pass for nq queries (d_qs on device). max_hi: max over queries of the
+// verdict bitmaps' bits (0: off). fold: some view has its fold flag set, their folded
+// nets are packed; *d_unfolded (optional) then gains the queries that did not fold.
+void launch_prologue(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long max_hi,
+                     bool fold, unsigned long long* d_unfolded);
+// Tables and constants of the general screens, after it (folded queries are left out).
+// max_sr: max over queries of s * R.
+void launch_prologue_screens(const NetView& net, QueryView* d_qs, int nq, int max_sr, cudaStream_t st);
 
 // Folded nets (fold.cu): a net whose calls may fold; the packed form of the
 // queries' rows after the base pass; the first pass over folded queries; the

@@ -494,11 +494,14 @@ void launch_pro_layer(const NetView& net, QueryView* d_qs, int nq, int l, cudaSt
         k_pro_layer<1><<<dim3((net.dims[l] + 7) / 8, nq), 256, 0, st>>>(net, d_qs, nq, l);
 }
 
-void launch_prologue(const NetView& net, QueryView* d_qs, int nq, int max_sr, cudaStream_t st,
-                     unsigned long long max_hi, bool fold, unsigned long long* d_unfolded) {
+void launch_prologue(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long max_hi,
+                     bool fold, unsigned long long* d_unfolded) {
     launch_pro_init(net, d_qs, nq, st, max_hi);
     for (int l = 1; l <= net.L; ++l) launch_pro_layer(net, d_qs, nq, l, st);
     if (fold) launch_fold_pack(net, d_qs, nq, st, d_unfolded);
+}
+
+void launch_prologue_screens(const NetView& net, QueryView* d_qs, int nq, int max_sr, cudaStream_t st) {
     if (max_sr > 0) k_pro_tables<<<dim3(max_sr, nq), 256, 0, st>>>(net, d_qs, nq);
     k_pro_finish<<<nq, 256, 0, st>>>(net, d_qs, nq);
 }

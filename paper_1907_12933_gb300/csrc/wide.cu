@@ -1030,6 +1030,8 @@ void wide_work_free(WideWork& w) {
     w.chunk = 0;
 }
 
+void wide_done(QueryView* d_q, cudaStream_t st) { k_wide_work_done<<<1, 1, 0, st>>>(d_q); }
+
 vbmc_status wide_run(const WideNet& wn, int type, WideWork& w, const NetView& v, QueryView* d_q,
                      const QueryView& hq, unsigned long long lo, unsigned long long hi, unsigned long long* d_qcount,
                      QEntry* const* d_queue, unsigned long long cap, int n_sm, cudaStream_t st) {
@@ -1038,15 +1040,6 @@ vbmc_status wide_run(const WideNet& wn, int type, WideWork& w, const NetView& v,
     Queue q32{d_queue[1], d_qcount + 1, cap};
     Queue qdf{d_queue[2], d_qcount + 2, cap};
     Queue q64{d_queue[3], d_qcount + 3, cap};
-    // the folded net (fold.cu) checks the query where its set-up built one: the
-    // chunks, which clear a workspace each, are then not started
-    if (hq.fold) {
-        int fst = 0;
-        if (cudaMemcpyAsync(&fst, hq.fst, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return VBMC_ERR_CUDA;
-        if (fst) hi = lo;
-    }
     // the query's error flags (for waits that gave up) live in its counters
     unsigned int* err = &hq.cnt->err;
     for (unsigned long long c0 = lo; c0 < hi; c0 += w.chunk) {
@@ -1066,7 +1059,7 @@ vbmc_status wide_run(const WideNet& wn, int type, WideWork& w, const NetView& v,
         launch_df(v, d_q, 1, d_queue[2], d_qcount + 2, cap, q64, 3, n_sm, st);
         launch_fp64(v, d_q, 1, d_queue[3], d_qcount + 3, cap, 0, 0, n_sm, st);
     }
-    k_wide_work_done<<<1, 1, 0, st>>>(d_q);
+    wide_done(d_q, st);
     return cudaGetLastError() == cudaSuccess ? VBMC_OK : VBMC_ERR_CUDA;
 }
 

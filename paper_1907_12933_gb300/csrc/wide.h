@@ -88,7 +88,10 @@ struct WideTrace {
 };
 void wide_set_trace(const WideTrace* t);
 
-// Screen [lo, hi) of query d_q[0] (hq: its host copy) chunk by chunk, nothing where it folded. Each chunk's undecided points
+// The query's one unit of work (time to verdict) is done.
+void wide_done(QueryView* d_q, cudaStream_t st);
+
+// Screen [lo, hi) of query d_q[0] (hq: its host copy) chunk by chunk. Each chunk's undecided points
 // go through the FP32 (queue level 1), double-float (2) and FP64 (3) passes
 // before the next chunk starts; the queue counters are reset per chunk.
 vbmc_status wide_run(const WideNet& wn, int type, WideWork& w, const NetView& v, QueryView* d_q, const QueryView& hq,
