@@ -165,6 +165,8 @@ struct vbmc_result {
     // of a batch, whose views and counters lie in the arena)
     uint8_t* h_in = nullptr;
     uint8_t* d_in = nullptr;
+    uint8_t* d_group = nullptr;   // tile groups of vbmc_search_query (kGr*; with folded nets)
+    uint8_t* h_group = nullptr;   // pinned
     uint32_t* h_masks = nullptr;  // pinned: the coverage masks on their way out
     unsigned long long ntiles = 0;          // first-pass tiles of the last call
     int tile_pts = 0;                       // points per first-pass tile (0: no claim counter)
@@ -340,6 +342,18 @@ constexpr size_t kInTp = (sizeof(QueryView) + 15) & ~size_t(15);
 constexpr size_t kInPix = kInTp + 2 * sizeof(unsigned long long);
 constexpr size_t kInImage = kInPix + sizeof(int) * kMaxS;
 
+// A group of tiles of a search on a folded net is one launch of at most kGroupTiles
+// views, which share the query's set-up and count each for itself. A group has at most
+// kGroupPoints points: what lies behind the first witness is checked for nothing, and
+// that many points take about as long (75 us at the 57 points per ns of 784-512-512-10)
+// as the launches and the wait of one tile (65 us), so a group costs at most about one
+// tile more than its tiles one by one.
+constexpr int kGroupTiles = 64;
+constexpr uint64_t kGroupPoints = 1ull << 22;
+constexpr size_t kGrTp = (sizeof(QueryView) * kGroupTiles + 15) & ~size_t(15);
+constexpr size_t kGrCnt = kGrTp + sizeof(unsigned long long) * (kGroupTiles + 2);
+constexpr size_t kGrBytes = kGrCnt + sizeof(Counters) * kGroupTiles;
+
 size_t mask_bytes(const NetView& v) { return 8 * ((size_t)v.flip_words + (size_t)v.ss_words); }
 
 vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena* arena, int slot,
@@ -385,6 +399,8 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
             r->d_qcount = r->d_claim + 2;
         }
     }
+    const bool groups = !arena && fold_supported(v);
+    if (groups) A(&r->d_group, kGrBytes);
     A(&q.pix, (size_t)S);
     A(&q.dv, (size_t)S * RM);
     A(&q.ub, T);
@@ -447,6 +463,7 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
     if (!arena) {
         if (e == cudaSuccess) e = cudaMallocHost((void**)&r->h_in, kInImage + (size_t)v.dims[0]);
         if (e == cudaSuccess) e = cudaMallocHost((void**)&r->h_masks, mask_bytes(v));
+        if (groups && e == cudaSuccess) e = cudaMallocHost((void**)&r->h_group, kGrBytes);
     }
     if (e == cudaSuccess) e = cudaEventCreate(&r->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&r->ev1);
@@ -558,6 +575,7 @@ extern "C" vbmc_status vbmc_result_free(vbmc_result* r) {
     arena_release(r->arena);
     if (r->h_cnt) cudaFreeHost(r->h_cnt);
     if (r->h_in) {  // not a member of a batch
+        if (r->h_group) cudaFreeHost(r->h_group);
         cudaFreeHost(r->h_in);
         if (r->h_masks) cudaFreeHost(r->h_masks);
     }
@@ -620,7 +638,7 @@ enum { STAGE_SETUP = 1, STAGE_PASSES = 2, STAGE_ALL = 3 };
 // stage resets the counters and clears the masks and the verdict bitmap over
 // [0, hi); everything else it computes depends on the box, not on [lo, hi),
 // so one set-up over the whole space serves passes over any sub-ranges.
-// h_folded (pinned; one query): the call may wait for the set-up, so it learns here
+// h_folded (pinned; one query, or its set-up's answer for some tiles of it): the call may wait for the set-up, so it learns here
 // whether the query folded and launches the passes of that form only. Without it both
 // forms are launched and each leaves the other's queries out (about 20 us of launches
 // that return at once).
@@ -648,8 +666,9 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
     const bool wide = opt.precision == VBMC_PREC_FP8 || (tensor16 && !tc_supported(v, opt.precision));
     const bool tensor = tensor16 && !wide;
     const int wtype = wide_type(opt.precision);
+    const bool group = nq > 1 && !(stages & STAGE_SETUP) && h_folded && *h_folded;
     if (wide && any) {
-        if (nq != 1 || !ww) return fail(VBMC_ERR_UNSUPPORTED, "the wide-layer tensor screen serves one query per call");
+        if ((nq != 1 && !group) || !ww) return fail(VBMC_ERR_UNSUPPORTED, "the wide-layer tensor screen serves one query per call");
         if (!wide_supported(v))
             return fail(VBMC_ERR_UNSUPPORTED,
                         "tensor-core screen does not support this net/precision (wide layers: ReLU, hidden widths "
@@ -686,6 +705,9 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
             general = !fold;
         }
         if (general) launch_prologue_screens(v, d_qs, nq, max_sr, st);
+    } else if (fold && any && h_folded) {  // a tile or a group of tiles of one query
+        fold = *h_folded != 0;
+        general = !fold;
     } else if (wide && fold && any) {
         int here = 0;
         VB_CUDA(cudaMemcpyAsync(&here, hq[0].fst, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -718,15 +740,16 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
         // tiles as in the general first pass; the wide-layer path has none, and its
         // work count is one unit, which its own run takes away
         const int mt = opt.precision == VBMC_PREC_FP32 ? simt_tile_points(v) : tc_tile_points();
-        if (wide) ntiles = (hq[0].hi - (hq[0].lo & ~31ull) + mt - 1) / mt;
-        launch_fold(v, d_qs, nq, wide ? nullptr : d_tp, ntiles, mt, !wide, wide || !d_claim ? nullptr : d_claim + 1,
+        const bool whole = wide && nq == 1;
+        if (whole) ntiles = (hq[0].hi - (hq[0].lo & ~31ull) + mt - 1) / mt;
+        launch_fold(v, d_qs, nq, whole ? nullptr : d_tp, ntiles, mt, !wide, whole || !d_claim ? nullptr : d_claim + 1,
                     qsplit, 0, net->n_sm, st);
         launch_fold64(v, d_qs, d_queue[0], d_qcount + 0, cap, q64, 3, net->n_sm, st);
         if (!general) {
             VB_CUDA(record(ev[2]));
             VB_CUDA(record_rest());
             launch_fp64(v, d_qs, nq, d_queue[3], d_qcount + 3, cap, 0, 0, net->n_sm, st);
-            if (wide) wide_done(d_qs, st);
+            if (whole) wide_done(d_qs, st);
         }
     }
     if (!general) {
@@ -1466,8 +1489,10 @@ extern "C" vbmc_status vbmc_search_query(vbmc_net* net, const vbmc_query* q, int
     VB_CUDA(cudaMemcpyAsync(res->d_q, &qv, sizeof(QueryView), cudaMemcpyHostToDevice, sq));
     const cudaEvent_t ev_set[7] = {res->ev0,    res->ev_pro, res->ev_pro, res->ev_pro,
                                    res->ev_pro, res->ev_pro, res->ev_pro};
+    int* const h_folded = reinterpret_cast<int*>(res->h_claim + 1);
+    *h_folded = 0;
     st = enqueue_passes(net, res->d_q, &qv, 1, res->d_tp, tp[1], res->d_qcount, res->d_queue, cap, ev_set,
-                        *opt, sq, false, STAGE_SETUP, &res->ww, res->have_tw ? &res->tw : nullptr);
+                        *opt, sq, false, STAGE_SETUP, &res->ww, res->have_tw ? &res->tw : nullptr, nullptr, h_folded);
     if (st != VBMC_OK) return st;
     const cudaEvent_t ev_tile[7] = {res->ev_scr, res->ev_scr, res->ev_scr, res->ev1,
                                     res->ev_scr, res->ev_scr, res->ev_scr};
@@ -1475,9 +1500,83 @@ extern "C" vbmc_status vbmc_search_query(vbmc_net* net, const vbmc_query* q, int
     vbmc_search_out so{0, -1, 0, 0.0};
     vbmc_status run = VBMC_OK;
     bool any_tile = false;
-    for (int i = 0; i < n_tiles; ++i) {
-        const uint64_t lo = (uint64_t)order[i] * tsize;
-        const uint64_t hi = std::min<uint64_t>(n, lo + tsize);
+    // A folded query's tiles go in groups, 1, 4, 16, ... of them, where nothing but the
+    // counters is asked for. They add up, in order, to those of the tiles one by one; from
+    // a tile with ties (they share a list) or an overflow on, the tiles go one by one.
+    bool grouped = res->h_group && *h_folded && !opt->coverage && !opt->bitmap;
+    if (grouped) {
+        VB_CUDA(cudaMemcpyAsync(res->h_cnt, res->d_cnt, sizeof(Counters), cudaMemcpyDeviceToHost, sq));
+        VB_CUDA(cudaStreamSynchronize(sq));
+        grouped = counters_status(*res->h_cnt) == VBMC_OK;
+    }
+    auto tile_lo = [&](int i) { return (uint64_t)order[i] * tsize; };
+    auto tile_hi = [&](int i) { return std::min<uint64_t>(n, tile_lo(i) + tsize); };
+    int first = 0;  // first tile that no group has checked
+    for (int want = 1; grouped && first < n_tiles && so.witness_tile < 0; want = std::min(want * 4, kGroupTiles)) {
+        QueryView* const gq = reinterpret_cast<QueryView*>(res->h_group);
+        unsigned long long* const gtp = reinterpret_cast<unsigned long long*>(res->h_group + kGrTp);
+        Counters* const gc = reinterpret_cast<Counters*>(res->h_group + kGrCnt);
+        Counters zero = *res->h_cnt;
+        zero.n_adv = zero.n_ties = zero.n_points = 0;
+        zero.first = ~0ull;
+        for (unsigned long long& x : zero.n_q) x = 0;
+        const int mt = opt->precision == VBMC_PREC_FP32 ? simt_tile_points(net->v) : tc_tile_points();
+        int m = 0, end = first;
+        uint64_t points = 0;
+        gtp[0] = 0;
+        for (; end < n_tiles && m < want; ++end) {
+            const uint64_t lo = tile_lo(end), hi = tile_hi(end);
+            if (lo >= hi) continue;
+            if (m && points + (hi - lo) > kGroupPoints) break;
+            points += hi - lo;
+            gq[m] = qv;
+            gq[m].lo = lo;
+            gq[m].hi = hi;
+            gq[m].qid = m;
+            gq[m].cnt = reinterpret_cast<Counters*>(res->d_group + kGrCnt) + m;
+            gq[m].ties_cap = 0;
+            gc[m] = zero;
+            gq[m].ntiles = (hi - (lo & ~31ull) + mt - 1) / mt;
+            gtp[m + 1] = gtp[m] + gq[m].ntiles;
+            ++m;
+        }
+        if (m) {
+            VB_CUDA(cudaMemcpyAsync(res->d_group, res->h_group, kGrBytes, cudaMemcpyHostToDevice, sq));
+            st = enqueue_passes(net, reinterpret_cast<QueryView*>(res->d_group), gq, m,
+                                reinterpret_cast<unsigned long long*>(res->d_group + kGrTp), gtp[m], res->d_qcount,
+                                res->d_queue, cap, ev_tile, *opt, sq, false, STAGE_PASSES, &res->ww, nullptr,
+                                res->d_claim, h_folded);
+            if (st != VBMC_OK) return st;
+            any_tile = true;
+            VB_CUDA(cudaMemcpyAsync(gc, res->d_group + kGrCnt, sizeof(Counters) * m, cudaMemcpyDeviceToHost, sq));
+            VB_CUDA(cudaStreamSynchronize(sq));
+        }
+        for (int j = 0; first < end; ++first) {
+            if (tile_lo(first) < tile_hi(first)) {
+                const Counters& c = gc[j++];
+                if (c.err || c.n_ties) {
+                    grouped = false;
+                    break;
+                }
+                Counters& all = *res->h_cnt;
+                all.n_adv += c.n_adv;
+                all.first = std::min(all.first, c.first);
+                all.n_points += c.n_points;
+                for (int l = 0; l < 4; ++l) all.n_q[l] += c.n_q[l];
+                so.points_checked += tile_hi(first) - tile_lo(first);
+            }
+            so.tiles_checked += 1;
+            if (res->h_cnt->n_adv) {
+                so.witness_tile = order[first];
+                break;
+            }
+        }
+    }
+    if (first > 0 || any_tile)  // the tiles below and the result's getters add to these
+        VB_CUDA(cudaMemcpyAsync(res->d_cnt, res->h_cnt, sizeof(Counters), cudaMemcpyHostToDevice, sq));
+    for (int i = first; i < n_tiles && so.witness_tile < 0; ++i) {
+        const uint64_t lo = tile_lo(i);
+        const uint64_t hi = tile_hi(i);
         so.tiles_checked += 1;
         if (lo >= hi) continue;
         qv.lo = lo;
@@ -1487,7 +1586,8 @@ extern "C" vbmc_status vbmc_search_query(vbmc_net* net, const vbmc_query* q, int
         VB_CUDA(cudaMemcpyAsync(res->d_tp, tp.data(), sizeof(unsigned long long) * 2, cudaMemcpyHostToDevice,
                                 sq));
         st = enqueue_passes(net, res->d_q, &qv, 1, res->d_tp, tp[1], res->d_qcount, res->d_queue, cap, ev_tile,
-                            *opt, sq, false, STAGE_PASSES, &res->ww, res->have_tw ? &res->tw : nullptr);
+                            *opt, sq, false, STAGE_PASSES, &res->ww, res->have_tw ? &res->tw : nullptr, nullptr,
+                            h_folded);
         if (st != VBMC_OK) return st;
         any_tile = true;
         VB_CUDA(cudaMemcpyAsync(res->h_cnt, res->d_cnt, sizeof(Counters), cudaMemcpyDeviceToHost, sq));

@@ -204,3 +204,50 @@ def test_covered_fraction_of_dense_and_sparse_masks(vb, dims):
         assert vb.lib().vbmc_covered_fraction(vnet.h, 0, m.ctypes.data_as(C.POINTER(C.c_uint32)), C.byref(f)) == 0
         assert f.value == oracle.ss_covered_fraction(dims, m)
     vnet.free()
+
+
+@pytest.mark.parametrize("prec,dims,s,k,tiles,extra", [
+    ("bf16", [64, 64, 64, 10], 3, 12, 64, {}),
+    ("bf16", [64, 64, 64, 10], 3, 12, 257, {"queue_cap": 40}),
+    ("fp32", [40, 70, 33, 5], 5, 3, 100, {"filter": 3, "l2_max": 20}),
+    ("fp32", [40, 70, 33, 5], 2, 5, 300, {"threshold": 0.0}),
+    ("fp8", [784, 256, 256, 10], 3, 6, 33, {}),
+    ("bf16", [784, 512, 512, 10], 5, 10, 7, {}),
+])
+@pytest.mark.parametrize("ties", [False, True])
+def test_tile_groups_of_a_search(vb, prec, dims, s, k, tiles, extra, ties):
+    """Searches whose tiles go in groups against the same tiles one by one (a search that
+    asks for coverage) and against the general passes: orders with the witness early,
+    late and nowhere, tiles that straddle words, more tiles than points, queues that
+    overflow in a group, ties, filters; and calls after it add nothing to its counters."""
+    net = synth.make_net(821, dims, "relu", 2.0, "normal")
+    q = synth.make_query(821, 4, dims[0], s, k)
+    extra = dict(extra)
+    cap = extra.pop("queue_cap", 1 << 20)
+    if ties:  # an output equal to the decided one everywhere: every point is a margin tie
+        if oracle.space_size(s, k) > 20000 or extra.get("threshold") is not None:
+            pytest.skip("a tie at every point")
+        D = oracle.eval_point(net, q, 0)["D"]
+        net["W"][-1][(D + 1) % dims[-1]] = net["W"][-1][D]
+        net["b"][-1][(D + 1) % dims[-1]] = net["b"][-1][D]
+    vnet = vb.Net(net)
+    res = vb.Result(vnet, max_s=s, max_k=k, queue_cap=cap)
+    rng = np.random.default_rng(821)
+    keys = ("verdict", "n_points", "n_adversarial", "first_witness", "n_ties", "tiles_checked",
+            "points_checked", "witness_tile", "base_label")
+
+    def run(order, **kw):
+        try:
+            r = vb.search_query(vnet, res, q["image"], q["pixels"], k, order, precision=prec, **extra, **kw)
+        except vb.VbmcError as e:
+            return type(e), str(e)
+        at = vb.get_witness(res, s, dims[0])["index"] if r["n_adversarial"] else None
+        return [r.get(x) for x in keys] + [at, sorted(vb.get_ties(res))]
+
+    for order in (np.arange(tiles), np.arange(tiles)[::-1], rng.permutation(tiles)):
+        got = run(order)
+        assert got == run(order, coverage=True)
+        if cap == 1 << 20:
+            vb.set_folding(vnet, False)
+            assert got == run(order)
+            vb.set_folding(vnet, True)
