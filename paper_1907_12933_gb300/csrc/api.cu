@@ -169,6 +169,7 @@ struct vbmc_result {
     uint8_t* h_group = nullptr;   // pinned
     uint32_t* h_masks = nullptr;  // pinned: the coverage masks on their way out
     unsigned long long ntiles = 0;          // first-pass tiles of the last call
+    bool one_form = false;                  // the last call launched the folded passes only
     int tile_pts = 0;                       // points per first-pass tile (0: no claim counter)
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_pro = nullptr, ev_scr = nullptr;
     cudaEvent_t ev_split = nullptr, ev_f32 = nullptr, ev_df = nullptr;  // after each recheck pass
@@ -745,9 +746,8 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
         launch_fold(v, d_qs, nq, whole ? nullptr : d_tp, ntiles, mt, !wide, whole || !d_claim ? nullptr : d_claim + 1,
                     qsplit, 0, net->n_sm, st);
         launch_fold64(v, d_qs, d_queue[0], d_qcount + 0, cap, q64, 3, net->n_sm, st);
-        if (!general) {
+        if (!general) {  // (the passes in between take no time, see finish)
             VB_CUDA(record(ev[2]));
-            VB_CUDA(record_rest());
             launch_fp64(v, d_qs, nq, d_queue[3], d_qcount + 3, cap, 0, 0, net->n_sm, st);
             if (whole) wide_done(d_qs, st);
         }
@@ -883,10 +883,13 @@ vbmc_status enqueue(vbmc_net* net, vbmc_result* r, const uint8_t* d_image, const
         VB_CUDA(cudaMemcpyAsync(r->d_tp, tp.data(), sizeof(unsigned long long) * 2, cudaMemcpyHostToDevice, st));
     }
     const cudaEvent_t ev[7] = {r->ev0, r->ev_pro, r->ev_scr, r->ev1, r->ev_split, r->ev_f32, r->ev_df};
+    int* const h_folded = wait ? reinterpret_cast<int*>(r->h_claim + 1) : nullptr;
+    if (h_folded) *h_folded = 0;
     vbmc_status sst = enqueue_passes(net, r->d_q, &q, 1, r->d_tp, tp[1], r->d_qcount, r->d_queue,
                                      std::max<uint64_t>(1, r->caps.queue_cap), ev, opt, st, false, STAGE_ALL,
                                      &r->ww, r->have_tw ? &r->tw : nullptr, claims ? r->d_claim : nullptr,
-                                     wait ? reinterpret_cast<int*>(r->h_claim + 1) : nullptr);
+                                     h_folded);
+    r->one_form = h_folded && *h_folded;
     if (sst != VBMC_OK) {
         if (r->h_in) cudaStreamSynchronize(st);  // the pinned block has been read
         return sst;
@@ -964,10 +967,12 @@ vbmc_status finish(vbmc_result* r) {
         cudaEventElapsedTime(&ms_p, r->ev0, r->ev_pro);
         cudaEventElapsedTime(&ms_s, r->ev_pro, r->ev_scr);
         float mp[4] = {0.f, 0.f, 0.f, 0.f};
-        cudaEventElapsedTime(&mp[0], r->ev_scr, r->ev_split);
-        cudaEventElapsedTime(&mp[1], r->ev_split, r->ev_f32);
-        cudaEventElapsedTime(&mp[2], r->ev_f32, r->ev_df);
-        cudaEventElapsedTime(&mp[3], r->ev_df, r->ev1);
+        if (!r->one_form) {
+            cudaEventElapsedTime(&mp[0], r->ev_scr, r->ev_split);
+            cudaEventElapsedTime(&mp[1], r->ev_split, r->ev_f32);
+            cudaEventElapsedTime(&mp[2], r->ev_f32, r->ev_df);
+        }
+        cudaEventElapsedTime(&mp[3], r->one_form ? r->ev_scr : r->ev_df, r->ev1);
         (void)cudaGetLastError();  // timing is informative only
         fill_summary(r, *r->h_cnt, ms, ms_p, ms_s, mp);
         r->last_status = counters_status(*r->h_cnt);

@@ -81,6 +81,17 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
     return t;
 }
 
+// Kernels launched by launch_chained (launch.h) start while the kernel before them in
+// the stream still runs: chain_wait returns when that one has finished and its writes
+// are visible; chain_next, after it, lets the kernel behind start (without it that one
+// starts when this one's blocks leave). Nothing but the net's constants is touched
+// before chain_wait, and what the kernel before writes is not behind a __restrict__ pointer (a
+// load known to be invariant may move across it).
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 enum { FILTER_L2 = 1, FILTER_SHELL = 2 };
 enum { PROP_ARGMAX = 0, PROP_THRESHOLD = 1 };
 

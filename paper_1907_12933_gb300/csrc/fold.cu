@@ -101,6 +101,8 @@ __global__ void __launch_bounds__(256) k_fold_pack(NetView net, QueryView* qs, u
     __shared__ float eh[kFoldMax], eh64[kFoldMax], em_s[8], et_s[8];  // *_s: the warps' largest
     __shared__ int D_s, nv_s;
     __shared__ unsigned signs_s;
+    chain_wait();
+    chain_next();
     QueryView& Q = qs[blockIdx.x];
     if (!Q.fold || Q.fst[1] || (Q.cnt->err & DERR_PIXELS)) {
         if (threadIdx.x == 0 && unfolded) atomicAdd(unfolded, 1ull);
@@ -598,6 +600,7 @@ __global__ void __launch_bounds__(FT, 2) k_fold(NetView net, const QueryView* __
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FoldSm& S = *reinterpret_cast<FoldSm*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    chain_wait();  // (no chain_next: waiting blocks of k_fold64 take shared memory from this kernel's L1)
     if (nq == 1 && !folded(qs[0])) return;
     int cur = -1;
     bool small = true;
@@ -807,12 +810,13 @@ __device__ bool fold64_point(const NetView& net, const QueryView& Q, Fold64& F, 
 
 // Points k_fold left undecided.
 __global__ void __launch_bounds__(32 * F64W) k_fold64(NetView net, const QueryView* __restrict__ qs,
-                                                      const QEntry* __restrict__ in,
-                                                      const unsigned long long* __restrict__ count,
+                                                      const QEntry* in, const unsigned long long* count,
                                                       unsigned long long cap, Queue out, int out_level) {
     __shared__ Fold64 Fs[F64W];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Fold64& F = Fs[warp];
+    chain_wait();
+    chain_next();
     unsigned long long n = *count;
     if (n > cap) n = cap;
     const int L = net.L, offL = net.noff[L], HL = net.dims[L];
@@ -898,7 +902,7 @@ size_t fold_coeff_entries(const NetView& net, int max_s) {
 }
 
 void launch_fold_pack(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long* d_unfolded) {
-    k_fold_pack<<<nq, 256, 0, st>>>(net, d_qs, d_unfolded);
+    launch_chained(k_fold_pack, nq, 256, 0, st, net, d_qs, d_unfolded);
 }
 
 void launch_fold(const NetView& net, const QueryView* d_qs, int nq, const unsigned long long* d_tile_prefix,
@@ -914,13 +918,13 @@ void launch_fold(const NetView& net, const QueryView* d_qs, int nq, const unsign
     unsigned long long grid = nq == 1 ? (n_tiles * (unsigned)mt + 95) / 96 : (n_tiles + group - 1) / group;
     if (grid > ctas) grid = ctas;
     if (grid < 1) grid = 1;
-    k_fold<<<(unsigned)grid, FT, sizeof(FoldSm), st>>>(net, d_qs, nq, d_tile_prefix, n_tiles, mt, (int)group,
-                                                       work_units ? 1 : 0, claim, out, out_level);
+    launch_chained(k_fold, (unsigned)grid, FT, sizeof(FoldSm), st, net, d_qs, nq, d_tile_prefix, n_tiles, mt,
+                   (int)group, work_units ? 1 : 0, claim, out, out_level);
 }
 
 void launch_fold64(const NetView& net, const QueryView* d_qs, const QEntry* in, const unsigned long long* count,
                    unsigned long long cap, Queue out, int out_level, int n_sm, cudaStream_t st) {
-    k_fold64<<<(unsigned)n_sm * 4, 32 * F64W, 0, st>>>(net, d_qs, in, count, cap, out, out_level);
+    launch_chained(k_fold64, (unsigned)n_sm * 4, 32 * F64W, 0, st, net, d_qs, in, count, cap, out, out_level);
 }
 
 void launch_fold_margin(const NetView& net, const QueryView* d_qs, unsigned long long t, double* d_out,

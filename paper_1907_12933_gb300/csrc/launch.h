@@ -6,6 +6,25 @@
 
 namespace vbmc {
 
+// A launch that may start before the kernel in front of it has finished; the kernel
+// begins with chain_wait (dev.cuh). The set-up and the passes of a folded query are a
+// chain of short kernels: launch latency and the loads of their constants overlap.
+template <class... P, class... A>
+inline void launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... a) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, k, static_cast<P>(a)...);
+}
+
+
 // FP64 base pass for nq queries (d_qs on device). max_hi: max over queries of the
 // verdict bitmaps' bits (0: off). fold: some view has its fold flag set, their folded
 // nets are packed; *d_unfolded (optional) then gains the queries that did not fold.

@@ -19,6 +19,8 @@
 namespace vbmc {
 
 __global__ void k_pro_init(NetView net, QueryView* qs, int nq) {
+    chain_wait();
+    chain_next();
     QueryView& Q = qs[blockIdx.x];
     const int H0 = net.dims[0];
     if (blockIdx.y == 0 && threadIdx.x < 32) {
@@ -122,12 +124,17 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
     __shared__ float2 part[8][32];
     __shared__ double pdot[8];
     __shared__ float psum[8][4];
-    const QueryView& Q = qs[blockIdx.y];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wn = warp % WPN;  // warp of its neuron
     const int i = blockIdx.x * NPB + warp / WPN;
     const int tn = 32 * wn + lane, step = 32 * WPN;
     const int K = net.dims[l - 1], N = net.dims[l];
+    if (blockIdx.y == 0 && i < N)  // the row of W_l comes in while the layer below is at work
+        for (int j = 32 * tn; j < K; j += 32 * step)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(net.W[l] + (size_t)i * K + j));
+    chain_wait();
+    chain_next();
+    const QueryView& Q = qs[blockIdx.y];
     const int offp = l >= 2 ? net.noff[l - 1] : 0;
     const bool fold = Q.fold != 0;
     int npos = 0, nnode = 0, nb = 0;  // the layer below: "pos" neurons, nodes; nodes of the layers below it
@@ -462,6 +469,8 @@ __global__ void k_pro_finish(NetView net, QueryView* qs, int nq) {
 // Time to verdict of queries whose work count never reached zero inside a pass
 // (no screen tiles: empty ranges and the FP64-only path): the end of the last pass.
 __global__ void k_stamp_final(QueryView* qs, int nq) {
+    chain_wait();
+    chain_next();
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= nq) return;
     Counters* c = qs[q].cnt;
@@ -469,7 +478,7 @@ __global__ void k_stamp_final(QueryView* qs, int nq) {
 }
 
 void launch_stamp_final(QueryView* d_qs, int nq, cudaStream_t st) {
-    k_stamp_final<<<(nq + 127) / 128, 128, 0, st>>>(d_qs, nq);
+    launch_chained(k_stamp_final, (nq + 127) / 128, 128, 0, st, d_qs, nq);
 }
 
 // Blocks per query that clear the result buffers: one for the small masks, more
@@ -482,16 +491,16 @@ static unsigned clear_blocks(int nq, unsigned long long max_hi) {
 }
 
 void launch_pro_init(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long max_hi) {
-    k_pro_init<<<dim3((unsigned)nq, clear_blocks(nq, max_hi)), 256, 0, st>>>(net, d_qs, nq);
+    launch_chained(k_pro_init, dim3((unsigned)nq, clear_blocks(nq, max_hi)), 256, 0, st, net, d_qs, nq);
 }
 
 void launch_pro_layer(const NetView& net, QueryView* d_qs, int nq, int l, cudaStream_t st) {
     // eight warps per neuron for at least 256 inputs (one round of their lanes), until
     // the queries alone put about 16 warps on every SM
     if (net.dims[l - 1] >= 256 && (long long)nq * net.dims[l] <= 2432)
-        k_pro_layer<8><<<dim3(net.dims[l], nq), 256, 0, st>>>(net, d_qs, nq, l);
+        launch_chained(k_pro_layer<8>, dim3(net.dims[l], nq), 256, 0, st, net, d_qs, nq, l);
     else
-        k_pro_layer<1><<<dim3((net.dims[l] + 7) / 8, nq), 256, 0, st>>>(net, d_qs, nq, l);
+        launch_chained(k_pro_layer<1>, dim3((net.dims[l] + 7) / 8, nq), 256, 0, st, net, d_qs, nq, l);
 }
 
 void launch_prologue(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long max_hi,
