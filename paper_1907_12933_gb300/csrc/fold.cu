@@ -96,9 +96,14 @@ __device__ __forceinline__ double warp_max(double v) {
 // Base values of fill-up rows: a node that never crosses, a margin that never decides.
 constexpr float kNoNode = -1.f, kNoMargin = 1e30f;
 
-__global__ void __launch_bounds__(256) k_fold_pack(NetView net, QueryView* qs, unsigned long long* unfolded) {
+constexpr int kPackT = 512;
+
+// Barrier of n threads of a block.
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+__global__ void __launch_bounds__(kPackT) k_fold_pack(NetView net, QueryView* qs, unsigned long long* unfolded) {
     __shared__ FoldShape f;
-    __shared__ float eh[kFoldMax], eh64[kFoldMax], em_s[8], et_s[8];  // *_s: the warps' largest
+    __shared__ float eh[kFoldMax], eh64[kFoldMax], em_s[kPackT / 32], et_s[kPackT / 32];  // *_s: the warps' largest
     __shared__ int D_s, nv_s;
     __shared__ unsigned signs_s;
     chain_wait();
@@ -111,118 +116,137 @@ __global__ void __launch_bounds__(256) k_fold_pack(NetView net, QueryView* qs, u
     const int L = net.L, HL = net.dims[L], offL = net.noff[L], s = Q.s;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool eq11 = Q.prop == PROP_THRESHOLD, cov = Q.flip != nullptr;
-    if (warp == 0) {  // D: the largest output, the lowest index among equals; HL <= 32
-        const double y = lane < HL ? Q.ub[offL + lane] : -DBL_MAX;
-        const double top = warp_max(y);
-        const int D = __ffs(__ballot_sync(0xffffffffu, lane < HL && y == top)) - 1;
-        const double mx = warp_max(lane == D ? -DBL_MAX : y);
-        // outputs that can change their sign over the box
-        const bool cross = lane < HL && !(fabs(y) > ((double)Q.fbd[offL + lane] + (double)Q.fhe[offL + lane].y) *
-                                                            (1.0 + 1e-6) + 4.0 * kTau);
-        const unsigned signs = __ballot_sync(0xffffffffu, cov && cross);
-        if (lane == 0) {
-            D_s = D;
-            signs_s = signs;
-            nv_s = eq11 ? HL : __popc(signs);  // rows that are outputs
-            Q.cnt->D = D;
-            Q.cnt->base_margin = eq11 ? fmax(top - Q.V, Q.V - mx) : top - mx;
-            Q.fst[2 + L] = (eq11 ? 0 : (HL + 2) & ~3) + nv_s;
-            fold_shape(net, Q, f);
-        }
-    }
-    __syncthreads();
-    const int D = D_s, margins = f.margins;
-    const unsigned signs = signs_s;
-    if (warp == 0) {  // the outputs of the rows behind the margins; which of them have a sign test
-        const bool row = lane < HL && (eq11 || ((signs >> lane) & 1u));
-        const unsigned m = __ballot_sync(0xffffffffu, row);
-        if (row) Q.forow[__popc(m & ((1u << lane) - 1u))] = lane | (int)((signs >> lane) & 1u) << 8;
-    }
-    __syncthreads();
-    // coefficient pair k of row i of layer l (k = -1: base value)
-    auto coeff = [&](int l, int i, int k) -> float {
-        if (l == L && i < margins) {
-            const int o = i < D ? i : i + 1;
-            if (o >= HL) return k < 0 ? kNoMargin : 0.f;
-            if (k < 0) return (float)(Q.ub[offL + D] - Q.ub[offL + o]);
-            const float2 a = Q.fco[(size_t)(offL + D) * Q.fstride + k], b = Q.fco[(size_t)(offL + o) * Q.fstride + k];
-            return df_add(a, make_float2(-b.x, -b.y)).x;
-        }
-        if (i >= f.n[l]) return k < 0 ? kNoNode : 0.f;
-        const int nn = l < L ? Q.fnode[f.cb[l] + i] : offL + (Q.forow[i - margins] & 255);
-        const float c = k < 0 ? (float)Q.ub[nn] : Q.fco[(size_t)nn * Q.fstride + k].x;
-        return l < L && Q.fcls[nn] == 3 ? -c : c;
-    };
-    for (int e = threadIdx.x; e < f.entries; e += blockDim.x) {
-        int l = L;
-        while (e < f.off[l]) --l;  // layers without rows have the offset of the next one
-        const int cols = 1 + s + f.cb[l], g = (e - f.off[l]) / cols, k = e - f.off[l] - g * cols - 1;
-        Q.fc32[e] = make_float4(coeff(l, 4 * g, k), coeff(l, 4 * g + 1, k), coeff(l, 4 * g + 2, k),
-                                coeff(l, 4 * g + 3, k));
-    }
-    // error bounds (FP32, rounded up), layer by layer: a warp per row, its lanes over the
-    // sources; L + 1: the margins
+    // rows' errors (FP32, rounded up): a warp per row, its lanes over the sources; layer
+    // L + 1: the margins. Hidden rows depend on the layers below; outputs and margins on
+    // all of them. The first half of the warps does the hidden layers while the other one
+    // finds D and packs the coefficients: bound by the latency of dependent loads (one
+    // after the other: D 3 us, coefficients 5, errors 6 on 784-512-512-10).
     const float tau2 = __double2float_ru(2.0 * kTau);
     float em = 0.f, et = 0.f;
-    for (int l = 1; l <= L + (eq11 ? 0 : 1); ++l) {
-        const int cb = f.cb[l < L ? l : L], rows = l < L ? f.n[l] : (l == L ? HL : HL - 1);
-        for (int i = warp; i < rows; i += blockDim.x / 32) {
-            const int n1 = l < L ? Q.fnode[cb + i] : (l == L ? offL + out_of_row(i, D) : offL + D);
-            const int n2 = l <= L ? -1 : offL + (i < D ? i : i + 1);
-            const float2* r1 = Q.fco + (size_t)n1 * Q.fstride;
-            const float2* r2 = Q.fco + (size_t)(n2 < 0 ? n1 : n2) * Q.fstride;
-            float M = 0.f, pr = 0.f, pr64 = 0.f;
-            for (int k = lane; k < s + cb; k += 32) {
-                float2 c = r1[k];
-                if (n2 >= 0) c = df_add(c, make_float2(-r2[k].x, -r2[k].y));
-                const float w = abs_up(c);
-                if (k < s) {
-                    M = __fmaf_ru(w, Q.fx[k], M);
-                } else {
-                    M = __fmaf_ru(w, __fadd_ru(Q.fsb[Q.fnode[k - s]], eh[k - s]), M);
-                    pr = __fmaf_ru(w, eh[k - s], pr);
-                    pr64 = __fmaf_ru(w, eh64[k - s], pr64);
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                M = __fadd_ru(M, __shfl_xor_sync(0xffffffffu, M, o));
-                pr = __fadd_ru(pr, __shfl_xor_sync(0xffffffffu, pr, o));
-                pr64 = __fadd_ru(pr64, __shfl_xor_sync(0xffffffffu, pr64, o));
-            }
-            if (lane) continue;
-            double ub = Q.ub[n1];
-            float fer = Q.fer[n1], eub = Q.fhe[n1].y;
-            if (n2 >= 0) {
-                ub -= Q.ub[n2];
-                fer = __fadd_ru(fer, Q.fer[n2]);
-                eub = __fadd_ru(eub, Q.fhe[n2].y);
-            }
-            const float ub32 = (float)ub;
-            const float mag = __fadd_ru(__fadd_ru(fabsf(ub32), M), 1e-30f);
-            float e = __fadd_ru(__fmaf_ru((float)(s + cb + 8) * 0x1p-24f, mag, pr), __fadd_ru(fer, 1e-37f));
-            e = __fadd_ru(__fadd_ru(e, __double2float_ru(fabs((double)ub32 - ub))), eub);
-            const float e2 = __fadd_ru(e, tau2);
-            if (l > L) {
-                // only a margin that can come near 0 over the box has a say in the common bound
-                if (ub - (double)M - (double)e <= 1e-3) em = fmaxf(em, e2);
-                continue;
-            }
-            // the same in FP64 (u = 2^-53; x_p = dv_p / 255 rounds once, the rows' pairs are exact in it)
-            const float e64 = __fmaf_ru((float)(s + cb + 12) * 0x1p-53f, mag, __fadd_ru(pr64, __fadd_ru(fer, eub)));
-            Q.fe64[l < L ? cb + i : kFoldMax + i] = e64;
-            const float thr = fabs(ub) < kTau ? INFINITY : e2;  // a base tie: every sign is a tie
-            if (l < L) {
-                eh[cb + i] = e;
-                eh64[cb + i] = e64;
-                et = fmaxf(et, thr);
+    int D = 0;
+    unsigned signs = 0;
+    auto bound = [&](int l, int cb, int i) {
+        const int n1 = l < L ? Q.fnode[cb + i] : (l == L ? offL + out_of_row(i, D) : offL + D);
+        const int n2 = l <= L ? -1 : offL + (i < D ? i : i + 1);
+        const float2* r1 = Q.fco + (size_t)n1 * Q.fstride;
+        const float2* r2 = Q.fco + (size_t)(n2 < 0 ? n1 : n2) * Q.fstride;
+        float M = 0.f, pr = 0.f, pr64 = 0.f;
+        for (int k = lane; k < s + cb; k += 32) {
+            float2 c = r1[k];
+            if (n2 >= 0) c = df_add(c, make_float2(-r2[k].x, -r2[k].y));
+            const float w = abs_up(c);
+            if (k < s) {
+                M = __fmaf_ru(w, Q.fx[k], M);
             } else {
-                const int o = out_of_row(i, D);
-                Q.fk32[1 + o].y = e2;
-                if ((signs >> o) & 1u) et = fmaxf(et, thr);
+                M = __fmaf_ru(w, __fadd_ru(Q.fsb[Q.fnode[k - s]], eh[k - s]), M);
+                pr = __fmaf_ru(w, eh[k - s], pr);
+                pr64 = __fmaf_ru(w, eh64[k - s], pr64);
             }
         }
-        __syncthreads();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            M = __fadd_ru(M, __shfl_xor_sync(0xffffffffu, M, o));
+            pr = __fadd_ru(pr, __shfl_xor_sync(0xffffffffu, pr, o));
+            pr64 = __fadd_ru(pr64, __shfl_xor_sync(0xffffffffu, pr64, o));
+        }
+        if (lane) return;
+        double ub = Q.ub[n1];
+        float fer = Q.fer[n1], eub = Q.fhe[n1].y;
+        if (n2 >= 0) {
+            ub -= Q.ub[n2];
+            fer = __fadd_ru(fer, Q.fer[n2]);
+            eub = __fadd_ru(eub, Q.fhe[n2].y);
+        }
+        const float ub32 = (float)ub;
+        const float mag = __fadd_ru(__fadd_ru(fabsf(ub32), M), 1e-30f);
+        float e = __fadd_ru(__fmaf_ru((float)(s + cb + 8) * 0x1p-24f, mag, pr), __fadd_ru(fer, 1e-37f));
+        e = __fadd_ru(__fadd_ru(e, __double2float_ru(fabs((double)ub32 - ub))), eub);
+        const float e2 = __fadd_ru(e, tau2);
+        if (l > L) {
+            // only a margin that can come near 0 over the box has a say in the common bound
+            if (ub - (double)M - (double)e <= 1e-3) em = fmaxf(em, e2);
+            return;
+        }
+        // the same in FP64 (u = 2^-53; x_p = dv_p / 255 rounds once, the rows' pairs are exact in it)
+        const float e64 = __fmaf_ru((float)(s + cb + 12) * 0x1p-53f, mag, __fadd_ru(pr64, __fadd_ru(fer, eub)));
+        Q.fe64[l < L ? cb + i : kFoldMax + i] = e64;
+        const float thr = fabs(ub) < kTau ? INFINITY : e2;  // a base tie: every sign is a tie
+        if (l < L) {
+            eh[cb + i] = e;
+            eh64[cb + i] = e64;
+            et = fmaxf(et, thr);
+        } else {
+            const int o = out_of_row(i, D);
+            Q.fk32[1 + o].y = e2;
+            if ((signs >> o) & 1u) et = fmaxf(et, thr);
+        }
+    };
+    if (warp < kPackT / 64) {
+        int cb = 0;
+        for (int l = 1; l < L; ++l) {
+            const int rows = Q.fst[2 + l];
+            for (int i = warp; i < rows; i += kPackT / 64) bound(l, cb, i);
+            cb += rows;
+            bar_sync(1, kPackT / 2);
+        }
+    } else {
+        if (warp == kPackT / 64) {  // D: the largest output, the lowest index among equals; HL <= 32
+            const double y = lane < HL ? Q.ub[offL + lane] : -DBL_MAX;
+            const double top = warp_max(y);
+            D = __ffs(__ballot_sync(0xffffffffu, lane < HL && y == top)) - 1;
+            const double mx = warp_max(lane == D ? -DBL_MAX : y);
+            // outputs that can change their sign over the box
+            const bool cross = lane < HL && !(fabs(y) > ((double)Q.fbd[offL + lane] + (double)Q.fhe[offL + lane].y) *
+                                                                (1.0 + 1e-6) + 4.0 * kTau);
+            signs = __ballot_sync(0xffffffffu, cov && cross);
+            if (lane == 0) {
+                D_s = D;
+                signs_s = signs;
+                nv_s = eq11 ? HL : __popc(signs);  // rows that are outputs
+                Q.cnt->D = D;
+                Q.cnt->base_margin = eq11 ? fmax(top - Q.V, Q.V - mx) : top - mx;
+                Q.fst[2 + L] = (eq11 ? 0 : (HL + 2) & ~3) + nv_s;
+                fold_shape(net, Q, f);
+            }
+        }
+        bar_sync(2, kPackT / 2);
+        D = D_s;
+        signs = signs_s;
+        const int margins = f.margins;
+        if (warp == kPackT / 64) {  // the outputs of the rows behind the margins; which of them have a sign test
+            const bool row = lane < HL && (eq11 || ((signs >> lane) & 1u));
+            const unsigned m = __ballot_sync(0xffffffffu, row);
+            if (row) Q.forow[__popc(m & ((1u << lane) - 1u))] = lane | (int)((signs >> lane) & 1u) << 8;
+        }
+        bar_sync(2, kPackT / 2);
+        // coefficient pair k of row i of layer l (k = -1: base value)
+        auto coeff = [&](int l, int i, int k) -> float {
+            if (l == L && i < margins) {
+                const int o = i < D ? i : i + 1;
+                if (o >= HL) return k < 0 ? kNoMargin : 0.f;
+                if (k < 0) return (float)(Q.ub[offL + D] - Q.ub[offL + o]);
+                const float2 a = Q.fco[(size_t)(offL + D) * Q.fstride + k], b = Q.fco[(size_t)(offL + o) * Q.fstride + k];
+                return df_add(a, make_float2(-b.x, -b.y)).x;
+            }
+            if (i >= f.n[l]) return k < 0 ? kNoNode : 0.f;
+            const int nn = l < L ? Q.fnode[f.cb[l] + i] : offL + (Q.forow[i - margins] & 255);
+            const float c = k < 0 ? (float)Q.ub[nn] : Q.fco[(size_t)nn * Q.fstride + k].x;
+            return l < L && Q.fcls[nn] == 3 ? -c : c;
+        };
+        for (int e = threadIdx.x - kPackT / 2; e < f.entries; e += kPackT / 2) {
+            int l = L;
+            while (e < f.off[l]) --l;  // layers without rows have the offset of the next one
+            const int cols = 1 + s + f.cb[l], g = (e - f.off[l]) / cols, k = e - f.off[l] - g * cols - 1;
+            Q.fc32[e] = make_float4(coeff(l, 4 * g, k), coeff(l, 4 * g + 1, k), coeff(l, 4 * g + 2, k),
+                                    coeff(l, 4 * g + 3, k));
+        }
+    }
+    __syncthreads();
+    D = D_s;
+    signs = signs_s;
+    for (int i = warp; i < HL + (eq11 ? 0 : HL - 1); i += kPackT / 32) {
+        if (i < HL) bound(L, f.nodes, i);
+        else bound(L + 1, f.nodes, i - HL);
     }
     if (lane == 0) {
         em_s[warp] = em;
@@ -230,7 +254,7 @@ __global__ void __launch_bounds__(256) k_fold_pack(NetView net, QueryView* qs, u
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) {
+        for (int w = 1; w < kPackT / 32; ++w) {
             em = fmaxf(em, em_s[w]);
             et = fmaxf(et, et_s[w]);
         }
@@ -902,7 +926,7 @@ size_t fold_coeff_entries(const NetView& net, int max_s) {
 }
 
 void launch_fold_pack(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long* d_unfolded) {
-    launch_chained(k_fold_pack, nq, 256, 0, st, net, d_qs, d_unfolded);
+    launch_chained(k_fold_pack, nq, kPackT, 0, st, net, d_qs, d_unfolded);
 }
 
 void launch_fold(const NetView& net, const QueryView* d_qs, int nq, const unsigned long long* d_tile_prefix,

@@ -19,6 +19,11 @@
 namespace vbmc {
 
 __global__ void k_pro_init(NetView net, QueryView* qs, int nq) {
+    if (blockIdx.x == 0) {  // W_1 comes in meanwhile
+        const size_t n1 = (size_t)net.dims[0] * net.dims[1];
+        for (size_t j = 32 * ((size_t)blockIdx.y * blockDim.x + threadIdx.x); j < n1; j += 32 * (size_t)gridDim.y * blockDim.x)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(net.W[1] + j));
+    }
     chain_wait();
     chain_next();
     QueryView& Q = qs[blockIdx.x];
@@ -112,18 +117,23 @@ __device__ constexpr Grey kGrey;
 // are FP32 pairs (dfloat.cuh: 10 FP32 instructions against 32 cycles), bounds FP32.
 // Few queries leave most of the chip idle with one warp per neuron (an output layer
 // of 10 is 10 warps, each walking 512 inputs one load latency after the other), so
-// wide layers take eight; with many queries the warps come from them. The set-up of
-// one query (init, layers, pack, and the launches that return at once), before (a
-// warp per neuron, FP64 throughout) and after: 784-512-512-10 142 -> 70 us,
-// 784-1024x3-10 310 -> 147 us.
+// wide layers take eight and an output layer 32; with many queries the warps come from
+// them. One warp adds up its neuron's partial sums, the others go on to the columns
+// (every warp adding them up kept the FP64 pipe busy for 3 to 4 us of each layer).
+// The set-up of one query (init, layers, pack), at first (a warp per neuron, FP64
+// throughout), with eight warps, and now: 784-512-512-10 142 -> 73 -> 60 us,
+// 784-1024x3-10 310 -> 154 -> 106 us, 784-300-100-10 (80 ->) 51 us.
 template <int WPN>
-__global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, int nq, int l) {
-    constexpr int NPB = 8 / WPN;  // neurons per block
+__global__ void __launch_bounds__(32 * (WPN > 8 ? WPN : 8)) k_pro_layer(NetView net, QueryView* qs, int nq, int l) {
+    constexpr int NW = WPN > 8 ? WPN : 8;  // warps of a block
+    constexpr int NPB = NW / WPN;          // neurons per block
+    constexpr int LR = kMaxWidth / (32 * NW);  // rounds of the block's lanes over the widest layer
+    constexpr int PS = WPN > 1 ? WPN : 1;
     __shared__ short plist[kMaxWidth], clist[kFoldMax];
-    __shared__ int wpos[8], wnode[8];
-    __shared__ float2 part[8][32];
-    __shared__ double pdot[8];
-    __shared__ float psum[8][4];
+    __shared__ int wpos[NW], wnode[NW];
+    __shared__ float2 part[PS][32];
+    __shared__ double pdot[PS][32];
+    __shared__ float psum[4][PS][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wn = warp % WPN;  // warp of its neuron
     const int i = blockIdx.x * NPB + warp / WPN;
@@ -141,11 +151,11 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
     bool rows = fold;                 // false: more nodes than a folded net holds
     if (fold && l >= 2) {
         const unsigned char* cls = Q.fcls + offp;
-        unsigned mp[kMaxWidth / 256], mn[kMaxWidth / 256];
+        unsigned mp[LR], mn[LR];
         int cp = 0, cn = 0;
 #pragma unroll
-        for (int e = 0; e < kMaxWidth / 256; ++e) {
-            const int j = warp * (kMaxWidth / 8) + 32 * e + lane;
+        for (int e = 0; e < LR; ++e) {
+            const int j = 32 * (warp * LR + e) + lane;
             const int c = j < K ? cls[j] : 1;
             mp[e] = __ballot_sync(0xffffffffu, c == 0 || c == 3);
             mn[e] = __ballot_sync(0xffffffffu, c >= 2);
@@ -160,7 +170,7 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
         __syncthreads();
         int bp = 0, bn = 0;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) {
+        for (int w = 0; w < NW; ++w) {
             if (w < warp) {
                 bp += wpos[w];
                 bn += wnode[w];
@@ -171,8 +181,8 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
         rows = nb + nnode <= kFoldMax;  // the same for every block (and for the layers above)
         if (rows) {
 #pragma unroll
-            for (int e = 0; e < kMaxWidth / 256; ++e) {
-                const int j = warp * (kMaxWidth / 8) + 32 * e + lane;
+            for (int e = 0; e < LR; ++e) {
+                const int j = 32 * (warp * LR + e) + lane;
                 const unsigned below = (1u << lane) - 1u;
                 if ((mp[e] >> lane) & 1u) plist[bp + __popc(mp[e] & below)] = (short)j;
                 if ((mn[e] >> lane) & 1u) {
@@ -190,7 +200,7 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
         }
         __syncthreads();
     }
-    if (WPN == 1 && i >= N) return;  // (WPN == 8: one neuron per block, the grid has N)
+    if (WPN == 1 && i >= N) return;  // (else one neuron per block, the grid has N)
     const float* Wr = net.W[l] + (size_t)i * K;
     double dot = 0.0;
     float b[4] = {0.f, 0.f, 0.f, 0.f};  // sum |w h|, sum |w| e; of the carried rows: sum |w| fer, sum |w| B
@@ -235,35 +245,43 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
             }
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        dot += __shfl_xor_sync(0xffffffffu, dot, o);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) b[m] = __fadd_ru(b[m], __shfl_xor_sync(0xffffffffu, b[m], o));
-    }
-    if (WPN > 1) {
-        if (lane == 0) {
-            pdot[warp] = dot;
-#pragma unroll
-            for (int m = 0; m < 4; ++m) psum[warp][m] = b[m];
-        }
-        __syncthreads();
-        dot = 0.0;
-        b[0] = b[1] = b[2] = b[3] = 0.f;
-#pragma unroll
-        for (int w = 0; w < WPN; ++w) {
-            dot += pdot[w];
-#pragma unroll
-            for (int m = 0; m < 4; ++m) b[m] = __fadd_ru(b[m], psum[w][m]);
-        }
-    }
     const int n = net.noff[l] + i;
-    const float bias = net.b[l][i];
-    const double u = dot + (double)bias;
-    // (activations add 2^-50 |u|)
-    float eu = __fmul_ru((float)((K + step - 1) / step + 17) * 0x1p-53f, __fadd_ru(b[0], fabsf(bias)));
-    eu = __fmaf_ru(0x1p-50f, __double2float_ru(fabs(u)), __fadd_ru(eu, b[1]));
-    eu = __fmul_ru(eu, 1.f + 0x1p-20f);
+    double u = 0.0;
+    float eu = 0.f;
+    if (WPN > 1) {  // the neuron's first warp adds up, in 4 chains
+        pdot[wn][lane] = dot;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) psum[m][wn][lane] = b[m];
+        __syncthreads();
+        if (wn == 0) {
+            double d4[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) d4[c] = pdot[c % PS][lane];
+#pragma unroll
+            for (int w = 4; w < WPN; ++w) d4[w & 3] += pdot[w % PS][lane];
+            dot = (d4[0] + d4[1]) + (d4[2] + d4[3]);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                b[m] = psum[m][0][lane];
+#pragma unroll
+                for (int w = 1; w < WPN; ++w) b[m] = __fadd_ru(b[m], psum[m][w][lane]);
+            }
+        }
+    }
+    if (wn == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            dot += __shfl_xor_sync(0xffffffffu, dot, o);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) b[m] = __fadd_ru(b[m], __shfl_xor_sync(0xffffffffu, b[m], o));
+        }
+        const float bias = net.b[l][i];
+        u = dot + (double)bias;
+        // (activations add 2^-50 |u|)
+        eu = __fmul_ru((float)((K + step - 1) / step + 17) * 0x1p-53f, __fadd_ru(b[0], fabsf(bias)));
+        eu = __fmaf_ru(0x1p-50f, __double2float_ru(fabs(u)), __fadd_ru(eu, b[1]));
+        eu = __fmul_ru(eu, 1.f + 0x1p-20f);
+    }
     if (tn == 0) {
         const double h = (l < net.L) ? act64(net.act, u) : u;
         Q.ub[n] = u;
@@ -311,11 +329,16 @@ __global__ void __launch_bounds__(256) k_pro_layer(NetView net, QueryView* qs, i
                 a = df_add(a, make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o)));
             if (WPN > 1) {
                 __syncthreads();
-                part[warp][lane] = a;
+                part[wn][lane] = a;
                 __syncthreads();
-                a = part[0][lane];
+                if (wn == 0) {
+                    float2 a4[4];
 #pragma unroll
-                for (int w = 1; w < WPN; ++w) a = df_add(a, part[w][lane]);
+                    for (int c = 0; c < 4; ++c) a4[c] = part[c % PS][lane];
+#pragma unroll
+                    for (int w = 4; w < WPN; ++w) a4[w & 3] = df_add(a4[w & 3], part[w % PS][lane]);
+                    a = df_add(df_add(a4[0], a4[1]), df_add(a4[2], a4[3]));
+                }
             }
             if (wn == 0 && lane < sp && k < S) {
                 row[k] = a;
@@ -496,8 +519,12 @@ void launch_pro_init(const NetView& net, QueryView* d_qs, int nq, cudaStream_t s
 
 void launch_pro_layer(const NetView& net, QueryView* d_qs, int nq, int l, cudaStream_t st) {
     // eight warps per neuron for at least 256 inputs (one round of their lanes), until
-    // the queries alone put about 16 warps on every SM
-    if (net.dims[l - 1] >= 256 && (long long)nq * net.dims[l] <= 2432)
+    // the queries alone put about 16 warps on every SM; where the neurons alone leave
+    // most SMs empty (output layers of few queries) 32 of them, eight for few inputs
+    const long long neurons = (long long)nq * net.dims[l];
+    if (net.dims[l - 1] >= 256 && neurons <= 152)
+        launch_chained(k_pro_layer<32>, dim3(net.dims[l], nq), 1024, 0, st, net, d_qs, nq, l);
+    else if (neurons <= (net.dims[l - 1] >= 256 ? 2432 : 152))
         launch_chained(k_pro_layer<8>, dim3(net.dims[l], nq), 256, 0, st, net, d_qs, nq, l);
     else
         launch_chained(k_pro_layer<1>, dim3((net.dims[l] + 7) / 8, nq), 256, 0, st, net, d_qs, nq, l);
