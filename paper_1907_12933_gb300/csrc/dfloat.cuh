@@ -1,7 +1,7 @@
 // dfloat.cuh -- FP32 pairs (hi + lo) that stand for values of about 48 significant
-// bits, with the error bounds of df.cu: the double-float pass and the rows of folded
-// nets (prologue.cu) are computed in them, on a part that runs FP64 at a
-// sixty-fourth of its FP32 rate.
+// bits, with the error bounds of df.cu: the double-float pass, the rows of folded nets
+// (prologue.cu) and the potentials of the covers over pairs (pairs.cu) are computed in
+// them, on a part that runs FP64 at a sixty-fourth of its FP32 rate.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -24,6 +24,35 @@ __device__ __forceinline__ float2 split64(double v) {
     const float hi = (float)v;
     return make_float2(hi, (float)(v - (double)hi));
 }
+
+// Two FP32 lanes in one 64-bit register (fma.rn.f32x2: two results an instruction).
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(v));
+    return d;
+}
+
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, 0xBF800000BF800000ull, a); }  // a - b, rounded once
 
 __device__ __forceinline__ float abs_up(float2 a) { return __fmul_ru(fabsf(a.x), 1.f + 0x1p-22f); }
 

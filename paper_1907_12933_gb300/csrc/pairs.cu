@@ -180,16 +180,20 @@ __global__ void __launch_bounds__(TP) k_pairs(NetView net, const uint8_t* x1s, c
 // value ratio, distance) has to clear its threshold by the potentials' error bound,
 // else the CTA evaluates that pair in FP64 (k_pairs's own steps).
 //
-// A dot product against an anchor sigma = 1.5 2^M, 2^(M-1) >= ||W_i|| ||h|| (so that no
-// partial sum leaves the binade): t = fma(w, h, sigma); q = t - sigma, the product on
-// the grid 2^(M-23), summed exactly; r = fma(w, h, -q) its rest, summed plainly over 16
-// terms and then by two_sum. Per 16 terms the rests lose at most 136 2^(M-48), each
-// rest 2^(M-48); with 2^M < 4 ||W_i|| ||h||: |error| <= 5 (K + 16) 2^-45 ||W_i|| ||h||.
+// A dot product against an anchor: a starts at sigma = 1.5 2^M, 2^(M-1) >= (1 + K 2^-22)
+// ||W_i|| ||h||, so that no partial sum, the roundings included, leaves the binade
+// [2^M, 2^(M+1)]; a' = fma(w, h, a) then rounds to the grid 2^(M-23), a - a' is exact, and
+// r = fma(w, h, a - a') is what that step lost, summed plainly over 16 terms and then by
+// two_sum. Per 16 terms the rests lose at most 136 2^(M-48), each rest 2^(M-48); with
+// 2^M < 4 (1 + K 2^-22) ||W_i|| ||h||: |error| <= 5 (K + 16) 2^-45 ||W_i|| ||h||.
 // Layer 1 runs on the grey levels (exact in FP32) and divides by 255 as a pair.
 //
 // CTA = IB images (IB / 2 pairs), a thread per neuron: one weight load serves IB
-// images, whose activations are shared-memory broadcasts. Bound by FP32 issue. 8,192
-// pairs on 784-512-512-10: 55.3 -> 3.7 ms (0.40 -> 6.0 TFLOP/s of dot products).
+// images, whose activations are shared-memory broadcasts, high parts and low parts of
+// an input side by side so that two images make one f32x2 operand: 4 (layer 1) or 5
+// instructions for two multiply-adds. Bound by FP32 issue. 8,192 pairs on
+// 784-512-512-10: FP64 55.5 ms, one image an instruction and a sum of its own 3.95 ms,
+// now 3.45 ms (the kernel 2.87; its FMA pipe is 69 % busy, two cycles an f32x2).
 constexpr int TPD = 256;
 
 template <int IB>
@@ -203,71 +207,100 @@ struct PairDf {
     int undec[IB / 2];
 };
 
-// K terms of neuron column w0 (stride N) against IB images' inputs.
-template <int IB, bool L1>
-__device__ __forceinline__ void anchored_dot(const float* __restrict__ w0, int N, int K, const void* in, float sig,
-                                             float2 (&u)[IB]) {
-    float S[IB], H[IB], Lo[IB];
+// K terms of neuron column w0 (stride N) against NP pairs of images, whose inputs start
+// at in, row floats from one term to the next, the low parts lo floats behind the high ones.
+template <int NP, bool L1>
+__device__ __forceinline__ void anchored_dot(const float* __restrict__ w0, int N, int K, const float* in, int row,
+                                             int lo, float sig, float2 (&u)[2 * NP]) {
+    f32x2 A[NP], H[NP], Lo[NP];
 #pragma unroll
-    for (int m = 0; m < IB; ++m) S[m] = H[m] = Lo[m] = 0.f;
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        float r[IB];
+    for (int m = 0; m < NP; ++m) {
+        A[m] = pack2(sig, sig);
+        H[m] = Lo[m] = 0ull;
+    }
+    f32x2 r[NP];
+    auto term = [&](float w1, const float* h) {
+        const f32x2 w = pack2(w1, w1);
+        f32x2 hx[NP], hy[NP];
+        if (NP % 2 == 0) {
 #pragma unroll
-        for (int m = 0; m < IB; ++m) r[m] = 0.f;
-        const int k1 = min(K, k0 + 16);
-#pragma unroll 4
-        for (int k = k0; k < k1; ++k) {
-            const float w = __ldg(w0 + (size_t)k * N);
-            float hx[IB], hy[IB];
-            if (L1) {
-                const float* h = static_cast<const float*>(in) + (size_t)k * IB;
-#pragma unroll
-                for (int m = 0; m < IB; m += 2) {
-                    const float2 v = *reinterpret_cast<const float2*>(h + m);
-                    hx[m] = v.x;
-                    hx[m + 1] = v.y;
-                }
-            } else {
-                const float2* h = static_cast<const float2*>(in) + (size_t)k * IB;
-#pragma unroll
-                for (int m = 0; m < IB; m += 2) {
-                    const float4 v = *reinterpret_cast<const float4*>(h + m);
-                    hx[m] = v.x;
-                    hy[m] = v.y;
-                    hx[m + 1] = v.z;
-                    hy[m + 1] = v.w;
+            for (int m = 0; m < NP; m += 2) {
+                const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(h + 2 * m);
+                hx[m] = x.x;
+                hx[(m + 1) % NP] = x.y;
+                if (!L1) {
+                    const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(h + lo + 2 * m);
+                    hy[m] = y.x;
+                    hy[(m + 1) % NP] = y.y;
                 }
             }
+        } else {
 #pragma unroll
-            for (int m = 0; m < IB; ++m) {
-                const float q = __fsub_rn(__fmaf_rn(w, hx[m], sig), sig);
-                S[m] = __fadd_rn(S[m], q);
-                float e = __fmaf_rn(w, hx[m], -q);
-                if (!L1) e = __fmaf_rn(w, hy[m], e);
-                r[m] = __fadd_rn(r[m], e);
+            for (int m = 0; m < NP; ++m) {
+                hx[m] = *reinterpret_cast<const f32x2*>(h + 2 * m);
+                if (!L1) hy[m] = *reinterpret_cast<const f32x2*>(h + lo + 2 * m);
             }
         }
 #pragma unroll
-        for (int m = 0; m < IB; ++m) {
-            const float2 t = two_sum(H[m], r[m]);
-            H[m] = t.x;
-            Lo[m] = __fadd_rn(Lo[m], t.y);
+        for (int m = 0; m < NP; ++m) {
+            const f32x2 a = fma2(w, hx[m], A[m]);
+            f32x2 e = fma2(w, hx[m], sub2(A[m], a));
+            if (!L1) e = fma2(w, hy[m], e);
+            r[m] = add2(r[m], e);
+            A[m] = a;
+        }
+    };
+    constexpr int KB = 16;
+    float w[KB];  // a block's weights come in while the block before is at work
+    const float* wp = w0;
+    if (K >= KB) {
+#pragma unroll
+        for (int j = 0; j < KB; ++j) w[j] = __ldg(wp + (size_t)j * N);
+    }
+    for (int k0 = 0; k0 < K; k0 += KB) {
+#pragma unroll
+        for (int m = 0; m < NP; ++m) r[m] = 0ull;
+        const float* h = in + (size_t)k0 * row;
+        if (k0 + KB <= K) {
+            float c[KB];
+#pragma unroll
+            for (int j = 0; j < KB; ++j) c[j] = w[j];
+            wp += (size_t)KB * N;
+            if (k0 + 2 * KB <= K) {
+#pragma unroll
+                for (int j = 0; j < KB; ++j) w[j] = __ldg(wp + (size_t)j * N);
+            }
+#pragma unroll
+            for (int j = 0; j < KB; ++j) term(c[j], h + (size_t)j * row);
+        } else {
+#pragma unroll 1
+            for (int j = 0; k0 + j < K; ++j) term(__ldg(w0 + (size_t)(k0 + j) * N), h + (size_t)j * row);
+        }
+#pragma unroll
+        for (int m = 0; m < NP; ++m) {  // two_sum
+            const f32x2 t = add2(H[m], r[m]), b = sub2(t, H[m]);
+            Lo[m] = add2(Lo[m], add2(sub2(H[m], sub2(t, b)), sub2(r[m], b)));
+            H[m] = t;
         }
     }
 #pragma unroll
-    for (int m = 0; m < IB; ++m) u[m] = df_add(make_float2(S[m], 0.f), two_sum(H[m], Lo[m]));
+    for (int m = 0; m < NP; ++m) {
+        const float2 a = unpack2(A[m]), h = unpack2(H[m]), l = unpack2(Lo[m]);
+        u[2 * m] = df_add(make_float2(__fsub_rn(a.x, sig), 0.f), two_sum(h.x, l.x));
+        u[2 * m + 1] = df_add(make_float2(__fsub_rn(a.y, sig), 0.f), two_sum(h.y, l.y));
+    }
 }
 
 template <int IB>
-__global__ void __launch_bounds__(TPD) k_pairs_df(NetView net, const uint8_t* __restrict__ x1s,
+__global__ void __launch_bounds__(TPD, 2) k_pairs_df(NetView net, const uint8_t* __restrict__ x1s,
                                                   const uint8_t* __restrict__ x2s, int n_pairs, double g, double d,
                                                   PairOut o, int bufw) {
     constexpr int PB = IB / 2;
     extern __shared__ double sh[];
     __shared__ PairDf<IB> T;
-    float2* const buf0 = reinterpret_cast<float2*>(sh);      // [bufw][IB]
-    float2* const buf1 = buf0 + (size_t)bufw * IB;           // the same; layer 1's grey levels first
-    unsigned char* const fl = reinterpret_cast<unsigned char*>(buf1 + (size_t)bufw * IB);  // [total][PB]
+    float* const buf0 = reinterpret_cast<float*>(sh);   // [bufw][2][IB]: high parts, low parts
+    float* const buf1 = buf0 + (size_t)bufw * 2 * IB;   // the same; layer 1's grey levels first
+    unsigned char* const fl = reinterpret_cast<unsigned char*>(buf1 + (size_t)bufw * 2 * IB);  // [total][PB]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int H0 = net.dims[0], L = net.L;
     const bool relu = net.act == ACT_RELU;
@@ -276,7 +309,7 @@ __global__ void __launch_bounds__(TPD) k_pairs_df(NetView net, const uint8_t* __
     const float2 inv = make_float2(inv_hi, (float)(1.0 / 255.0 - (double)inv_hi));
     for (int p0 = blockIdx.x * PB; p0 < n_pairs; p0 += gridDim.x * PB) {
         const int np = min(PB, n_pairs - p0);
-        float* const in0 = reinterpret_cast<float*>(buf1);
+        float* const in0 = buf1;  // [H0][IB]
         for (int im = 0; im < IB; ++im) {
             const uint8_t* x = (im & 1 ? x2s : x1s) + (size_t)(p0 + (im >> 1)) * H0;
             for (int k = tid; k < H0; k += TPD) in0[k * IB + im] = (im >> 1) < np ? (float)x[k] : 0.f;
@@ -294,13 +327,14 @@ __global__ void __launch_bounds__(TPD) k_pairs_df(NetView net, const uint8_t* __
         __syncthreads();
         for (int l = 1; l <= L; ++l) {
             const int K = net.dims[l - 1], N = net.dims[l], off = net.noff[l];
-            const void* in = l == 1 ? static_cast<const void*>(buf1) : (l & 1 ? buf1 : buf0);
-            float2* const outb = l & 1 ? buf0 : buf1;
+            const float* in = l & 1 ? buf1 : buf0;
+            float* const outb = l & 1 ? buf0 : buf1;
             const float* __restrict__ WT = net.WT[l];
             const float cK = 5.f * (float)(K + 16) * 0x1p-45f;
             float Nm = 0.f;
             for (int m = 0; m < IB; ++m) Nm = fmaxf(Nm, T.N[m]);
-            // sigma of a neuron: 1.5 2^M with 2^(M-1) >= ||W_i|| max ||h|| (and above 0)
+            Nm = __fmul_ru(Nm, __fmaf_ru((float)K, 0x1p-22f, 1.f));
+            // sigma of a neuron: 1.5 2^M with 2^(M-1) >= (1 + K 2^-22) ||W_i|| max ||h|| (and above 0)
             auto anchor = [&](int n) {
                 const int ex = ilogbf(fmaxf(__fmul_ru(net.rownorm[l][n], Nm), 1e-30f));
                 return 1.5f * ldexpf(1.f, ex + 2);
@@ -319,47 +353,27 @@ __global__ void __launch_bounds__(TPD) k_pairs_df(NetView net, const uint8_t* __
             if (N * 4 >= TPD) {
                 for (int n = tid; n < N; n += TPD) {
                     float2 u[IB];
-                    if (l == 1) anchored_dot<IB, true>(WT + n, N, K, in, anchor(n), u);
-                    else anchored_dot<IB, false>(WT + n, N, K, in, anchor(n), u);
+                    if (l == 1) anchored_dot<PB, true>(WT + n, N, K, in, IB, 0, anchor(n), u);
+                    else anchored_dot<PB, false>(WT + n, N, K, in, 2 * IB, IB, anchor(n), u);
 #pragma unroll
-                    for (int m = 0; m < IB; ++m) outb[(size_t)n * IB + m] = finish(u[m], n);
+                    for (int m = 0; m < IB; ++m) {
+                        const float2 v = finish(u[m], n);
+                        outb[(size_t)n * 2 * IB + m] = v.x;
+                        outb[(size_t)n * 2 * IB + IB + m] = v.y;
+                    }
                 }
             } else {  // a narrow layer: a thread per neuron and pair
                 for (int it = tid; it < N * PB; it += TPD) {
                     const int n = it / PB, pp = it % PB;
-                    float S[2] = {0.f, 0.f}, Hh[2] = {0.f, 0.f}, Lo[2] = {0.f, 0.f};
-                    const float sig = anchor(n);
-                    for (int k0 = 0; k0 < K; k0 += 16) {
-                        float r[2] = {0.f, 0.f};
-                        const int k1 = min(K, k0 + 16);
-#pragma unroll 4
-                        for (int k = k0; k < k1; ++k) {
-                            const float w = __ldg(WT + (size_t)k * N + n);
-                            float4 h;
-                            if (l == 1) {
-                                const float2 v = *reinterpret_cast<const float2*>(in0 + (size_t)k * IB + 2 * pp);
-                                h = make_float4(v.x, 0.f, v.y, 0.f);
-                            } else {
-                                h = *reinterpret_cast<const float4*>(static_cast<const float2*>(in) + (size_t)k * IB + 2 * pp);
-                            }
-                            float q = __fsub_rn(__fmaf_rn(w, h.x, sig), sig);
-                            S[0] = __fadd_rn(S[0], q);
-                            r[0] = __fadd_rn(r[0], __fmaf_rn(w, h.y, __fmaf_rn(w, h.x, -q)));
-                            q = __fsub_rn(__fmaf_rn(w, h.z, sig), sig);
-                            S[1] = __fadd_rn(S[1], q);
-                            r[1] = __fadd_rn(r[1], __fmaf_rn(w, h.w, __fmaf_rn(w, h.z, -q)));
-                        }
+                    float2 u[2];
+                    if (l == 1) anchored_dot<1, true>(WT + n, N, K, in + 2 * pp, IB, 0, anchor(n), u);
+                    else anchored_dot<1, false>(WT + n, N, K, in + 2 * pp, 2 * IB, IB, anchor(n), u);
 #pragma unroll
-                        for (int m = 0; m < 2; ++m) {
-                            const float2 t = two_sum(Hh[m], r[m]);
-                            Hh[m] = t.x;
-                            Lo[m] = __fadd_rn(Lo[m], t.y);
-                        }
+                    for (int m = 0; m < 2; ++m) {
+                        const float2 v = finish(u[m], n);
+                        outb[(size_t)n * 2 * IB + 2 * pp + m] = v.x;
+                        outb[(size_t)n * 2 * IB + IB + 2 * pp + m] = v.y;
                     }
-#pragma unroll
-                    for (int m = 0; m < 2; ++m)
-                        outb[(size_t)n * IB + 2 * pp + m] =
-                            finish(df_add(make_float2(S[m], 0.f), two_sum(Hh[m], Lo[m])), n);
                 }
             }
             if (tid < IB) {  // layer 1: the input's norm and error on the [0, 1] scale
@@ -377,8 +391,10 @@ __global__ void __launch_bounds__(TPD) k_pairs_df(NetView net, const uint8_t* __
             float h1 = 0.f, h2 = 0.f, s1 = 0.f, s2 = 0.f;
             double dd = 0.0;
             for (int n = tid / PB; n < N; n += TPD / PB) {
-                float2* up = outb + (size_t)n * IB + 2 * pp;
-                const float2 a = up[0], b = up[1];
+                float2* const hi = reinterpret_cast<float2*>(outb + (size_t)n * 2 * IB + 2 * pp);
+                float2* const lo = hi + IB / 2;
+                const float2 uh = *hi, ul = *lo;
+                const float2 a = make_float2(uh.x, ul.x), b = make_float2(uh.y, ul.y);
                 if (live) {
                     const float rn = net.rownorm[l][n];
                     const float e1 = __fmaf_ru(rn, X1, __fmul_ru(0x1p-42f, fabsf(a.x)));
@@ -413,8 +429,8 @@ __global__ void __launch_bounds__(TPD) k_pairs_df(NetView net, const uint8_t* __
                 s2 = __fmaf_ru(b.x, b.x, s2);
                 if (l < L) {
                     if (relu) {
-                        up[0] = a.x > 0.f ? a : make_float2(0.f, 0.f);
-                        up[1] = b.x > 0.f ? b : make_float2(0.f, 0.f);
+                        *hi = make_float2(fmaxf(a.x, 0.f), fmaxf(b.x, 0.f));
+                        *lo = make_float2(a.x > 0.f ? a.y : 0.f, b.x > 0.f ? b.y : 0.f);
                     }
                     const float p = relu ? fmaxf(a.x, 0.f) : a.x, q = relu ? fmaxf(b.x, 0.f) : b.x;
                     h1 = __fmaf_ru(p, p, h1);
