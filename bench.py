@@ -261,6 +261,70 @@ def launches_per_step(precision, L, batch=False, n_points=0):
     return pro + (6 if batch else 7)
 
 
+def folded_nodes(net, q, precision):
+    """Nodes per hidden layer of the query's folded net (csrc/fold.cu: the neurons that
+    can change sign over the box), from interval bounds in FP64; None where the general
+    passes run (no ReLU net, FP64, more than 128 nodes, more than 32 outputs, small FP32 nets)."""
+    W, b = net["W"], net["b"]
+    dims = [W[0].shape[1]] + [w.shape[0] for w in W]
+    if net["act"] != "relu" or precision == "fp64" or len(W) < 2 or dims[-1] > 32 or \
+            (precision == "fp32" and max(dims[1:]) <= 32):
+        return None
+    v = np.asarray(q["image"]).astype(int)[q["pixels"]]
+    bound = np.maximum(np.minimum(q["k"], 255 - v), np.minimum(q["k"], v)) / 255.0
+    h, rows, nodes = np.asarray(q["image"]) / 255.0, None, []
+    for l in range(len(W) - 1):
+        w = W[l].astype(np.float64)
+        u = w @ h + b[l]
+        a = w[:, q["pixels"]] if rows is None else np.hstack([(w * carried) @ rows, w[:, cross]])
+        reach = np.abs(a) @ bound
+        keeps = np.abs(u) > reach
+        cross, carried = np.where(~keeps)[0], (u >= 0).astype(np.float64)
+        nodes.append(len(cross))
+        bound = np.concatenate([bound, reach[cross] - np.abs(u[cross])])
+        h, rows = np.maximum(u, 0.0), a
+    return nodes if sum(nodes) <= 128 else None
+
+
+def folded_launches(precision, L, waits):
+    """Kernels of the library per call of a folded query: init, L base layers, pack, folded
+    pass, its FP64 pass, whole-net FP64 pass, time stamps (wide layers: the work count).
+    A call that does not wait launches the general passes as well; they leave it out."""
+    if precision == "fp8":
+        return L + 7
+    return L + 6 if waits else launches_per_step(precision, L) + 3
+
+
+def search_launches(L, tiles, tile_points, folded):
+    """Kernels of a tile search that checks `tiles` tiles: set-up, then 6 per tile (screen,
+    split pass, FP32, double-float, FP64, stamps) or, folded, 4 per group of 1, 4, 16, 64
+    tiles of at most 2^22 points."""
+    if not folded:
+        return L + 4 + 6 * tiles
+    groups, want, done = 0, 1, 0
+    while done < tiles:
+        done += max(1, min(want, (1 << 22) // max(1, tile_points)))
+        groups, want = groups + 1, min(4 * want, 64)
+    return L + 2 + 4 * groups
+
+
+def folded_roofline(nodes, dims, s, n_pts, sums, pk):
+    """Roofline of a folded query's first pass (csrc/fold.cu). Work it cannot do without:
+    the linear part, 2 s FLOP per point and row (nodes and the HL - 1 margins); the sources
+    of crossed nodes, the sign tests and the decode come on top, so the fraction is small:
+    the pass is bound by issue slots."""
+    ms = statistics.median(x["ms_screen"] for x in sums)
+    flops = 2 * s * (sum(nodes) + dims[-1] - 1) * n_pts
+    alu = 152 * 128 * 2 * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
+    ach = flops / (ms / 1000.0) / 1e12
+    top = {"bound": "alu", "achieved": ach, "peak": alu, "unit": "TFLOP/s", "frac": ach / alu, "traffic": None,
+           "kernel": "folded first pass (k_fold, k_fold64)", "peak_kind": "derived FP32 ALU",
+           "flops_per_launch": flops, "launch_ms": ms}
+    return dict(top, nodes=list(nodes), points_per_ns=n_pts / (ms * 1e6),
+                passes=[{key: top[key] for key in ("kernel", "launch_ms", "flops_per_launch", "bound", "achieved",
+                                                   "peak", "peak_kind", "frac", "traffic")}])
+
+
 def pass_rooflines(precision, dims, s, n_pts, sums, pk, pk_kind, traffic=None):
     """Roofline of each pass of a verify call (CUDA-event times from the library,
     medians over the timed steps) and, at the top level, the pass that took
@@ -367,7 +431,8 @@ def main_batch(a):
                          "ties_only": sum(x["verdict"] == "TIES_ONLY" for x in sums),
                          "n_recheck": [sum(x["n_recheck"][i] for x in sums) for i in range(4)]},
             # the smallest-first schedule runs min(8, queries) waves, each a full chain of passes
-            "gpu_launches": a.steps * launches_per_step(a.precision, len(cfg["dims"]) - 1, batch=True)
+            "gpu_launches": a.steps * (launches_per_step(a.precision, len(cfg["dims"]) - 1, batch=True) +
+                                       (3 if cfg["act"] == "relu" and a.precision != "fp64" else 0))
             * (min(8, len(qs)) if a.schedule == "small_first" else 1)}
     if ck:
         line["clocks"] = ck
@@ -462,9 +527,9 @@ def main_proposal(a):
                        "witness_tiles_mean": float((ctr > 0).sum(1).mean())},
             "training": {"seconds": train_s, "best_epoch": hist["best_epoch"],
                          "val_rank": hist["val_rank"]},
-            # per search: set-up (init, L base layers, tables, finish, column classes)
-            # plus 6 per checked tile (screen, split pass, FP32, double-float, FP64, stamps)
-            "gpu_launches": int(sum(len(cfg["dims"]) + 3 + 6 * t for n in tiles for t in tiles[n])),
+            "gpu_launches": int(sum(search_launches(len(cfg["dims"]) - 1, t, -(-(2 * cfg["k"] + 1) ** cfg["s"] // T),
+                                                    cfg["act"] == "relu" and a.precision != "fp64")
+                                    for n in tiles for t in tiles[n])),
             "wall_s": time.perf_counter() - t0}
     if ck:
         line["clocks"] = ck
@@ -534,6 +599,9 @@ def main_pairs(a):
     fw, sw = vnet.mask_words()
     pk, pk_kind = peaks()
     ach = flops_pair * n / (ms / 1000.0) / 1e12
+    # ReLU nets: FP32 pairs, 4 (layer 1) or 5 two-lane FP32 instructions for two multiply-adds
+    pair32 = cfg["act"] != "sigmoid"
+    pk_pair = 152 * 128 * 2 * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12 * 2 / 9 if pair32 else 1.25
     line = {"metric": "image pairs/sec (all covers)", "value": n / (ms / 1000.0), "unit": "pairs/s",
             "n_gpus": 1, "steps": a.steps, "warmup": a.warmup, "ms_per_step": ms, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
@@ -542,9 +610,11 @@ def main_pairs(a):
             "e2e": {"value": n / statistics.median(e2e), "unit": "pairs/s",
                     "h2d_bytes_per_step": int(2 * x1.size), "d2h_bytes_per_step": int(4 * (6 * fw + 4 * sw))},
             "gpu_launches": a.steps,
-            "roofline": {"bound": "alu", "achieved": ach, "peak": 1.25, "unit": "TFLOP/s", "frac": ach / 1.25,
-                         "traffic": None, "kernel": "k_pairs (two FP64 forward passes per pair)",
-                         "peak_kind": "nominal FP64 ALU", "flops_per_launch": flops_pair * n,
+            "roofline": {"bound": "alu", "achieved": ach, "peak": pk_pair, "unit": "TFLOP/s", "frac": ach / pk_pair,
+                         "traffic": None, "kernel": "k_pairs_df (two forward passes per pair, FP32 pairs)" if pair32
+                         else "k_pairs (two FP64 forward passes per pair)",
+                         "peak_kind": "derived FP32 ALU x 2/9" if pair32 else "nominal FP64 ALU",
+                         "flops_per_launch": flops_pair * n,
                          "launch_ms": ms},
             "covers": {k: out[k + "_fraction"] for k in ("ss", "sv", "ds", "dv")}}
     if ck:
@@ -809,10 +879,12 @@ def main():
     if a.precision in ("bf16", "fp16", "fp8") and not a.no_fp32_arm:
         ref_cov = None if a.no_coverage else vb.get_coverage(res)
         ref_bm = vb.get_verdict_bitmap(res, n_pts)
+        vb.set_folding(vnet, False)  # the plain passes over every point
         step("fp32")
         vb.result_summary(res)
         k32 = max(3, min(a.steps, 5))
         ms32, sums32, merge32, _ = timed_steps("fp32", k32)
+        vb.set_folding(vnet, True)
         m32 = sum(ms32) / len(ms32) + (statistics.median(merge32) if split else 0.0)
         ms32_max, _, value32 = job_throughput(m32, n_chk, world, dev)
         a0, b0 = sums[-1], sums32[-1]
@@ -822,7 +894,7 @@ def main():
             cov32 = vb.get_coverage(res)
             same = same and all(np.array_equal(cov32[f], ref_cov[f]) for f in ("flip", "flip_tie", "ss", "ss_tie"))
         fp32_arm = {"value": value32, "unit": UNIT, "ms_per_step": ms32_max, "steps": k32,
-                    "call": "vbmc_verify_query_device, precision fp32 (no tensor cores)",
+                    "call": "vbmc_verify_query_device, precision fp32 (no tensor cores, folding off)",
                     "identical_results": bool(same),
                     "ms_pass": dict(zip(("split", "fp32", "double_float", "fp64"), b0["ms_pass"])),
                     "ms_screen": b0["ms_screen"], "n_recheck": b0["n_recheck"]}
@@ -852,7 +924,9 @@ def main():
         L = len(cfg["dims"]) - 1
         traffic = PROFILED_TRAFFIC.get((a.workload, a.precision, not a.no_coverage, s, k)) \
             if plain and not split else None
-        roof = pass_rooflines(a.precision, cfg["dims"], s, n_chk, sums, pk, pk_kind, traffic)
+        nodes = folded_nodes(net_d, dict(q, k=k), a.precision)
+        roof = pass_rooflines(a.precision, cfg["dims"], s, n_chk, sums, pk, pk_kind, traffic) if nodes is None \
+            else folded_roofline(nodes, cfg["dims"], s, n_chk, sums, pk)
         verdict = {"verdict": last["verdict"], "n_adversarial": last["n_adversarial"],
                    "first_witness": last["first_witness"], "n_ties": last["n_ties"],
                    "n_recheck": last["n_recheck"], "ms_prologue": last["ms_prologue"],
@@ -889,7 +963,8 @@ def main():
                 "e2e": {"value": e2e_value, "unit": UNIT,
                         "h2d_bytes_per_step": int(cfg["dims"][0] + 4 * s),
                         "d2h_bytes_per_step": int(4 * ((n_pts + 31) // 32) + 8 * fw + 8 * sw + 128)},
-                "gpu_launches": a.steps * launches_per_step(a.precision, L, n_points=n_pts),
+                "gpu_launches": a.steps * (launches_per_step(a.precision, L, n_points=n_pts) if nodes is None
+                                           else folded_launches(a.precision, L, not plain)),
                 "roofline": roof,
                 "verdict": verdict,
                 "wall_s": wall}
