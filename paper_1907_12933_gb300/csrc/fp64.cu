@@ -12,6 +12,13 @@
 //   * SS-Cover of (j in layer l, i in layer l+1): certain when layer l has no
 //     tie and exactly one change (j) and i changes without tie; pairs that
 //     hold only under some resolution of the ties go to the SS-tie mask.
+//
+// A range has a CTA per point. Queued points are few, and one CTA is bound by its SM's
+// FP64 pipe (16 cycles a warp instruction: two layers of 1024 take 1.3 ms), so a cluster
+// of CL CTAs shares a point: a layer's neurons are dealt to the cluster's warps, their
+// outputs go to every CTA's shared memory, and the first CTA does the rest. A weight
+// becomes FP64 by its bits, not on that pipe. The sums keep their order. One queued
+// point of 784-1024x3-10: 1,375 -> 380 us, now bound by the latency of the weights.
 #include "dev.cuh"
 #include "launch.h"
 
@@ -28,6 +35,31 @@ __device__ __forceinline__ double act64(int act, double u) {
     return u;
 }
 
+// (double)w of an FP32 number by its bits; zero, subnormal and non-finite ones by conversion.
+__device__ __forceinline__ double widen(float w) {
+    const unsigned b = __float_as_uint(w);
+    if (((b >> 23) & 255u) - 1u >= 254u) return (double)w;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// *p of CTA rank's shared memory = v.
+__device__ __forceinline__ void store_cluster(double* p, unsigned rank, double v) {
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), ra;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
+}
+
+template <int CL>
 __global__ void __launch_bounds__(T64)
 k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__ gather,
        const unsigned long long* __restrict__ gather_count, unsigned long long gather_cap,
@@ -35,11 +67,12 @@ k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int total = net.total, hmax = net.hmax;
     double* u = reinterpret_cast<double*>(smem_raw);       // [total]
-    double* h = u + total;                                   // [hmax]
-    unsigned char* fl = reinterpret_cast<unsigned char*>(h + hmax);  // [total]
-    unsigned char* ti = fl + total;                                   // [total]
+    constexpr int HB = CL > 1 ? 2 : 1;
+    double* h0 = u + total;                                  // [HB][hmax]: layer l's outputs in l % HB
+    unsigned char* fl = reinterpret_cast<unsigned char*>(h0 + HB * hmax);  // [total]
+    unsigned char* ti = fl + total;                                         // [total]
     __shared__ int nflip[kMaxL + 2], ntie[kMaxL + 2], only[kMaxL + 2];
-    __shared__ int dstep[kMaxS];
+    __shared__ double dstep[kMaxS];
     __shared__ int skip;
 
     unsigned long long n;
@@ -50,7 +83,9 @@ k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__
         n = range_hi - range_lo;
     }
     const int L = net.L;
-    for (unsigned long long e = blockIdx.x; e < n; e += gridDim.x) {
+    const unsigned rank = CL > 1 ? cluster_rank() : 0u;
+    if (CL > 1 && n > 0) cluster_barrier();  // every CTA of the cluster has started
+    for (unsigned long long e = blockIdx.x / CL; e < n; e += gridDim.x / CL) {
         unsigned long long t;
         int qi;
         if (gather) {
@@ -65,7 +100,7 @@ k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__
         if (threadIdx.x == 0) {
             int d[kMaxS];
             decode_digits(t, Q.s, Q.R, d);
-            for (int p = 0; p < Q.s; ++p) dstep[p] = Q.dv[p * Q.R + d[p]];
+            for (int p = 0; p < Q.s; ++p) dstep[p] = (double)Q.dv[p * Q.R + d[p]] / 255.0;
             skip = !gather && Q.filter && !in_filter(Q, d);  // outside the L2 ball / shell
             if (!gather && Q.filter && !skip) atomicAdd(&Q.cnt->n_points, 1ull);
         }
@@ -83,96 +118,115 @@ k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__
             const float* W1 = net.W[1];
             for (int j = threadIdx.x; j < H1; j += T64) {
                 double a = Q.ub[j];
-                for (int p = 0; p < Q.s; ++p)
-                    a += (double)W1[(size_t)j * H0 + Q.pix[p]] * ((double)dstep[p] / 255.0);
+                for (int p = 0; p < Q.s; ++p) a += (double)W1[(size_t)j * H0 + Q.pix[p]] * dstep[p];
                 u[j] = a;
-                h[j] = (L > 1) ? act64(net.act, a) : a;
+                h0[(1 % HB) * hmax + j] = (L > 1) ? act64(net.act, a) : a;
             }
         }
         __syncthreads();
         for (int l = 2; l <= L; ++l) {
             const int K = net.dims[l - 1], N = net.dims[l];
-            const float* WT = net.WT[l];
+            const float* __restrict__ WT = net.WT[l];
             const float* b = net.b[l];
             const int off = net.noff[l];
-            for (int i = threadIdx.x; i < N; i += T64) {
+            const double* h = h0 + (size_t)((l - 1) % HB) * hmax;
+            double* const hn = h0 + (size_t)(l % HB) * hmax;
+            // 32 neurons a warp, the cluster's CTAs in turn
+            for (int i = (int)((threadIdx.x >> 5) * CL + rank) * 32 + (int)(threadIdx.x & 31); i < N; i += T64 * CL) {
                 double a = 0.0;
-                for (int j = 0; j < K; ++j) a += (double)WT[(size_t)j * N + i] * h[j];
-                u[off + i] = a + (double)b[i];
-            }
-            __syncthreads();
-            if (l < L)
-                for (int i = threadIdx.x; i < N; i += T64) h[i] = act64(net.act, u[off + i]);
-            __syncthreads();
-        }
-        // signs, ties, changes
-        for (int nn = threadIdx.x; nn < total; nn += T64) {
-            const double ub = Q.ub[nn], ut = u[nn];
-            const bool tie = fabs(ut) < kTau || fabs(ub) < kTau;
-            const bool ch = ((ut >= 0.0) != (ub >= 0.0)) && !tie;
-            fl[nn] = ch;
-            ti[nn] = tie;
-            int l = 1;
-            while (l < L && nn >= net.noff[l + 1]) ++l;
-            if (ch) {
-                atomicAdd(&nflip[l], 1);
-                atomicMax(&only[l], nn - net.noff[l]);
-                if (Q.flip) set_bit_once(Q.flip, nn);
-            }
-            if (tie) {
-                atomicAdd(&ntie[l], 1);
-                if (Q.flip_tie) set_bit_once(Q.flip_tie, nn);
-            }
-        }
-        __syncthreads();
-        // SS-Cover pairs (j in l, i in l+1)
-        if (Q.ss) {
-            for (int l = 1; l < L; ++l) {
-                const int Hl = net.dims[l], Hn = net.dims[l + 1];
-                const int ol = net.noff[l], on = net.noff[l + 1];
-                const bool certain = ntie[l] == 0 && nflip[l] == 1;
-                if (!certain && ntie[l] == 0) continue;  // no flip or >= 2 certain flips
-                if (!certain && nflip[l] >= 2) continue;
-                for (int j = 0; j < Hl; ++j) {
-                    bool cand;
-                    if (certain || nflip[l] == 1) cand = (j == only[l]);
-                    else cand = ti[ol + j];  // no certain flip, some ties: each tie may be the one
-                    if (!cand) continue;
-                    for (int i = threadIdx.x; i < Hn; i += T64) {
-                        const unsigned long long bit = (unsigned long long)net.ssoff[l] +
-                                                       (unsigned long long)j * Hn + i;
-                        if (certain && fl[on + i]) set_bit_once(Q.ss, bit);
-                        else if (fl[on + i] || ti[on + i]) set_bit_once(Q.ss_tie, bit);
+#pragma unroll 16
+                for (int j = 0; j < K; ++j) a += widen(__ldg(WT + (size_t)j * N + i)) * h[j];
+                const double v = a + (double)b[i];
+                if (CL == 1) {
+                    u[off + i] = v;
+                } else {
+                    store_cluster(u + off + i, 0u, v);
+                    if (l < L) {
+                        const double y = act64(net.act, v);
+                        for (unsigned c = 0; c < CL; ++c) store_cluster(hn + i, c, y);
                     }
                 }
             }
-        }
-        // verdict
-        if (threadIdx.x == 0) {
-            const int HL = net.dims[L];
-            const double* y = u + net.noff[L];
-            const int D = Q.cnt->D;
-            int am = 0;
-            double mx = -DBL_MAX;
-            for (int i = 0; i < HL; ++i) {
-                if (y[i] > y[am]) am = i;
-                if (i != D && y[i] > mx) mx = y[i];
+            if (CL > 1) {
+                cluster_barrier();
+            } else {
+                __syncthreads();
+                if (l < L)
+                    for (int i = threadIdx.x; i < N; i += T64) hn[i] = act64(net.act, u[off + i]);
+                __syncthreads();
             }
-            // Eq. 10: m = y_D - max_{i!=D} y_i; Eq. 11: m = max(y_D - V, V - max_{i!=D} y_i),
-            // negative iff y_D < V < some other output
-            const bool thr = Q.prop == PROP_THRESHOLD;
-            const double m = thr ? fmax(y[D] - Q.V, Q.V - mx) : y[D] - mx;
-            if (thr) am = m < 0.0 ? -1 : D;
-            if (fabs(m) < kTau) {
-                unsigned long long k = atomicAdd(&Q.cnt->n_ties, 1ull);
-                if (k < Q.ties_cap) Q.ties[k] = t;
-                else atomicOr(&Q.cnt->err, DERR_TIES);
-            } else if (am != D) {
-                record_adversarial(Q, t);
-            }
-            if (gather) work_done(Q.cnt, 1);  // time to verdict: this queued point is resolved
         }
-        __syncthreads();
+        if (CL == 1 || rank == 0) {
+            // signs, ties, changes
+            for (int nn = threadIdx.x; nn < total; nn += T64) {
+                const double ub = Q.ub[nn], ut = u[nn];
+                const bool tie = fabs(ut) < kTau || fabs(ub) < kTau;
+                const bool ch = ((ut >= 0.0) != (ub >= 0.0)) && !tie;
+                fl[nn] = ch;
+                ti[nn] = tie;
+                int l = 1;
+                while (l < L && nn >= net.noff[l + 1]) ++l;
+                if (ch) {
+                    atomicAdd(&nflip[l], 1);
+                    atomicMax(&only[l], nn - net.noff[l]);
+                    if (Q.flip) set_bit_once(Q.flip, nn);
+                }
+                if (tie) {
+                    atomicAdd(&ntie[l], 1);
+                    if (Q.flip_tie) set_bit_once(Q.flip_tie, nn);
+                }
+            }
+            __syncthreads();
+            // SS-Cover pairs (j in l, i in l+1)
+            if (Q.ss) {
+                for (int l = 1; l < L; ++l) {
+                    const int Hl = net.dims[l], Hn = net.dims[l + 1];
+                    const int ol = net.noff[l], on = net.noff[l + 1];
+                    const bool certain = ntie[l] == 0 && nflip[l] == 1;
+                    if (!certain && ntie[l] == 0) continue;  // no flip or >= 2 certain flips
+                    if (!certain && nflip[l] >= 2) continue;
+                    for (int j = 0; j < Hl; ++j) {
+                        bool cand;
+                        if (certain || nflip[l] == 1) cand = (j == only[l]);
+                        else cand = ti[ol + j];  // no certain flip, some ties: each tie may be the one
+                        if (!cand) continue;
+                        for (int i = threadIdx.x; i < Hn; i += T64) {
+                            const unsigned long long bit = (unsigned long long)net.ssoff[l] +
+                                                           (unsigned long long)j * Hn + i;
+                            if (certain && fl[on + i]) set_bit_once(Q.ss, bit);
+                            else if (fl[on + i] || ti[on + i]) set_bit_once(Q.ss_tie, bit);
+                        }
+                    }
+                }
+            }
+            // verdict
+            if (threadIdx.x == 0) {
+                const int HL = net.dims[L];
+                const double* y = u + net.noff[L];
+                const int D = Q.cnt->D;
+                int am = 0;
+                double mx = -DBL_MAX;
+                for (int i = 0; i < HL; ++i) {
+                    if (y[i] > y[am]) am = i;
+                    if (i != D && y[i] > mx) mx = y[i];
+                }
+                // Eq. 10: m = y_D - max_{i!=D} y_i; Eq. 11: m = max(y_D - V, V - max_{i!=D} y_i),
+                // negative iff y_D < V < some other output
+                const bool thr = Q.prop == PROP_THRESHOLD;
+                const double m = thr ? fmax(y[D] - Q.V, Q.V - mx) : y[D] - mx;
+                if (thr) am = m < 0.0 ? -1 : D;
+                if (fabs(m) < kTau) {
+                    unsigned long long k = atomicAdd(&Q.cnt->n_ties, 1ull);
+                    if (k < Q.ties_cap) Q.ties[k] = t;
+                    else atomicOr(&Q.cnt->err, DERR_TIES);
+                } else if (am != D) {
+                    record_adversarial(Q, t);
+                }
+                if (gather) work_done(Q.cnt, 1);  // time to verdict: this queued point is resolved
+            }
+        }
+        if (CL == 1) __syncthreads();
+        else cluster_barrier();  // the first CTA has read what the next point's layers write
     }
 }
 
@@ -239,15 +293,31 @@ void launch_fp64(const NetView& net, const QueryView* d_qs, int nq, const QEntry
                  const unsigned long long* gather_count, unsigned long long gather_cap,
                  unsigned long long range_lo, unsigned long long range_hi, int n_sm,
                  cudaStream_t st) {
-    const size_t smem = sizeof(double) * (net.total + net.hmax) + 2 * (size_t)net.total;
-    cudaFuncSetAttribute(k_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr int CL = 8;
+    auto smem = [&](int buffers) { return sizeof(double) * (net.total + buffers * (size_t)net.hmax) + 2 * (size_t)net.total; };
+    if (gather && smem(2) <= 200 * 1024 && n_sm * 2 >= CL) {
+        cudaFuncSetAttribute(k_fp64<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(2));
+        cudaLaunchConfig_t c{};
+        c.gridDim = (unsigned)(n_sm * 2 / CL * CL);
+        c.blockDim = T64;
+        c.dynamicSmemBytes = smem(2);
+        c.stream = st;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = CL;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        c.attrs = &at;
+        c.numAttrs = 1;
+        cudaLaunchKernelEx(&c, k_fp64<CL>, net, d_qs, gather, gather_count, gather_cap, range_lo, range_hi);
+        return;
+    }
+    cudaFuncSetAttribute(k_fp64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(1));
     unsigned grid = (unsigned)n_sm * 8;
     if (!gather) {
-        unsigned long long n = range_hi - range_lo;
+        const unsigned long long n = range_hi - range_lo;
         if (n < grid) grid = (unsigned)(n ? n : 1);
     }
-    k_fp64<<<grid, T64, smem, st>>>(net, d_qs, gather, gather_count, gather_cap, range_lo,
-                                    range_hi);
+    k_fp64<1><<<grid, T64, smem(1), st>>>(net, d_qs, gather, gather_count, gather_cap, range_lo, range_hi);
 }
 
 }  // namespace vbmc

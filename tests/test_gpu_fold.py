@@ -251,3 +251,21 @@ def test_tile_groups_of_a_search(vb, prec, dims, s, k, tiles, extra, ties):
             vb.set_folding(vnet, False)
             assert got == run(order)
             vb.set_folding(vnet, True)
+
+
+@pytest.mark.parametrize("dims,s,k", [([20, 33, 5], 2, 4), ([20, 1, 2], 1, 100), ([30, 257, 64, 3], 2, 9),
+                                      ([40, 1000, 700, 7], 1, 3), ([25, 31, 32, 33, 32], 3, 2)])
+def test_queued_points_shared_by_a_cluster(vb, dims, s, k):
+    """Sigmoid nets (general passes) with two equal outputs: every point is a margin tie and
+    is settled by the FP64 pass, each by a cluster of CTAs; more points than clusters,
+    layers of fewer neurons than a warp, of more than a warp per CTA, odd ones."""
+    net = synth.make_net(822, dims, "sigmoid", 2.0, "normal")
+    q = synth.make_query(822, 6, dims[0], s, k)
+    D = oracle.eval_point(net, q, 0)["D"]
+    net["W"][-1][(D + 1) % dims[-1]] = net["W"][-1][D]
+    net["b"][-1][(D + 1) % dims[-1]] = net["b"][-1][D]
+    o = oracle.verify(net, q)
+    assert o["n_ties"] == oracle.space_size(s, k)
+    g = run_gpu(vb, net, q, "fp32")
+    assert g["summary"]["n_recheck"][3] == o["n_ties"]
+    compare(g, o, net, q)
