@@ -7,7 +7,8 @@ already in device memory (vbmc_verify_query_device, CUDA events on the
 launching stream); `e2e` through vbmc_verify_query with host buffers plus the
 device-to-host copies of the verdict bitmap and coverage masks.
 
-The same step on the plain FP32 GPU path (no tensor cores) is timed in the same
+The same step on the plain FP32 GPU path (no tensor cores, folding off: every point
+through the whole net) is timed in the same
 run for the tensor precisions: `fp32_path` and the ratio `vs_fp32_path`, with a
 check that both paths give identical results.
 

@@ -1,6 +1,7 @@
 // pairs.cu -- the covering methods of Sec. III-B over a set of input pairs
-// (x1, x2) without enumeration: one CTA per pair, FP64 potentials of both
-// inputs (Eq. 1, the hidden activation on layers 1..L-1), then per pair
+// (x1, x2) without enumeration: potentials of both inputs (Eq. 1, the hidden
+// activation on layers 1..L-1; FP64 with a CTA per pair in k_pairs, FP32 pairs with
+// FP64 for undecided pairs in k_pairs_df), then per pair
 //   sc(n)   sign change (sign(u) = 1 iff u >= 0)
 //   vc(n)   no sign change and max(|u1|, |u2|) >= g min(|u1|, |u2|)
 //   dc(k)   no sign change in layer k and ||u_k(x1) - u_k(x2)||_2 >= d
