@@ -683,7 +683,10 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
     // the folded net checks the queries whose set-up builds one (fold.cu)
     bool fold = false, general = true;  // forms to launch
     for (int i = 0; i < nq; ++i) fold = fold || hq[i].fold;
-    unsigned long long* const d_unfolded = nq > 1 && d_claim ? d_claim + 2 : nullptr;
+    // a batch's count of queries that did not fold: k_fold_pack raises it, so it says nothing
+    // (and the general passes run) where no query may fold; a result's own counters have none
+    unsigned long long* const d_unfolded =
+        fold && nq > 1 && d_claim && (stages & STAGE_SETUP) ? d_claim + 2 : nullptr;
     if (d_claim && d_qcount == d_claim + 2) {  // a result's own counters lie in a row
         VB_CUDA(cudaMemsetAsync(d_claim, 0, sizeof(unsigned long long) * 6, st));
     } else {
