@@ -21,6 +21,7 @@ constexpr int kMaxWidth = 1024;
 constexpr double kTau = 1e-9;  // tie band of margins and potentials
 constexpr int kFoldMax = 128;  // neurons whose sign can change that a folded net holds (fold.cu)
 constexpr int kFoldOut = 32;   // classes (output width) it holds
+constexpr float kFoldBig = 1e37f;  // its values and bounds stay below (FP32 sums of them are finite)
 
 enum { ACT_IDENTITY = 0, ACT_SIGMOID = 1, ACT_RELU = 2 };
 
@@ -153,7 +154,8 @@ struct QueryView {
     float* fx;              // [kMaxS] max over the digits of |dv_p| / 255 (rounded up)
     float* fsb;             // [total] bound on a node's source (0 at the unperturbed image)
     unsigned char* fcls;    // [total] hidden neurons: 0 pos, 1 neg, 2 / 3 node (sign can change; ub < 0 / >= 0)
-    int* fst;               // [kFoldSt]: [0] 1: folded, [1] 1: more than kFoldMax nodes,
+    int* fst;               // [kFoldSt]: [0] 1: folded, [1] 1: not to be folded (more than kFoldMax
+                            //   nodes, a value that is not below kFoldBig),
                             //   [2 + l] rows of layer l: its nodes, the output layer's rows
     int* fnode;             // [kFoldMax] node -> neuron (concatenated index)
     float4* fc32;           // packed FP32 coefficients, see FoldLayout

@@ -22,8 +22,10 @@
 //   k_fold64      the points it left undecided, a warp each, the same rows in FP64:
 //                 every result by its definition, sign ties and margin ties included
 // and what lies within its error of the tie band's edge (about 1e-12 around tau)
-// goes to the FP64 pass on the whole net. A query with more than kFoldMax nodes is not folded; its general
-// passes run instead (they return at once for folded queries).
+// goes to the FP64 pass on the whole net. A query with more than kFoldMax nodes is not
+// folded, nor one with a row, a base value or a bound that is not below kFoldBig (weights
+// need only be finite, and rows are products of them); its general passes run instead
+// (they return at once for folded queries). So every value here is finite.
 //
 // Error of k_fold, constant per row (a node, an output, a margin; u = 2^-24, K sources,
 // M_n = |ub_n| + sum_k |c_nk| bound of source k): the FMA chain from the base value on
@@ -104,7 +106,7 @@ __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync
 __global__ void __launch_bounds__(kPackT) k_fold_pack(NetView net, QueryView* qs, unsigned long long* unfolded) {
     __shared__ FoldShape f;
     __shared__ float eh[kFoldMax], eh64[kFoldMax], em_s[kPackT / 32], et_s[kPackT / 32];  // *_s: the warps' largest
-    __shared__ int D_s, nv_s;
+    __shared__ int D_s, nv_s, big_s;
     __shared__ unsigned signs_s;
     chain_wait();
     chain_next();
@@ -116,6 +118,8 @@ __global__ void __launch_bounds__(kPackT) k_fold_pack(NetView net, QueryView* qs
     const int L = net.L, HL = net.dims[L], offL = net.noff[L], s = Q.s;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool eq11 = Q.prop == PROP_THRESHOLD, cov = Q.flip != nullptr;
+    if (threadIdx.x == 0) big_s = 0;
+    __syncthreads();
     // rows' errors (FP32, rounded up): a warp per row, its lanes over the sources; layer
     // L + 1: the margins. Hidden rows depend on the layers below; outputs and margins on
     // all of them. The first half of the warps does the hidden layers while the other one
@@ -161,10 +165,11 @@ __global__ void __launch_bounds__(kPackT) k_fold_pack(NetView net, QueryView* qs
         const float mag = __fadd_ru(__fadd_ru(fabsf(ub32), M), 1e-30f);
         float e = __fadd_ru(__fmaf_ru((float)(s + cb + 8) * 0x1p-24f, mag, pr), __fadd_ru(fer, 1e-37f));
         e = __fadd_ru(__fadd_ru(e, __double2float_ru(fabs((double)ub32 - ub))), eub);
+        if (!(mag < kFoldBig) || !(e < kFoldBig)) big_s = 1;  // (or NaN)
         const float e2 = __fadd_ru(e, tau2);
         if (l > L) {
             // only a margin that can come near 0 over the box has a say in the common bound
-            if (ub - (double)M - (double)e <= 1e-3) em = fmaxf(em, e2);
+            if (!(ub - (double)M - (double)e > 1e-3)) em = fmaxf(em, e2);
             return;
         }
         // the same in FP64 (u = 2^-53; x_p = dv_p / 255 rounds once, the rows' pairs are exact in it)
@@ -257,6 +262,11 @@ __global__ void __launch_bounds__(kPackT) k_fold_pack(NetView net, QueryView* qs
         for (int w = 1; w < kPackT / 32; ++w) {
             em = fmaxf(em, em_s[w]);
             et = fmaxf(et, et_s[w]);
+        }
+        if (big_s) {
+            Q.fst[1] = 1;
+            if (unfolded) atomicAdd(unfolded, 1ull);
+            return;
         }
         Q.fk32[0] = make_float4(em, et, 0.f, 0.f);
         Q.fst[0] = 1;
@@ -802,7 +812,7 @@ __device__ bool fold64_point(const NetView& net, const QueryView& Q, Fold64& F, 
                 const bool base_tie = fabs(ub) < kTau;  // every evaluation of this neuron is a sign tie
                 ti = fabs(u) < kTau || base_tie;
                 ch = !ti && ((u >= 0.0) != (ub >= 0.0));
-                edge = edge || (cov && !base_tie && fabs(fabs(u) - kTau) <= 2.0 * e);
+                edge = edge || (cov && !base_tie && !(fabs(fabs(u) - kTau) > 2.0 * e));
                 if (l < L) {
                     F.x[K + i] = fmax(ub >= 0.0 ? -u : u, 0.0);
                 } else {
@@ -827,7 +837,7 @@ __device__ bool fold64_point(const NetView& net, const QueryView& Q, Fold64& F, 
     const double mx = warp_max(lane > 0 && lane < HL ? y : -DBL_MAX);
     const double em = warp_max(lane < HL ? ey : 0.0);
     *m = Q.prop == PROP_THRESHOLD ? fmax(yD - Q.V, Q.V - mx) : yD - mx;
-    if (fabs(fabs(*m) - kTau) <= 4.0 * em + 0x1p-51 * (fabs(yD) + fabs(mx) + fabs(Q.V))) edge = true;
+    if (!(fabs(fabs(*m) - kTau) > 4.0 * em + 0x1p-51 * (fabs(yD) + fabs(mx) + fabs(Q.V)))) edge = true;
     __syncwarp();
     return !__any_sync(0xffffffffu, edge);
 }

@@ -359,6 +359,9 @@ __global__ void __launch_bounds__(32 * (WPN > 8 ? WPN : 8)) k_pro_layer(NetView 
         B = __fadd_ru(B, er);
         Q.fbd[n] = B;
         Q.fer[n] = er;
+        // products of weights may pass FP32's range: an infinity or NaN in a row (or er) is
+        // one in B too, times whatever its source's bound is, and the query does not fold
+        if (!(B < kFoldBig) || !(eu < kFoldBig)) Q.fst[1] = 1;
         // a neuron keeps its sign, clear of the tie band, over the whole box
         if (l < net.L) {
             const bool keeps = fabs(u) > ((double)B + (double)eu) * (1.0 + 1e-6) + 4.0 * kTau;
