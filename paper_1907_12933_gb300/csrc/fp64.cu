@@ -106,13 +106,14 @@ k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__
             if (!gather && Q.filter && !skip) atomicAdd(&Q.cnt->n_points, 1ull);
         }
         __syncthreads();
-        if (skip) continue;
+        const bool out = skip;
         if (threadIdx.x <= kMaxL + 1) {
             nflip[threadIdx.x] = 0;
             ntie[threadIdx.x] = 0;
             only[threadIdx.x] = -1;
         }
         __syncthreads();
+        if (out) continue;  // every thread has read skip before the next point's overwrites it
         // layer 1, incremental in FP64
         {
             const int H0 = net.dims[0], H1 = net.dims[1];
