@@ -42,6 +42,7 @@
 // second pass. Whole calls, before and after: 784-512-512-10, s = 6, k = 7 (11.4 M
 // points near the boundary) 28.7 -> 1.5 ms; 784-1024x3-10, s = 4, k = 15 with coverage
 // 191 -> 4.3 ms; 784-300-100-10, s = 5, k = 9 in an L2 ball 27.7 -> 0.52 ms.
+#include "counts.cuh"
 #include "dev.cuh"
 #include "dfloat.cuh"
 #include "launch.h"
@@ -58,6 +59,10 @@ constexpr int FP = 4;            // points per thread: neighbours in the last pi
 constexpr int kXp = 7;           // outer pixels whose changes a thread holds in registers
 constexpr int kFoldSm = 1024;    // coefficient entries kept in shared memory (larger nets: through L1)
 constexpr int kPairW = kFoldMax / 32;
+// Steps of a thread (FP points each) between two additions of its 32-bit counts to the
+// query's: one query's launch gives a warp its share of up to 2^62 points.
+constexpr unsigned long long kFlushSteps = 1ull << 29;
+static_assert(kFlushSteps * FP < (1ull << 32), "a thread's counts fit 32 bits between flushes");
 
 // Rows and packed coefficients by layer: layer l's n[l] rows have s + cb[l] columns;
 // the rows 4 g .. 4 g + 3 take 1 + s + cb[l] entries of fc32 from
@@ -288,11 +293,6 @@ struct FoldSm {
     unsigned long long g;
 };
 
-struct FoldAcc {  // per thread, over a segment of one query
-    unsigned adv = 0, pts = 0;
-    unsigned long long first = ~0ull;
-};
-
 // x / d and the remainder by the 32-bit reciprocal inv = floor((2^32 - 1) / d): the
 // product's high word is at most one too small.
 __device__ __forceinline__ unsigned divmod(unsigned x, unsigned d, unsigned inv, unsigned& r) {
@@ -337,7 +337,7 @@ struct FoldUnits {
 template <bool SM>
 __device__ __forceinline__ void fold_points(const NetView& net, const QueryView& Q, FoldSm& S,
                                             unsigned long long pf, unsigned c, bool on, bool pf32,
-                                            unsigned long long ta, unsigned long long te, FoldAcc& acc,
+                                            unsigned long long ta, unsigned long long te, PointCounts& acc,
                                             const Queue& out, int out_level, unsigned q) {
     const int lane = threadIdx.x & 31;
     const int s = Q.s, R = Q.R, L = net.L;
@@ -690,30 +690,21 @@ __global__ void __launch_bounds__(FT, 2) k_fold(NetView net, const QueryView* __
     auto segment = [&](int q, unsigned long long ta, unsigned long long te, unsigned long long u0,
                        unsigned long long stride) {
         const QueryView& Q = qs[q];
-        FoldAcc acc;
+        PointCounts acc;
         if (ta < te) {
             const FoldUnits U(Q, ta, te);
-            for (unsigned long long u = u0; u < U.n; u += stride) {
-                unsigned c;
-                const unsigned long long pf = U.prefix(u + lane, c);
-                const bool on = u + lane < U.n;
-                if (small) fold_points<true>(net, Q, S, pf, c, on, U.pf32, ta, te, acc, out, out_level, (unsigned)q);
-                else fold_points<false>(net, Q, S, pf, c, on, U.pf32, ta, te, acc, out, out_level, (unsigned)q);
+            for (unsigned long long u = u0; u < U.n;) {
+                const unsigned long long end = U.n - u > stride * kFlushSteps ? u + stride * kFlushSteps : U.n;
+                for (; u < end; u += stride) {
+                    unsigned c;
+                    const unsigned long long pf = U.prefix(u + lane, c);
+                    const bool on = u + lane < U.n;
+                    if (small) fold_points<true>(net, Q, S, pf, c, on, U.pf32, ta, te, acc, out, out_level, (unsigned)q);
+                    else fold_points<false>(net, Q, S, pf, c, on, U.pf32, ta, te, acc, out, out_level, (unsigned)q);
+                }
+                acc.flush(Q.cnt);
             }
         }
-        const unsigned adv = __reduce_add_sync(0xffffffffu, acc.adv), pts = __reduce_add_sync(0xffffffffu, acc.pts);
-        if (adv) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long f = __shfl_xor_sync(0xffffffffu, acc.first, o);
-                acc.first = f < acc.first ? f : acc.first;
-            }
-            if (lane == 0) {
-                atomicAdd(&Q.cnt->n_adv, (unsigned long long)adv);
-                atomicMin(&Q.cnt->first, acc.first);
-            }
-        }
-        if (pts && lane == 0) atomicAdd(&Q.cnt->n_points, (unsigned long long)pts);
         __syncthreads();  // every push of the segment is out
     };
     if (nq == 1) {
