@@ -293,8 +293,9 @@ __global__ void __launch_bounds__(32 * (WPN > 8 ? WPN : 8)) k_pro_layer(NetView 
     const int s = Q.s;
     float2* row = Q.fco + (size_t)n * Q.fstride;
     float B = 0.f;  // sum of |coefficient| x bound of its source (over lanes of the first warp)
-    // the rows of the layer below carry errors fer; a pair sum over npos inputs, split
-    // over lanes and warps, adds at most (npos + 32) 2^-45 sum_j |w_j| B_j
+    // the rows of the layer below carry errors fer; a pair sum over npos inputs adds at
+    // most (6.5 npos + 20) 2^-48 sum_j |w_j| B_j (PairSum), and joining its parts over
+    // lanes and warps, in at most 14 steps, 42 2^-48 of it: below (npos + 32) 2^-45
     const float er = l == 1 ? 0.f : __fmaf_ru((float)(npos + 32) * 0x1p-45f, b[3], b[2]);
     if (l == 1) {
         if (wn == 0 && lane < s) {
@@ -310,21 +311,24 @@ __global__ void __launch_bounds__(32 * (WPN > 8 ? WPN : 8)) k_pro_layer(NetView 
             while (sp < 32 && sp < S - k0) sp <<= 1;
             const int per = 32 / sp;
             const int k = k0 + (lane & (sp - 1)), g = wn * per + lane / sp, G = WPN * per;
-            float2 a = make_float2(0.f, 0.f);
+            PairSum sum;
             if (k < S) {
-#pragma unroll 8
-                for (int jj = g; jj < npos; jj += G) {
-                    const int j = plist[jj];
-                    const float w = Wr[j];
-                    const float2 h = prev[(size_t)j * Q.fstride + k];
-                    const float pr = __fmul_rn(w, h.x);
-                    float ep = __fmaf_rn(w, h.x, -pr);
-                    ep = __fmaf_rn(w, h.y, ep);
-                    const float2 t = two_sum(a.x, pr);
-                    a = make_float2(t.x, __fadd_rn(a.y, __fadd_rn(t.y, ep)));
+                for (int jj = g; jj < npos; jj += kSettle * G) {
+                    float w[kSettle];
+                    float2 h[kSettle];
+#pragma unroll
+                    for (int e = 0; e < kSettle; ++e) {  // in flight together, also the last few
+                        const bool in = jj + e * G < npos;
+                        const int j = plist[in ? jj + e * G : jj];
+                        w[e] = in ? Wr[j] : 0.f;
+                        h[e] = prev[(size_t)j * Q.fstride + k];
+                    }
+#pragma unroll
+                    for (int e = 0; e < kSettle; ++e) sum.add(w[e], h[e]);
+                    sum.settle();
                 }
-                a = two_sum(a.x, a.y);
             }
+            float2 a = sum.a;
             for (int o = sp; o < 32; o <<= 1)
                 a = df_add(a, make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o)));
             if (WPN > 1) {
