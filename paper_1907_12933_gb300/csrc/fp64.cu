@@ -84,9 +84,11 @@ k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__
         n = range_hi - range_lo;
     }
     const int L = net.L;
-    const unsigned rank = CL > 1 ? cluster_rank() : 0u;
-    if (CL > 1 && n > 0) cluster_barrier();  // every CTA of the cluster has started
-    for (unsigned long long e = blockIdx.x / CL; e < n; e += gridDim.x / CL) {
+    // more points than clusters: a CTA per point after all (the same choice in every CTA)
+    const bool solo = CL == 1 || n > gridDim.x / CL;
+    const unsigned parts = solo ? 1u : CL, rank = solo ? 0u : cluster_rank();
+    if (!solo && n > 0) cluster_barrier();  // every CTA of the cluster has started
+    for (unsigned long long e = blockIdx.x / parts; e < n; e += gridDim.x / parts) {
         unsigned long long t;
         int qi;
         if (gather) {
@@ -133,14 +135,16 @@ k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__
             const int off = net.noff[l];
             const double* h = h0 + (size_t)((l - 1) % HB) * hmax;
             double* const hn = h0 + (size_t)(l % HB) * hmax;
-            // 32 neurons a warp, the cluster's CTAs in turn
-            for (int i = (int)((threadIdx.x >> 5) * CL + rank) * 32 + (int)(threadIdx.x & 31); i < N; i += T64 * CL) {
+            // 32 neurons a warp, the point's CTAs in turn
+            for (int i = (int)((threadIdx.x >> 5) * parts + rank) * 32 + (int)(threadIdx.x & 31); i < N;
+                 i += (int)(T64 * parts)) {
                 double a = 0.0;
 #pragma unroll 16
                 for (int j = 0; j < K; ++j) a += widen(__ldg(WT + (size_t)j * N + i)) * h[j];
                 const double v = a + (double)b[i];
-                if (CL == 1) {
+                if (solo) {
                     u[off + i] = v;
+                    if (HB > 1 && l < L) hn[i] = act64(net.act, v);
                 } else {
                     store_cluster(u + off + i, 0u, v);
                     if (l < L) {
@@ -149,16 +153,18 @@ k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__
                     }
                 }
             }
-            if (CL > 1) {
+            if (!solo) {
                 cluster_barrier();
             } else {
                 __syncthreads();
-                if (l < L)
-                    for (int i = threadIdx.x; i < N; i += T64) hn[i] = act64(net.act, u[off + i]);
-                __syncthreads();
+                if (HB == 1) {  // layer l's outputs take the place of its inputs
+                    if (l < L)
+                        for (int i = threadIdx.x; i < N; i += T64) hn[i] = act64(net.act, u[off + i]);
+                    __syncthreads();
+                }
             }
         }
-        if (CL == 1 || rank == 0) {
+        if (rank == 0) {
             // signs, ties, changes
             for (int nn = threadIdx.x; nn < total; nn += T64) {
                 const double ub = Q.ub[nn], ut = u[nn];
@@ -227,7 +233,7 @@ k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__
                 if (gather) work_done(Q.cnt, 1);  // time to verdict: this queued point is resolved
             }
         }
-        if (CL == 1) __syncthreads();
+        if (solo) __syncthreads();
         else cluster_barrier();  // the first CTA has read what the next point's layers write
     }
 }
@@ -295,12 +301,12 @@ void launch_fp64(const NetView& net, const QueryView* d_qs, int nq, const QEntry
                  const unsigned long long* gather_count, unsigned long long gather_cap,
                  unsigned long long range_lo, unsigned long long range_hi, int n_sm,
                  cudaStream_t st) {
-    constexpr int CL = 8;
+    constexpr int CL = 8, kGatherCtas = 8;
     auto smem = [&](int buffers) { return sizeof(double) * (net.total + buffers * (size_t)net.hmax) + 2 * (size_t)net.total; };
-    if (gather && smem(2) <= 200 * 1024 && n_sm * 2 >= CL) {
+    if (gather && smem(2) <= 200 * 1024 && n_sm * kGatherCtas >= CL) {
         cudaFuncSetAttribute(k_fp64<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(2));
         cudaLaunchConfig_t c{};
-        c.gridDim = (unsigned)(n_sm * 2 / CL * CL);
+        c.gridDim = (unsigned)(n_sm * kGatherCtas / CL * CL);
         c.blockDim = T64;
         c.dynamicSmemBytes = smem(2);
         c.stream = st;
