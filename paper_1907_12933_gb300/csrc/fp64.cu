@@ -13,13 +13,18 @@
 //     tie and exactly one change (j) and i changes without tie; pairs that
 //     hold only under some resolution of the ties go to the SS-tie mask.
 //
-// A range has a CTA per point. Queued points are few, and one CTA is bound by its SM's
+// A range has a CTA per point. Queued points are mostly few, and one CTA is bound by its SM's
 // FP64 pipe (16 cycles a warp instruction: two layers of 1024 take 1.3 ms), so a cluster
 // of CL CTAs shares a point: a layer's neurons are dealt to the cluster's warps, their
 // outputs go to every CTA's shared memory, and the first CTA does the rest. A weight
 // becomes FP64 by its bits, not on that pipe. The sums keep their order. One queued
 // point of 784-1024x3-10: 1,375 -> 380 us, now bound by the chain of dependent FP64 sums
 // (weights loaded a block ahead: 380 us too, and ranges of small nets 11.1 -> 16.6 ms).
+// A queue that holds more points than the launch has clusters fills the chip with a CTA
+// per point: a dead neuron or two equal outputs send every point here, and clusters then
+// wait at their barriers more than they compute (whole calls, 4,913 such points on 25-10-5
+// 1,700 us by clusters, 430 a CTA each; on 784-512-512-10, sigmoid, 19.2 and 8.2 ms; 289
+// points on it 1,730 and 1,200 us).
 #include "dev.cuh"
 #include "launch.h"
 
@@ -301,6 +306,9 @@ void launch_fp64(const NetView& net, const QueryView* d_qs, int nq, const QEntry
                  const unsigned long long* gather_count, unsigned long long gather_cap,
                  unsigned long long range_lo, unsigned long long range_hi, int n_sm,
                  cudaStream_t st) {
+    // 8 CTAs per SM, most of them resident: with 6 or 4 the last points of a long queue leave
+    // the chip idle (25-10-5, 83,521 points: 5.0 ms, 5.3 with 6; sigmoid 784-512-512-10,
+    // 4,913 points: 8.2 ms, 9.0 with 4)
     constexpr int CL = 8, kGatherCtas = 8;
     auto smem = [&](int buffers) { return sizeof(double) * (net.total + buffers * (size_t)net.hmax) + 2 * (size_t)net.total; };
     if (gather && smem(2) <= 200 * 1024 && n_sm * kGatherCtas >= CL) {
