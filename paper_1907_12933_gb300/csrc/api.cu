@@ -868,6 +868,7 @@ vbmc_status enqueue(vbmc_net* net, vbmc_result* r, const uint8_t* d_image, const
                     int k, uint64_t lo, uint64_t hi, uint64_t n, const vbmc_options& opt,
                     cudaStream_t st, const QueryExtra& x = QueryExtra(), bool fold = true, bool wait = false) {
     QueryView q = make_view(r, d_image, d_pix, s, k, lo, hi, n, opt, 0, x, fold);
+    if (d_image != r->d_image) q.image_keep = r->d_image;
     q.budget_ns = opt.time_budget_ms > 0.0 ? (unsigned long long)(opt.time_budget_ms * 1e6) : 0ull;
     std::vector<unsigned long long> tp = tile_prefix(net->v, opt.precision, &q, 1);
     // the first pass takes its tiles from the claim counter on the fused tensor
@@ -1006,6 +1007,7 @@ extern "C" vbmc_status vbmc_verify_query_device(vbmc_net* net, const uint8_t* d_
     if (st != VBMC_OK) return st;
     res->image.clear();
     res->pixels.clear();
+    res->hq.image = nullptr;  // the witness is made from the copy that the call keeps (d_image)
     return enqueue(net, res, d_image, d_pixels, s, k, lo, h, n, *opt, (cudaStream_t)stream);
 }
 

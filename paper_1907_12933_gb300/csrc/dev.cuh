@@ -107,6 +107,7 @@ struct QueryView {
     unsigned long long budget_ns;         // time budget of the call from the query's prologue
                                           // (0: none); see claim_tile
     const uint8_t* image;   // H_0 grey levels (device)
+    uint8_t* image_keep;    // where the set-up copies a caller's device image to (nullptr: nowhere)
     const int* pix_in;      // s pixel indices as given (device)
     int* pix;               // validated copy
     int* dv;                // [s][R]: clamp(v_p + d - k, 0, 255) - v_p

@@ -54,6 +54,8 @@ __global__ void k_pro_init(NetView net, QueryView* qs, int nq) {
             if (Q.fst) Q.fst[0] = Q.fst[1] = 0;
         }
     }
+    if (Q.image_keep && blockIdx.y == 0)
+        for (int j = threadIdx.x; j < H0; j += blockDim.x) Q.image_keep[j] = Q.image[j];
     // results start from zero on every call
     const int nb = gridDim.y, bt = blockIdx.y * blockDim.x + threadIdx.x, nt = nb * blockDim.x;
     if (Q.flip)
