@@ -643,13 +643,16 @@ enum { STAGE_SETUP = 1, STAGE_PASSES = 2, STAGE_ALL = 3 };
 // whether the query folded and launches the passes of that form only. Without it both
 // forms are launched and each leaves the other's queries out (about 20 us of launches
 // that return at once).
+// fold_part (one query; 0: none): the folded net takes its points in parts of so many, and
+// finishes each before the next, so that whatever it leaves undecided fits the queues.
 vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, int nq,
                            const unsigned long long* d_tp, unsigned long long ntiles,
                            unsigned long long* d_qcount, QEntry* const* d_queue,
                            unsigned long long cap, const cudaEvent_t* ev, const vbmc_options& opt,
                            cudaStream_t st, bool capturing = false, int stages = STAGE_ALL,
                            WideWork* ww = nullptr, TcQueryWork* tw = nullptr,
-                           unsigned long long* d_claim = nullptr, int* h_folded = nullptr) {
+                           unsigned long long* d_claim = nullptr, int* h_folded = nullptr,
+                           uint64_t fold_part = 0) {
     if (nq != 1) tw = nullptr;  // compacted columns are per query: single-query calls only
     const NetView& v = net->v;
     // inside a stream capture an event record must be an explicit graph node
@@ -746,11 +749,19 @@ vbmc_status enqueue_passes(vbmc_net* net, QueryView* d_qs, const QueryView* hq, 
         const int mt = opt.precision == VBMC_PREC_FP32 ? simt_tile_points(v) : tc_tile_points();
         const bool whole = wide && nq == 1;
         if (whole) ntiles = (hq[0].hi - (hq[0].lo & ~31ull) + mt - 1) / mt;
-        launch_fold(v, d_qs, nq, whole ? nullptr : d_tp, ntiles, mt, !wide, whole || !d_claim ? nullptr : d_claim + 1,
-                    qsplit, 0, net->n_sm, st);
+        uint64_t lo = hq[0].lo;
+        for (; nq == 1 && fold_part && hq[0].hi - lo > fold_part; lo += fold_part) {
+            launch_fold(v, d_qs, 1, lo, lo + fold_part, nullptr, 0, mt, false, nullptr, qsplit, 0, net->n_sm, st);
+            launch_fold64(v, d_qs, d_queue[0], d_qcount + 0, cap, q64, 3, net->n_sm, st);
+            launch_fp64(v, d_qs, 1, d_queue[3], d_qcount + 3, cap, 0, 0, net->n_sm, st);
+            VB_CUDA(cudaMemsetAsync(d_qcount, 0, sizeof(unsigned long long) * 4, st));
+        }
+        launch_fold(v, d_qs, nq, lo, hq[0].hi, whole ? nullptr : d_tp, ntiles, mt, !wide,
+                    whole || !d_claim ? nullptr : d_claim + 1, qsplit, 0, net->n_sm, st);
         launch_fold64(v, d_qs, d_queue[0], d_qcount + 0, cap, q64, 3, net->n_sm, st);
         if (!general) {  // (the passes in between take no time, see finish)
             VB_CUDA(record(ev[2]));
+            if (!h_folded) VB_CUDA(record_rest());
             launch_fp64(v, d_qs, nq, d_queue[3], d_qcount + 3, cap, 0, 0, net->n_sm, st);
             if (whole) wide_done(d_qs, st);
         }
@@ -862,11 +873,23 @@ QueryView make_view(const vbmc_result* r, const uint8_t* d_image, const int* d_p
     return q;
 }
 
+// Points that the folded net takes at a time where a call cannot try them all at once and
+// go back when the queues overflow (0: it does not fold). A part is 3 to 5 launches; below
+// 2^16 points (1 us of k_fold's work) the general passes are left to it, whose overflow is then
+// the call's.
+uint64_t fold_part_of(const vbmc_result* r, uint64_t points) {
+    const uint64_t cap = std::max<uint64_t>(1, r->caps.queue_cap);
+    return points <= cap || cap >= (1ull << 16) ? cap : 0;
+}
+
 // Enqueue the full pipeline for one query whose image/pixels are on the device. wait:
-// the caller waits for the result anyway (see h_folded of enqueue_passes).
+// the caller waits for the result anyway (see h_folded of enqueue_passes), and calls again
+// without it when the folded net's undecided points overflowed the queues.
 vbmc_status enqueue(vbmc_net* net, vbmc_result* r, const uint8_t* d_image, const int* d_pix, int s,
                     int k, uint64_t lo, uint64_t hi, uint64_t n, const vbmc_options& opt,
                     cudaStream_t st, const QueryExtra& x = QueryExtra(), bool fold = true, bool wait = false) {
+    const uint64_t part = wait ? 0 : fold_part_of(r, hi - lo);
+    if (!wait && !part) fold = false;
     QueryView q = make_view(r, d_image, d_pix, s, k, lo, hi, n, opt, 0, x, fold);
     if (d_image != r->d_image) q.image_keep = r->d_image;
     q.budget_ns = opt.time_budget_ms > 0.0 ? (unsigned long long)(opt.time_budget_ms * 1e6) : 0ull;
@@ -895,7 +918,7 @@ vbmc_status enqueue(vbmc_net* net, vbmc_result* r, const uint8_t* d_image, const
     vbmc_status sst = enqueue_passes(net, r->d_q, &q, 1, r->d_tp, tp[1], r->d_qcount, r->d_queue,
                                      std::max<uint64_t>(1, r->caps.queue_cap), ev, opt, st, false, STAGE_ALL,
                                      &r->ww, r->have_tw ? &r->tw : nullptr, claims ? r->d_claim : nullptr,
-                                     h_folded);
+                                     h_folded, part);
     r->one_form = h_folded && *h_folded;
     if (sst != VBMC_OK) {
         if (r->h_in) cudaStreamSynchronize(st);  // the pinned block has been read
@@ -1048,7 +1071,13 @@ vbmc_status verify_query(vbmc_net* net, const vbmc_query* q, const vbmc_options*
     if (st != VBMC_OK) return st;
     res->image.assign(q->image, q->image + H0);
     res->pixels.assign(q->pixels, q->pixels + q->s);
-    return finish(res);
+    st = finish(res);
+    if (res->one_form && (res->h_cnt->err & DERR_QUEUE)) {
+        st = enqueue(net, res, res->d_image, res->d_pix_in, q->s, q->k, q->lo, h, n, *opt, stq, x, fold);
+        if (st != VBMC_OK) return st;
+        st = finish(res);
+    }
+    return st;
 }
 
 }  // namespace
@@ -1171,9 +1200,10 @@ extern "C" vbmc_status vbmc_get_ties(vbmc_result* res, uint64_t* idx, size_t cap
     return VBMC_OK;
 }
 
-extern "C" vbmc_status vbmc_verify_batch(vbmc_net* net, const vbmc_query* queries, int32_t nq,
-                                         const vbmc_options* opt, vbmc_result* const* results,
-                                         void* stream) {
+namespace {
+
+vbmc_status verify_batch(vbmc_net* net, const vbmc_query* queries, int32_t nq, const vbmc_options* opt,
+                         vbmc_result* const* results, void* stream, bool fold) {
     if (!net || (!queries && nq > 0) || !opt || (!results && nq > 0))
         return fail(VBMC_ERR_ARG, "null argument");
     if (nq == 0) return VBMC_OK;
@@ -1228,7 +1258,7 @@ extern "C" vbmc_status vbmc_verify_batch(vbmc_net* net, const vbmc_query* querie
         QueryExtra x;
         const vbmc_status xs = query_extra(q, &x);
         if (xs != VBMC_OK) return xs;
-        hq[i] = make_view(r, d_img, d_pix, q.s, q.k, q.lo, h, n, *opt, i, x);
+        hq[i] = make_view(r, d_img, d_pix, q.s, q.k, q.lo, h, n, *opt, i, x, fold);
         nsp[i] = n;
     }
     std::vector<unsigned long long> tp = tile_prefix(v, opt->precision, hq.data(), nq);
@@ -1338,6 +1368,9 @@ extern "C" vbmc_status vbmc_verify_batch(vbmc_net* net, const vbmc_query* querie
     }
     VB_CUDA(cudaMemcpyAsync(ar->h_cnt, ar->d_cnt, sizeof(Counters) * (size_t)nq, cudaMemcpyDeviceToHost, st));
     VB_CUDA(cudaStreamSynchronize(st));
+    for (int i = 0; i < nq; ++i)  // the folded nets' undecided points may not fit the queues
+        if (hq[i].fold && (ar->h_cnt[i].err & DERR_QUEUE))
+            return verify_batch(net, queries, nq, opt, results, stream, false);
     float ms = 0.f, ms_p = 0.f, ms_s = 0.f;
     cudaEventElapsedTime(&ms, ar->ev[0], ar->ev[3]);
     cudaEventElapsedTime(&ms_p, ar->ev[0], ar->ev[1]);
@@ -1372,6 +1405,14 @@ extern "C" vbmc_status vbmc_verify_batch(vbmc_net* net, const vbmc_query* querie
         if (r->last_status != VBMC_OK && result == VBMC_OK) result = r->last_status;
     }
     return result;
+}
+
+}  // namespace
+
+extern "C" vbmc_status vbmc_verify_batch(vbmc_net* net, const vbmc_query* queries, int32_t nq,
+                                         const vbmc_options* opt, vbmc_result* const* results,
+                                         void* stream) {
+    return verify_batch(net, queries, nq, opt, results, stream, true);
 }
 
 namespace vbmc {
@@ -1460,9 +1501,10 @@ extern "C" vbmc_status vbmc_wide_trace(vbmc_net* net, const vbmc_query* q, int32
     return st;
 }
 
-extern "C" vbmc_status vbmc_search_query(vbmc_net* net, const vbmc_query* q, int32_t n_tiles,
-                                         const int32_t* order, const vbmc_options* opt, vbmc_result* res,
-                                         vbmc_search_out* out, void* stream) {
+namespace {
+
+vbmc_status search_query(vbmc_net* net, const vbmc_query* q, int32_t n_tiles, const int32_t* order,
+                         const vbmc_options* opt, vbmc_result* res, vbmc_search_out* out, void* stream, bool fold) {
     if (!net || !q || !res || !opt || !order || !q->image || (!q->pixels && q->s > 0))
         return fail(VBMC_ERR_ARG, "null argument");
     if (res->net != net) return fail(VBMC_ERR_ARG, "result belongs to another net");
@@ -1497,7 +1539,7 @@ extern "C" vbmc_status vbmc_search_query(vbmc_net* net, const vbmc_query* q, int
     QueryExtra x;
     st = query_extra(*q, &x);
     if (st != VBMC_OK) return st;
-    QueryView qv = make_view(res, res->d_image, res->d_pix_in, q->s, q->k, 0, n, n, *opt, 0, x);
+    QueryView qv = make_view(res, res->d_image, res->d_pix_in, q->s, q->k, 0, n, n, *opt, 0, x, fold);
     std::vector<unsigned long long> tp = tile_prefix(net->v, opt->precision, &qv, 1);
     VB_CUDA(cudaMemcpyAsync(res->d_q, &qv, sizeof(QueryView), cudaMemcpyHostToDevice, sq));
     const cudaEvent_t ev_set[7] = {res->ev0,    res->ev_pro, res->ev_pro, res->ev_pro,
@@ -1600,13 +1642,15 @@ extern "C" vbmc_status vbmc_search_query(vbmc_net* net, const vbmc_query* q, int
                                 sq));
         st = enqueue_passes(net, res->d_q, &qv, 1, res->d_tp, tp[1], res->d_qcount, res->d_queue, cap, ev_tile,
                             *opt, sq, false, STAGE_PASSES, &res->ww, res->have_tw ? &res->tw : nullptr, nullptr,
-                            h_folded);
+                            h_folded, fold_part_of(res, hi - lo));
         if (st != VBMC_OK) return st;
         any_tile = true;
         VB_CUDA(cudaMemcpyAsync(res->h_cnt, res->d_cnt, sizeof(Counters), cudaMemcpyDeviceToHost, sq));
         VB_CUDA(cudaStreamSynchronize(sq));
         so.points_checked += hi - lo;
         run = counters_status(*res->h_cnt);
+        if (*h_folded && (res->h_cnt->err & DERR_QUEUE))  // a tile too large for the queues
+            return search_query(net, q, n_tiles, order, opt, res, out, stream, false);
         if (run != VBMC_OK) break;
         if (res->h_cnt->n_adv > 0) {
             so.witness_tile = order[i];
@@ -1643,6 +1687,14 @@ extern "C" vbmc_status vbmc_search_query(vbmc_net* net, const vbmc_query* q, int
     res->last_status = run;
     if (out) *out = so;
     return run;
+}
+
+}  // namespace
+
+extern "C" vbmc_status vbmc_search_query(vbmc_net* net, const vbmc_query* q, int32_t n_tiles,
+                                         const int32_t* order, const vbmc_options* opt, vbmc_result* res,
+                                         vbmc_search_out* out, void* stream) {
+    return search_query(net, q, n_tiles, order, opt, res, out, stream, true);
 }
 
 extern "C" vbmc_status vbmc_tile_counts(vbmc_result* res, int32_t n_tiles, uint64_t* counts) {

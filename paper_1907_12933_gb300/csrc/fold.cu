@@ -628,6 +628,7 @@ __device__ __forceinline__ void fold_points(const NetView& net, const QueryView&
 // k = 7 (11.4 M points) 356 -> 199 us, 784-1024x3-10, s = 4, k = 15 337 -> 97 us, the
 // last wave of 64 queries on 784-256-256-10 1,255 -> 665 us.
 __global__ void __launch_bounds__(FT, 2) k_fold(NetView net, const QueryView* __restrict__ qs, int nq,
+                                                unsigned long long lo, unsigned long long hi,
                                                 const unsigned long long* __restrict__ tile_prefix,
                                                 unsigned long long ntiles, int mt, int group, int work_units,
                                                 unsigned long long* claim, Queue out, int out_level) {
@@ -710,7 +711,7 @@ __global__ void __launch_bounds__(FT, 2) k_fold(NetView net, const QueryView* __
     if (nq == 1) {
         load(0);
         // consecutive pieces go to different CTAs, so that a small range spreads
-        segment(0, qs[0].lo, qs[0].hi, 32ull * (blockIdx.x + gridDim.x * (unsigned)warp), 32ull * gridDim.x * FW);
+        segment(0, lo, hi, 32ull * (blockIdx.x + gridDim.x * (unsigned)warp), 32ull * gridDim.x * FW);
         flush();
         __syncthreads();
         if (threadIdx.x == 0 && work_units)  // the launch's share of the query's tiles
@@ -930,9 +931,9 @@ void launch_fold_pack(const NetView& net, QueryView* d_qs, int nq, cudaStream_t 
     launch_chained(k_fold_pack, nq, kPackT, 0, st, net, d_qs, d_unfolded);
 }
 
-void launch_fold(const NetView& net, const QueryView* d_qs, int nq, const unsigned long long* d_tile_prefix,
-                 unsigned long long n_tiles, int mt, bool work_units, unsigned long long* claim, Queue out,
-                 int out_level, int n_sm, cudaStream_t st) {
+void launch_fold(const NetView& net, const QueryView* d_qs, int nq, unsigned long long lo, unsigned long long hi,
+                 const unsigned long long* d_tile_prefix, unsigned long long n_tiles, int mt, bool work_units,
+                 unsigned long long* claim, Queue out, int out_level, int n_sm, cudaStream_t st) {
     cudaFuncSetAttribute(k_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FoldSm));
     const unsigned long long ctas = (unsigned long long)n_sm * 2;
     // one query: a warp for every 32 units of up to 4 points, as many as fit. Many: a claim
@@ -940,10 +941,10 @@ void launch_fold(const NetView& net, const QueryView* d_qs, int nq, const unsign
     const unsigned long long per_round = (unsigned long long)(FT * FP / mt);
     unsigned long long group = std::min<unsigned long long>(n_tiles / (ctas * 2), 16 * per_round);
     if (group < 1) group = 1;
-    unsigned long long grid = nq == 1 ? (n_tiles * (unsigned)mt + 95) / 96 : (n_tiles + group - 1) / group;
+    unsigned long long grid = nq == 1 ? (hi - lo + 127) / 96 : (n_tiles + group - 1) / group;
     if (grid > ctas) grid = ctas;
     if (grid < 1) grid = 1;
-    launch_chained(k_fold, (unsigned)grid, FT, sizeof(FoldSm), st, net, d_qs, nq, d_tile_prefix, n_tiles, mt,
+    launch_chained(k_fold, (unsigned)grid, FT, sizeof(FoldSm), st, net, d_qs, nq, lo, hi, d_tile_prefix, n_tiles, mt,
                    (int)group, work_units ? 1 : 0, claim, out, out_level);
 }
 

@@ -40,12 +40,12 @@ void launch_prologue_screens(const NetView& net, QueryView* d_qs, int nq, int ma
 bool fold_supported(const NetView& net);
 size_t fold_coeff_entries(const NetView& net, int max_s);  // float4 entries of QueryView::fc32
 void launch_fold_pack(const NetView& net, QueryView* d_qs, int nq, cudaStream_t st, unsigned long long* d_unfolded);
-// Tiles of mt points, numbered as in the general first pass (d_tile_prefix; null
-// with one query); work_units: the queries' work counts are in these tiles;
-// claim: tile counter (many queries).
-void launch_fold(const NetView& net, const QueryView* d_qs, int nq, const unsigned long long* d_tile_prefix,
-                 unsigned long long n_tiles, int mt, bool work_units, unsigned long long* claim, Queue out,
-                 int out_level, int n_sm, cudaStream_t st);
+// One query: its points [lo, hi). Many: tiles of mt points, numbered as in the general
+// first pass (d_tile_prefix, claim: tile counter). n_tiles: tiles of the launch, which its
+// end takes from the queries' work counts where those are in tiles (work_units).
+void launch_fold(const NetView& net, const QueryView* d_qs, int nq, unsigned long long lo, unsigned long long hi,
+                 const unsigned long long* d_tile_prefix, unsigned long long n_tiles, int mt, bool work_units,
+                 unsigned long long* claim, Queue out, int out_level, int n_sm, cudaStream_t st);
 void launch_fold64(const NetView& net, const QueryView* d_qs, const QEntry* in, const unsigned long long* count,
                    unsigned long long cap, Queue out, int out_level, int n_sm, cudaStream_t st);
 // FP64 margin of point t of query 0 into *d_out where it folded (nothing otherwise).
