@@ -422,7 +422,7 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
     q.ss_tie = q.ss + v.ss_words;
     A(&q.ties, (size_t)std::max<uint32_t>(1, caps->ties_cap));
     if (arena) A(&r->d_qcount, 4);
-    A(&r->d_margin, 1);
+    A(&r->d_margin, 1 + 2 * (size_t)v.hmax);  // and the outputs of two layers
     if (caps->max_points) A(&q.bitmap, (size_t)((caps->max_points + 31) / 32));
     // members of a batch keep small queues of their own (the batch shares the arena's)
     uint64_t qc = std::max<uint64_t>(1, caps->queue_cap);

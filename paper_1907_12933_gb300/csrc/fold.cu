@@ -905,16 +905,6 @@ __global__ void __launch_bounds__(32 * F64W) k_fold64(NetView net, const QueryVi
     }
 }
 
-// FP64 margin of one point of query 0, where it folded (k_margin64 otherwise).
-__global__ void __launch_bounds__(32) k_fold_margin(NetView net, const QueryView* __restrict__ qs,
-                                                    unsigned long long t, double* out) {
-    __shared__ Fold64 F;
-    if (!folded(qs[0])) return;
-    double m;
-    fold64_point(net, qs[0], F, t, threadIdx.x, &m);
-    if (threadIdx.x == 0) *out = m;
-}
-
 }  // namespace
 
 bool fold_supported(const NetView& net) {
@@ -951,11 +941,6 @@ void launch_fold(const NetView& net, const QueryView* d_qs, int nq, unsigned lon
 void launch_fold64(const NetView& net, const QueryView* d_qs, const QEntry* in, const unsigned long long* count,
                    unsigned long long cap, Queue out, int out_level, int n_sm, cudaStream_t st) {
     launch_chained(k_fold64, (unsigned)n_sm * 4, 32 * F64W, 0, st, net, d_qs, in, count, cap, out, out_level);
-}
-
-void launch_fold_margin(const NetView& net, const QueryView* d_qs, unsigned long long t, double* d_out,
-                        cudaStream_t st) {
-    k_fold_margin<<<1, 32, 0, st>>>(net, d_qs, t, d_out);
 }
 
 }  // namespace vbmc

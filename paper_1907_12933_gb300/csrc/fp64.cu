@@ -243,63 +243,82 @@ k_fp64(NetView net, const QueryView* __restrict__ qs, const QEntry* __restrict__
     }
 }
 
-// FP64 margin of one point (for witnesses): y_D - max_{i != D} y_i.
-__global__ void __launch_bounds__(T64)
-k_margin64(NetView net, const QueryView* __restrict__ qs, unsigned long long t, double* out) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double* u = reinterpret_cast<double*>(smem_raw);
-    double* h = u + net.total;
-    __shared__ int dstep[kMaxS];
+// Potential i of layer l at the point whose pixel changes are the lanes' x (lane p: pixel
+// p's dv / 255), from layer l - 1's outputs h: a warp, its lanes over the inputs, so that a
+// sum passes K / 32 + 6 roundings.
+__device__ __forceinline__ double warp_potential(const NetView& net, const QueryView& Q, int l, int i, double x,
+                                                 const double* h) {
+    const int lane = threadIdx.x & 31, K = net.dims[l - 1];
+    double a = 0.0;
+    if (l == 1) {
+        if (lane < Q.s) a = (double)net.W[1][(size_t)i * K + Q.pix[lane]] * x;
+    } else {
+        const float* w = net.W[l] + (size_t)i * K;
+#pragma unroll 8
+        for (int j = lane; j < K; j += 32) a = fma(widen(__ldg(w + j)), h[j], a);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a + (l == 1 ? Q.ub[i] : (double)net.b[l][i]);
+}
+
+// dv / 255 of pixel `lane` at point t.
+__device__ __forceinline__ double lane_change(const QueryView& Q, unsigned long long t) {
+    int d[kMaxS];
+    decode_digits(t, Q.s, Q.R, d);
+    double x = 0.0;
+    for (int p = 0; p < Q.s; ++p)
+        if ((int)(threadIdx.x & 31) == p) x = (double)Q.dv[p * Q.R + d[p]] / 255.0;
+    return x;
+}
+
+// Outputs of hidden layer l at point t of query 0 into out, a warp per neuron.
+__global__ void __launch_bounds__(T64) k_margin_layer(NetView net, const QueryView* qs, int l, unsigned long long t,
+                                                      const double* h, double* out) {
+    const int i = blockIdx.x * (T64 / 32) + (threadIdx.x >> 5);
+    chain_wait();
+    chain_next();
+    if (i >= net.dims[l]) return;
     const QueryView& Q = qs[0];
-    if (folded(Q)) return;  // launch_fold_margin wrote it
-    const int L = net.L;
-    if (threadIdx.x == 0) {
-        int d[kMaxS];
-        decode_digits(t, Q.s, Q.R, d);
-        for (int p = 0; p < Q.s; ++p) dstep[p] = Q.dv[p * Q.R + d[p]];
+    const double u = warp_potential(net, Q, l, i, l == 1 ? lane_change(Q, t) : 0.0, h);
+    if ((threadIdx.x & 31) == 0) out[i] = act64(net.act, u);
+}
+
+// The output layer, and the FP64 margin: y_D - max_{i != D} y_i (Eq. 10), or Eq. 11's.
+__global__ void __launch_bounds__(1024) k_margin_out(NetView net, const QueryView* qs, unsigned long long t,
+                                                     const double* h, double* out) {
+    __shared__ double y[kMaxWidth];
+    chain_wait();
+    const QueryView& Q = qs[0];
+    const int L = net.L, HL = net.dims[L];
+    const double x = L == 1 ? lane_change(Q, t) : 0.0;
+    for (int i = threadIdx.x >> 5; i < HL; i += 32) {
+        const double u = warp_potential(net, Q, L, i, x, h);
+        if ((threadIdx.x & 31) == 0) y[i] = u;
     }
     __syncthreads();
-    const int H0 = net.dims[0], H1 = net.dims[1];
-    for (int j = threadIdx.x; j < H1; j += T64) {
-        double a = Q.ub[j];
-        for (int p = 0; p < Q.s; ++p)
-            a += (double)net.W[1][(size_t)j * H0 + Q.pix[p]] * ((double)dstep[p] / 255.0);
-        u[j] = a;
-        h[j] = (L > 1) ? act64(net.act, a) : a;
-    }
-    __syncthreads();
-    for (int l = 2; l <= L; ++l) {
-        const int K = net.dims[l - 1], N = net.dims[l];
-        for (int i = threadIdx.x; i < N; i += T64) {
-            double a = 0.0;
-            for (int j = 0; j < K; ++j) a += (double)net.WT[l][(size_t)j * N + i] * h[j];
-            u[net.noff[l] + i] = a + (double)net.b[l][i];
-        }
-        __syncthreads();
-        if (l < L)
-            for (int i = threadIdx.x; i < N; i += T64) h[i] = act64(net.act, u[net.noff[l] + i]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const double* y = u + net.noff[L];
-        const int D = Q.cnt->D;
-        double mx = -DBL_MAX;
-        for (int i = 0; i < net.dims[L]; ++i)
-            if (i != D && y[i] > mx) mx = y[i];
-        *out = Q.prop == PROP_THRESHOLD ? fmax(y[D] - Q.V, Q.V - mx) : y[D] - mx;
-    }
+    if (threadIdx.x >= 32) return;
+    const int D = Q.cnt->D;
+    double mx = -DBL_MAX;
+    for (int i = threadIdx.x; i < HL; i += 32)
+        if (i != D && y[i] > mx) mx = y[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (threadIdx.x == 0) *out = Q.prop == PROP_THRESHOLD ? fmax(y[D] - Q.V, Q.V - mx) : y[D] - mx;
 }
 
 }  // namespace
 
 void launch_margin64(const NetView& net, const QueryView* d_qs, unsigned long long t, double* d_out,
                      cudaStream_t st) {
-    // one CTA walks the whole net (239 us on 784-512-512-10); a folded query's margin
-    // comes from its folded rows, one warp (about 10 us)
-    if (fold_supported(net)) launch_fold_margin(net, d_qs, t, d_out, st);
-    const size_t smem = sizeof(double) * (net.total + net.hmax);
-    cudaFuncSetAttribute(k_margin64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_margin64<<<1, T64, smem, st>>>(net, d_qs, t, d_out);
+    // a launch per layer, its neurons over the chip. The getter's whole call: 784-512-512-10
+    // 38 us, 784-1024x3-10 53 us (one CTA that walks the whole net, a thread per neuron: the
+    // kernel alone 239, the call 1,286; the rows of a folded net, in FP32 pairs: 63)
+    double* const h = d_out + 1;
+    for (int l = 1; l < net.L; ++l)
+        launch_chained(k_margin_layer, (net.dims[l] + T64 / 32 - 1) / (T64 / 32), T64, 0, st, net, d_qs, l, t,
+                       h + (size_t)((l - 1) & 1) * net.hmax, h + (size_t)(l & 1) * net.hmax);
+    launch_chained(k_margin_out, 1, 1024, 0, st, net, d_qs, t, h + (size_t)((net.L - 1) & 1) * net.hmax, d_out);
 }
 
 void launch_fp64(const NetView& net, const QueryView* d_qs, int nq, const QEntry* gather,

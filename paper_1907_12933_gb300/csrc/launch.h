@@ -48,9 +48,6 @@ void launch_fold(const NetView& net, const QueryView* d_qs, int nq, unsigned lon
                  unsigned long long* claim, Queue out, int out_level, int n_sm, cudaStream_t st);
 void launch_fold64(const NetView& net, const QueryView* d_qs, const QEntry* in, const unsigned long long* count,
                    unsigned long long cap, Queue out, int out_level, int n_sm, cudaStream_t st);
-// FP64 margin of point t of query 0 into *d_out where it folded (nothing otherwise).
-void launch_fold_margin(const NetView& net, const QueryView* d_qs, unsigned long long t, double* d_out,
-                        cudaStream_t st);
 
 // Shape class of the FP32 SIMT screen for a net (0: unsupported).
 int simt_variant(const NetView& net);
@@ -93,7 +90,8 @@ void launch_fp64(const NetView& net, const QueryView* d_qs, int nq, const QEntry
                  unsigned long long range_lo, unsigned long long range_hi, int n_sm,
                  cudaStream_t st);
 
-// FP64 margin of point t of query 0 into *d_out.
+// FP64 margin of point t of query 0 into *d_out; d_out[1 ..] holds the outputs of two layers
+// (2 hmax numbers) meanwhile.
 void launch_margin64(const NetView& net, const QueryView* d_qs, unsigned long long t, double* d_out,
                      cudaStream_t st);
 
