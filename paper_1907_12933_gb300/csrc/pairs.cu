@@ -165,7 +165,7 @@ __device__ void pair_covers(const NetView& net, const PairScratch& P, double g, 
 
 __global__ void __launch_bounds__(TP) k_pairs(NetView net, const uint8_t* x1s, const uint8_t* x2s, int n_pairs,
                                                double g, double d, PairOut o) {
-    extern __shared__ double sh[];
+    extern __shared__ __align__(16) double sh[];
     const PairScratch P = pair_scratch(net, sh);
     const int H0 = net.dims[0];
     for (int p = blockIdx.x; p < n_pairs; p += gridDim.x) {
@@ -297,8 +297,9 @@ __global__ void __launch_bounds__(TPD, 2) k_pairs_df(NetView net, const uint8_t*
                                                   const uint8_t* __restrict__ x2s, int n_pairs, double g, double d,
                                                   PairOut o, int bufw) {
     constexpr int PB = IB / 2;
-    extern __shared__ double sh[];
+    extern __shared__ __align__(16) double sh[];
     __shared__ PairDf<IB> T;
+    // (16-byte reads in anchored_dot: rows of 2 IB floats, from a start that is aligned for them)
     float* const buf0 = reinterpret_cast<float*>(sh);   // [bufw][2][IB]: high parts, low parts
     float* const buf1 = buf0 + (size_t)bufw * 2 * IB;   // the same; layer 1's grey levels first
     unsigned char* const fl = reinterpret_cast<unsigned char*>(buf1 + (size_t)bufw * 2 * IB);  // [total][PB]
@@ -531,7 +532,7 @@ __global__ void __launch_bounds__(TPD, 2) k_pairs_df(NetView net, const uint8_t*
 // layers 2..L in full.
 __global__ void __launch_bounds__(TP) k_enum_pairs(NetView net, QueryView Q, double g, double d, PairOut o,
                                                     unsigned long long* n_points) {
-    extern __shared__ double sh[];
+    extern __shared__ __align__(16) double sh[];
     const PairScratch P = pair_scratch(net, sh);
     __shared__ int dv[kMaxS];
     __shared__ int pass;
