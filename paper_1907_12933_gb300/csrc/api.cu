@@ -252,6 +252,7 @@ extern "C" vbmc_status vbmc_net_create(const vbmc_mlp_desc* desc, vbmc_net** out
                 r2 += w * w;
                 WT[(size_t)j * N + i] = W[(size_t)i * K + j];
             }
+            if (r2 == 0.0 && std::fabs((double)b[i]) < kTau) v.dead = 1;
             rn[i] = round_up_f(std::sqrt(r2) * (1.0 + 1e-12));
             frob2 += r2;
         }

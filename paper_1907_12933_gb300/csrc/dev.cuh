@@ -52,6 +52,7 @@ struct NetView {
     float lamsig[kMaxL + 1];          // lambda * sigma_max(W_l) (rounded up)
     float sig[kMaxL + 1];             // sigma_max(W_l) (rounded up)
     float frob[kMaxL + 1];            // ||W_l||_F (rounded up)
+    int dead;                         // 1: some neuron has neither weights nor a bias
     const float* pairw;               // [H_L][H_L]: ||W_L,D - W_L,o||_2 (rounded up)
     // launch shapes (0: the built-in choice; set by vbmc_autotune)
     int simt_var_range, simt_var_gather;    // FP32 pass variant, 1..6

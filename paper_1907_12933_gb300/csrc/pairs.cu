@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(TP) k_pairs(NetView net, const uint8_t* x1s, c
 // CTA = IB images (IB / 2 pairs), a thread per neuron: one weight load serves IB
 // images, whose activations are shared-memory broadcasts, high parts and low parts of
 // an input side by side so that two images make one f32x2 operand: 4 (layer 1) or 5
-// instructions for two multiply-adds. Bound by FP32 issue. 8,192 pairs on
+// instructions for two multiply-adds. Layers stop where every pair is undecided. Bound by FP32 issue. 8,192 pairs on
 // 784-512-512-10: FP64 55.5 ms, one image an instruction and a sum of its own 3.95 ms,
 // now 3.45 ms (the kernel 2.87; its FMA pipe is 69 % busy, two cycles an f32x2).
 constexpr int TPD = 256;
@@ -482,6 +482,9 @@ __global__ void __launch_bounds__(TPD, 2) k_pairs_df(NetView net, const uint8_t*
                 T.E[tid] = En;
             }
             __syncthreads();
+            bool left = false;  // a pair that is still decided
+            for (int q = 0; q < np; ++q) left = left || !T.undec[q];
+            if (!left) break;
         }
         // ---- covers: no sign is a tie in a decided pair, so every bit is certain
         for (int n = tid; n < net.total; n += TPD) {
@@ -637,7 +640,10 @@ extern "C" vbmc_status vbmc_pair_coverage(const vbmc_net* net, const uint8_t* d_
     const PairOut o{out->flip, out->flip_tie, out->ss, out->ss_tie, out->sv, out->sv_tie,
                     out->ds, out->ds_tie, out->dv, out->dv_tie};
     // FP32 pairs where the activation has a pair form, 8 images per CTA once that still
-    // gives every SM a CTA, else 2 (more CTAs, shorter chains per CTA)
+    // gives every SM a CTA, else 2 (more CTAs, shorter chains per CTA). A dead neuron is a
+    // sign tie in every pair, so none would be decided: FP64 at once, a CTA per pair (700 pairs
+    // on 784-512-512-10 5.2 ms, 8.5 by way of FP32 pairs, whose CTAs hold 4 pairs each; 8,192
+    // on 25-10-5 0.23 and 0.45 ms)
     const int bufw = std::max(v.hmax, (v.dims[0] + 1) / 2);
     auto df_smem = [&](int ib) {
         const size_t need = 2 * sizeof(float2) * (size_t)bufw * ib + (size_t)v.total * (ib / 2);
@@ -647,7 +653,7 @@ extern "C" vbmc_status vbmc_pair_coverage(const vbmc_net* net, const uint8_t* d_
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     const int ib = n_pairs >= 4 * n_sm && df_smem(8) <= 200 * 1024 ? 8 : 2;
-    if (v.act != ACT_SIGMOID && df_smem(ib) <= 200 * 1024) {
+    if (v.act != ACT_SIGMOID && !v.dead && df_smem(ib) <= 200 * 1024) {
         const size_t sm = df_smem(ib);
         const unsigned long long groups = ((unsigned long long)n_pairs + ib / 2 - 1) / (ib / 2);
         const unsigned grid = (unsigned)std::min<unsigned long long>(groups, (unsigned long long)n_sm * 8);
