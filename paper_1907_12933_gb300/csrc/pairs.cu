@@ -205,7 +205,7 @@ struct PairDf {
     float sq[TPD / 32][IB / 2][4];   // per warp: ||h||^2 and ||u||^2 of a pair's two images
     double ds[TPD / 32][IB / 2];
     int nflip[IB / 2][kMaxL + 2], only[IB / 2][kMaxL + 2];
-    int undec[IB / 2];
+    int undec[IB / 2], differ[IB / 2];  // undecided; the two images differ
 };
 
 // K terms of neuron column w0 (stride N) against NP pairs of images, whose inputs start
@@ -312,9 +312,15 @@ __global__ void __launch_bounds__(TPD, 2) k_pairs_df(NetView net, const uint8_t*
     for (int p0 = blockIdx.x * PB; p0 < n_pairs; p0 += gridDim.x * PB) {
         const int np = min(PB, n_pairs - p0);
         float* const in0 = buf1;  // [H0][IB]
+        if (tid < PB) T.differ[tid] = 0;
+        __syncthreads();
         for (int im = 0; im < IB; ++im) {
             const uint8_t* x = (im & 1 ? x2s : x1s) + (size_t)(p0 + (im >> 1)) * H0;
-            for (int k = tid; k < H0; k += TPD) in0[k * IB + im] = (im >> 1) < np ? (float)x[k] : 0.f;
+            for (int k = tid; k < H0; k += TPD) {
+                const float v = (im >> 1) < np ? (float)x[k] : 0.f;
+                in0[k * IB + im] = v;
+                if ((im & 1) && v != in0[k * IB + im - 1]) T.differ[im >> 1] = 1;
+            }
         }
         if (tid < PB) T.undec[tid] = 0;
         for (int e = tid; e < PB * (kMaxL + 2); e += TPD) {
@@ -472,10 +478,12 @@ __global__ void __launch_bounds__(TPD, 2) k_pairs_df(NetView net, const uint8_t*
                 const float other = __shfl_xor_sync((1u << IB) - 1u, En, 1);
                 if (im == 0) {
                     T.dist2[pq][l] = ds;
-                    // a layer without a sign change whose distance lies near d: undecided
-                    if (l < L && T.nflip[pq][l] == 0) {
+                    // a layer without a sign change whose distance lies at an edge of the tie
+                    // band around d: undecided (inside it the distance is a tie for certain; that
+                    // of identical images is 0)
+                    if (l < L && T.nflip[pq][l] == 0 && T.differ[pq]) {
                         const double dist = sqrt(ds), ed = (double)__fadd_ru(En, other) * 1.001 + 1e-12 * dist;
-                        if (fabs(dist - d) <= kTau + ed) T.undec[pq] = 1;
+                        if (!(fabs(fabs(dist - d) - kTau) > ed)) T.undec[pq] = 1;
                     }
                 }
                 T.N[tid] = __fmul_ru(__fsqrt_ru(hs), 1.f + 0x1p-20f);
@@ -486,7 +494,7 @@ __global__ void __launch_bounds__(TPD, 2) k_pairs_df(NetView net, const uint8_t*
             for (int q = 0; q < np; ++q) left = left || !T.undec[q];
             if (!left) break;
         }
-        // ---- covers: no sign is a tie in a decided pair, so every bit is certain
+        // ---- covers: no sign is a tie in a decided pair, only a distance may be one
         for (int n = tid; n < net.total; n += TPD) {
             bool any = false;
             for (int q = 0; q < np; ++q) any = any || (!T.undec[q] && (fl[(size_t)n * PB + q] & 1));
@@ -496,8 +504,11 @@ __global__ void __launch_bounds__(TPD, 2) k_pairs_df(NetView net, const uint8_t*
             if (T.undec[q]) continue;
             for (int l = 1; l < L; ++l) {
                 const int nf = T.nflip[q][l];
-                const bool dc = nf == 0 && sqrt(T.dist2[q][l]) - d > kTau;
-                if (nf != 1 && !dc) continue;
+                if (nf > 1) continue;
+                const double over = nf == 0 ? sqrt(T.dist2[q][l]) - d : 0.0;
+                if (!(over >= -kTau)) continue;
+                uint32_t* const ds = over > kTau ? o.ds : o.ds_tie;
+                uint32_t* const dv = over > kTau ? o.dv : o.dv_tie;
                 const int Hn = net.dims[l + 1], on = net.noff[l + 1];
                 const unsigned long long r0 = (unsigned long long)net.ssoff[l] + (unsigned long long)max(T.only[q][l], 0) * Hn;
                 for (int i = tid; i < Hn; i += TPD) {
@@ -506,8 +517,8 @@ __global__ void __launch_bounds__(TPD, 2) k_pairs_df(NetView net, const uint8_t*
                         if ((x & 1) && o.ss) set_bit_once(o.ss, r0 + i);
                         if ((x & 2) && o.sv) set_bit_once(o.sv, r0 + i);
                     } else {
-                        if ((x & 1) && o.ds) set_bit_once(o.ds, (unsigned long long)(on + i));
-                        if ((x & 2) && o.dv) set_bit_once(o.dv, (unsigned long long)(on + i));
+                        if ((x & 1) && ds) set_bit_once(ds, (unsigned long long)(on + i));
+                        if ((x & 2) && dv) set_bit_once(dv, (unsigned long long)(on + i));
                     }
                 }
             }
