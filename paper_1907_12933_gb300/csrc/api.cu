@@ -16,6 +16,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -168,6 +169,7 @@ struct vbmc_result {
     uint8_t* d_group = nullptr;   // tile groups of vbmc_search_query (kGr*; with folded nets)
     uint8_t* h_group = nullptr;   // pinned
     uint32_t* h_masks = nullptr;  // pinned: the coverage masks on their way out
+    std::mutex masks_mu;          // several threads may read a result
     unsigned long long ntiles = 0;          // first-pass tiles of the last call
     bool one_form = false;                  // the last call launched the folded passes only
     int tile_pts = 0;                       // points per first-pass tile (0: no claim counter)
@@ -1158,6 +1160,7 @@ extern "C" vbmc_status vbmc_get_coverage(vbmc_result* res, uint32_t* flip, size_
     const size_t words = ss_tie ? 2 * (fw + sw) : want_ss ? 2 * fw + sw : flip_tie ? 2 * fw : flip ? fw : 0;
     std::vector<uint32_t> own(res->h_masks ? 0 : words);  // a batch member's: no pinned block each
     uint32_t* const h = res->h_masks ? res->h_masks : own.data();
+    std::lock_guard<std::mutex> lk(res->masks_mu);
     if (words) VB_CUDA(cudaMemcpy(h, res->hq.flip, 4 * words, cudaMemcpyDeviceToHost));
     if (flip) std::memcpy(flip, h, 4 * fw);
     if (flip_tie) std::memcpy(flip_tie, h + fw, 4 * fw);
