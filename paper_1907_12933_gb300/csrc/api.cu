@@ -18,6 +18,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 using namespace vbmc;
@@ -125,6 +126,7 @@ struct BatchArena {
     unsigned long long* d_qcount = nullptr;
     unsigned long long* d_claim = nullptr;  // tile claims of each wave's first pass: the general
                                             // one, the folded nets'; queries not folded
+    uint8_t* d_fold = nullptr;              // the members' folded nets (fold_layout), by slot
     QEntry* d_queue[4] = {nullptr, nullptr, nullptr, nullptr};
     uint64_t queue_cap = 0;
     cudaEvent_t ev[7] = {};  // start, prologue, screen, end, split, FP32, double-float
@@ -358,6 +360,33 @@ constexpr size_t kGrTp = (sizeof(QueryView) * kGroupTiles + 15) & ~size_t(15);
 constexpr size_t kGrCnt = kGrTp + sizeof(unsigned long long) * (kGroupTiles + 2);
 constexpr size_t kGrBytes = kGrCnt + sizeof(Counters) * kGroupTiles;
 
+// The folded net's arrays of a query within caps, in one block at `at` (one by one they made
+// a batch's handles up to a third dearer to create); returns the block's bytes.
+size_t fold_layout(const NetView& v, const vbmc_caps& caps, QueryView* q, uint8_t* at) {
+    const size_t S = (size_t)std::max(1, caps.max_s), RM = 2 * (size_t)caps.max_k + 1, T = (size_t)v.total;
+    size_t bytes = 0;
+    auto P = [&](auto** p, size_t n) {
+        *p = reinterpret_cast<std::remove_reference_t<decltype(**p)>*>(at ? at + bytes : nullptr);
+        bytes += (n * sizeof(**p) + 255) & ~size_t(255);
+    };
+    q->fstride = (int)S + kFoldMax;
+    P(&q->fco, T * (size_t)q->fstride);
+    P(&q->fbd, T);
+    P(&q->fer, T);
+    P(&q->fhe, T);
+    P(&q->fsb, T);
+    P(&q->fx, (size_t)kMaxS);
+    P(&q->fcls, T);
+    P(&q->fst, (size_t)kFoldSt);
+    P(&q->fnode, (size_t)kFoldMax);
+    P(&q->fc32, fold_coeff_entries(v, (int)S));
+    P(&q->fk32, (size_t)1 + kFoldOut);
+    P(&q->forow, (size_t)kFoldOut);
+    P(&q->fe64, (size_t)kFoldMax + kFoldOut);
+    P(&q->fxs, S * RM);
+    return bytes;
+}
+
 size_t mask_bytes(const NetView& v) { return 8 * ((size_t)v.flip_words + (size_t)v.ss_words); }
 
 vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena* arena, int slot,
@@ -437,21 +466,9 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
     const bool tcnet = tc_supported(v, VBMC_PREC_BF16) || tc_supported(v, VBMC_PREC_FP16);
     const bool fused = !arena && tcnet;
     if (fold_supported(v)) {
-        q.fstride = S + kFoldMax;
-        A(&q.fco, T * (size_t)q.fstride);
-        A(&q.fbd, T);
-        A(&q.fer, T);
-        A(&q.fhe, T);
-        A(&q.fsb, T);
-        A(&q.fx, (size_t)kMaxS);
-        A(&q.fcls, T);
-        A(&q.fst, (size_t)kFoldSt);
-        A(&q.fnode, (size_t)kFoldMax);
-        A(&q.fc32, fold_coeff_entries(v, S));
-        A(&q.fk32, (size_t)1 + kFoldOut);
-        A(&q.forow, (size_t)kFoldOut);
-        A(&q.fe64, (size_t)kFoldMax + kFoldOut);
-        A(&q.fxs, (size_t)S * RM);
+        uint8_t* block = arena ? arena->d_fold + (size_t)slot * fold_layout(v, *caps, &q, nullptr) : nullptr;
+        if (!arena) A(&block, fold_layout(v, *caps, &q, nullptr));
+        fold_layout(v, *caps, &q, block);
     }
     if (tcnet) A(&q.kcol, 2 * T);
     if (fused) {
@@ -462,12 +479,20 @@ vbmc_status create_result(const vbmc_net* net, const vbmc_caps* caps, BatchArena
         A(&q.w1c, (size_t)kMaxS * v.dims[1]);
         for (int l = 2; l <= v.L; ++l) A(&q.wtc[l], (size_t)v.dims[l - 1] * v.dims[l]);
     }
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&r->h_cnt, sizeof(Counters) + 2 * sizeof(unsigned long long));
-    r->h_claim = reinterpret_cast<unsigned long long*>(r->h_cnt + 1);
-    if (!arena) {
-        if (e == cudaSuccess) e = cudaMallocHost((void**)&r->h_in, kInImage + (size_t)v.dims[0]);
-        if (e == cudaSuccess) e = cudaMallocHost((void**)&r->h_masks, mask_bytes(v));
-        if (groups && e == cudaSuccess) e = cudaMallocHost((void**)&r->h_group, kGrBytes);
+    // pinned: the counters and claims, then what members of a batch do without
+    auto up = [](size_t n) { return (n + 255) & ~size_t(255); };
+    const size_t at_in = up(sizeof(Counters) + 2 * sizeof(unsigned long long));
+    const size_t at_masks = at_in + up(kInImage + (size_t)v.dims[0]), at_group = at_masks + up(mask_bytes(v));
+    uint8_t* pinned = nullptr;
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&pinned, arena ? at_in : at_group + (groups ? kGrBytes : 0));
+    if (e == cudaSuccess) {
+        r->h_cnt = reinterpret_cast<Counters*>(pinned);
+        r->h_claim = reinterpret_cast<unsigned long long*>(r->h_cnt + 1);
+        if (!arena) {
+            r->h_in = pinned + at_in;
+            r->h_masks = reinterpret_cast<uint32_t*>(pinned + at_masks);
+            if (groups) r->h_group = pinned + at_group;
+        }
     }
     if (e == cudaSuccess) e = cudaEventCreate(&r->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&r->ev1);
@@ -547,6 +572,11 @@ extern "C" vbmc_status vbmc_result_create_batch(const vbmc_net* net, const vbmc_
     A(&ar->d_stage, ar->stage_stride * (size_t)nq);
     A(&ar->d_qcount, 4);
     A(&ar->d_claim, 3);
+    const bool caps_ok = caps->max_s >= 0 && caps->max_s <= kMaxS && caps->max_k >= 0 && caps->max_k <= VBMC_MAX_K;
+    if (caps_ok && fold_supported(net->v)) {  // (create_result reports bad caps)
+        QueryView q{};
+        A(&ar->d_fold, fold_layout(net->v, *caps, &q, nullptr) * (size_t)nq);
+    }
     ar->queue_cap = std::max<uint64_t>(1, caps->queue_cap);
     for (int i = 0; i < 4; ++i) A(&ar->d_queue[i], (size_t)ar->queue_cap);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&ar->h_cnt, sizeof(Counters) * (size_t)nq);
@@ -577,12 +607,7 @@ extern "C" vbmc_status vbmc_result_free(vbmc_result* r) {
     wide_work_free(r->ww);
     tc_query_work_free(r->tw);
     arena_release(r->arena);
-    if (r->h_cnt) cudaFreeHost(r->h_cnt);
-    if (r->h_in) {  // not a member of a batch
-        if (r->h_group) cudaFreeHost(r->h_group);
-        cudaFreeHost(r->h_in);
-        if (r->h_masks) cudaFreeHost(r->h_masks);
-    }
+    if (r->h_cnt) cudaFreeHost(r->h_cnt);  // and all that lies behind it
     if (r->ev0) cudaEventDestroy(r->ev0);
     if (r->ev1) cudaEventDestroy(r->ev1);
     if (r->ev_pro) cudaEventDestroy(r->ev_pro);
