@@ -198,6 +198,30 @@ k_tc(const __grid_constant__ TcParams P, NetView net, const QueryView* __restric
     // range mode: tiles from the claim counter (in order, under the time budget);
     // gather mode: statically strided
     unsigned long long* const ctr = SPLIT ? nullptr : claim_ctr;
+    if (SPLIT) {
+        // A layer l >= 3 wider than 64 reuses the accumulator columns of the layer below, so its
+        // MMAs wait for that layer's drain, and the drain needs its operand slots all at once:
+        // two a chunk of 64 here, for the high and the low part (tc_supported checks the
+        // screen's one). Where the ring has fewer, neither could go on; those queues pass on
+        // to the FP32 pass.
+        bool stuck = false;
+        for (int l = 3; l <= L; ++l) {
+            const int Kc = P.compact ? qs[0].kc[l - 1] : P.ly[l].K;
+            const int Nc = P.compact && l < L ? qs[0].kc[l] : P.ly[l].Npad;
+            stuck = stuck || (Nc > 64 && 2 * (Kc / 64) > NA);
+        }
+        if (stuck) {
+            for (unsigned long long e0 = (unsigned long long)blockIdx.x * TC_THREADS + 32 * warp; e0 < gn;
+                 e0 += (unsigned long long)gridDim.x * TC_THREADS) {
+                const bool want = e0 + lane < gn;
+                const unsigned long long t = want ? gather[e0 + lane].t : 0ull;
+                queue_push_warp(out, want, t, 0u, qs[0].cnt, out_level);  // (one query)
+                const unsigned n = __popc(__ballot_sync(0xffffffffu, want));
+                if (lane == 0) work_done(qs[0].cnt, n);
+            }
+            return;
+        }
+    }
     const unsigned long long deadline =
         (!SPLIT && qs[0].budget_ns) ? qs[0].cnt->t0 + qs[0].budget_ns : 0ull;
 
