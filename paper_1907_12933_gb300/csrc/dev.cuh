@@ -160,7 +160,7 @@ struct QueryView {
                             //   nodes, a value that is not below kFoldBig),
                             //   [2 + l] rows of layer l: its nodes, the output layer's rows
     int* fnode;             // [kFoldMax] node -> neuron (concatenated index)
-    float4* fc32;           // packed FP32 coefficients, see FoldLayout
+    float4* fc32;           // packed FP32 coefficients, see FoldShape (fold.cu)
     float4* fk32;           // [1 + kFoldOut]: (margin bound, sign bound, -, -); per output (-, e, -, -)
     int* forow;             // [kFoldOut] rows behind the margins: output, + 256 with a sign test
     float* fe64;            // [kFoldMax + kFoldOut] error bound of a node's or output's FP64 evaluation

@@ -39,9 +39,10 @@
 // can change sign, so a point costs a few hundred multiply-adds instead of the 268 k of
 // 784-512-512-10 (or 2.1 M of 784-1024-1024-1024-10), in FP32 with a bound of about
 // 1e-7 instead of a 16-bit screen's 1e-4..1e-2, and almost no point is left for a
-// second pass. Whole calls, before and after: 784-512-512-10, s = 6, k = 7 (11.4 M
-// points near the boundary) 28.7 -> 1.5 ms; 784-1024x3-10, s = 4, k = 15 with coverage
-// 191 -> 4.3 ms; 784-300-100-10, s = 5, k = 9 in an L2 ball 27.7 -> 0.52 ms.
+// second pass. Whole calls, before and now: 784-512-512-10, s = 6, k = 7 (11.4 M
+// points near the boundary) 38 -> 0.56 ms; 784-1024x3-10, s = 4, k = 15 with coverage
+// 211 -> 0.64 ms (up to 0.99 where a point needs the FP64 pass); 784-300-100-10, s = 5,
+// k = 9 in an L2 ball 27.5 -> 0.25 ms.
 #include "counts.cuh"
 #include "dev.cuh"
 #include "dfloat.cuh"

@@ -530,10 +530,11 @@ void launch_pro_layer(const NetView& net, QueryView* d_qs, int nq, int l, cudaSt
     // eight warps per neuron for at least 256 inputs (one round of their lanes), until
     // the queries alone put about 16 warps on every SM; where the neurons alone leave
     // most SMs empty (output layers of few queries) 32 of them, eight for few inputs
+    constexpr long long kSms = 152;
     const long long neurons = (long long)nq * net.dims[l];
-    if (net.dims[l - 1] >= 256 && neurons <= 152)
+    if (net.dims[l - 1] >= 256 && neurons <= kSms)
         launch_chained(k_pro_layer<32>, dim3(net.dims[l], nq), 1024, 0, st, net, d_qs, nq, l);
-    else if (neurons <= (net.dims[l - 1] >= 256 ? 2432 : 152))
+    else if (neurons <= (net.dims[l - 1] >= 256 ? 16 * kSms : kSms))
         launch_chained(k_pro_layer<8>, dim3(net.dims[l], nq), 256, 0, st, net, d_qs, nq, l);
     else
         launch_chained(k_pro_layer<1>, dim3((net.dims[l] + 7) / 8, nq), 256, 0, st, net, d_qs, nq, l);
