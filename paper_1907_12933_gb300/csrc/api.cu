@@ -902,12 +902,13 @@ QueryView make_view(const vbmc_result* r, const uint8_t* d_image, const int* d_p
 }
 
 // Points that the folded net takes at a time where a call cannot try them all at once and
-// go back when the queues overflow (0: it does not fold). A part is 3 to 5 launches; below
-// 2^16 points (1 us of k_fold's work) the general passes are left to it, whose overflow is then
-// the call's.
+// go back when the queues overflow (0: it does not fold). A part is 4 launches, about 10 us,
+// which 4,000 points of a general pass take as well (2.5 ns each on 784-512-512-10): with
+// more than 64 parts of fewer than 2^16 points the general passes check the query, and their
+// overflow is the call's.
 uint64_t fold_part_of(const vbmc_result* r, uint64_t points) {
     const uint64_t cap = std::max<uint64_t>(1, r->caps.queue_cap);
-    return points <= cap || cap >= (1ull << 16) ? cap : 0;
+    return cap >= (1ull << 16) || (points - 1) / cap < 64 ? cap : 0;
 }
 
 // Enqueue the full pipeline for one query whose image/pixels are on the device. wait:

@@ -105,7 +105,8 @@ def read(vb, res, s, n, dims, summary):
 
 # points per chunk of the wide-layer path, which drains its queues after each; capacity
 @pytest.mark.parametrize("tie", ["sign", "margin"])
-@pytest.mark.parametrize("s,k,chunk,cap", [(2, 30, 1024, 2048), (3, 20, 4096, 1 << 16), (2, 30, 1024, 1024)])
+@pytest.mark.parametrize("s,k,chunk,cap", [(2, 30, 1024, 2048), (3, 20, 4096, 1 << 16), (2, 30, 1024, 1024),
+                                             (3, 20, 256, 256), (2, 30, 128, 128)])
 @pytest.mark.parametrize("call", ["host", "device"])
 def test_wide_query_with_more_undecided_points_than_the_queue_holds(vb, tie, s, k, chunk, cap, call):
     net = all_undecided(843, tie)
